@@ -261,10 +261,11 @@ int pacer_profile_begin(pacer_ctx *ctx);
 int pacer_profile_end(pacer_ctx *ctx, double *fwd_ms, double *fwd_weight_bytes, int64_t *fwd_launches);
 
 /* Y[r][n] = sum_k X[r][k] * W[n][k]: a stand-alone skinny weight-streaming product
- * (a split-k kernel on mma.sync with plain bf16 activations; the projections inside
+ * (ONE kernel on mma.sync with plain bf16 activations; the projections inside
  * the forwards run on a different, tcgen05 path with split activations).  x: device bf16
- * [rows][K] row-major; w: device bf16 [N][K]; y: device f32 [rows][N];
- * scratch: device, at least pacer_linear_scratch_bytes(rows, N, K) bytes.
+ * [rows][K] row-major; w: device bf16 [N][K], 16-byte aligned; y: device f32 [rows][N];
+ * scratch: device, at least pacer_linear_scratch_bytes(rows, N, K) bytes (part of the
+ * interface; the kernel keeps its partial sums on chip and leaves it untouched).
  * rows <= 32, K a multiple of 32.  Enqueues on `cuda_stream`. */
 size_t pacer_linear_scratch_bytes(int rows, int N, int K);
 int pacer_linear(const void *x, const void *w, float *y, int rows, int N, int K, void *scratch,
@@ -275,24 +276,15 @@ int pacer_linear(const void *x, const void *w, float *y, int rows, int N, int K,
  * Who needs it: a serving process that handed all device memory to its own arena
  * at start-up, or a plug-in host without an allocator of its own, has nothing to
  * offer as `scratch`, and a cudaMalloc inside the decode loop would stall the whole
- * device (it synchronises) or simply fail once the arena owns the memory.  Here the
- * scratch is a fixed array of PACER_LINEAR_STATIC_BYTES bytes inside the library
- * image; every GPU that loads the library holds it until the process exits.
+ * device (it synchronises) or simply fail once the arena owns the memory.
  *   - x, w, y, rows, N, K, cuda_stream: exactly as pacer_linear; inputs and the
  *     output remain caller-owned device memory.
  *   - Shapes whose pacer_linear_scratch_bytes(rows, N, K) exceeds
  *     PACER_LINEAR_STATIC_BYTES are refused with PACER_ENOMEM before any launch.
- *   - No cudaMalloc, cudaFree or allocating library routine is called, ever.
- *   - The first call on each device looks up the device address of the array
- *     (cudaGetSymbolAddress, with that device current) and remembers it; make that
- *     first call before starting any stream capture on the device.
- *   - All calls on one device share the one array, which keeps whatever the last
- *     call left in it.  Nothing in it has to start at zero: the kernels overwrite
- *     every element they later read.  Two calls that overlap on the GPU (different
- *     streams, no ordering between them) race on the array; order them.
- *   - Host threads: the per-device address table is filled without a lock, so the first
- *     calls on a device must not come from two host threads at once; later calls only
- *     read it. */
+ *   - No cudaMalloc, cudaFree or allocating library routine is called, ever, and no
+ *     device memory of the library is used: calls may overlap on the GPU and may be
+ *     captured into a graph (not as the first call of a shape class on a device: it
+ *     sets the kernel's shared-memory attribute). */
 #define PACER_LINEAR_STATIC_BYTES (4u << 20)
 int pacer_linear_static(const void *x, const void *w, float *y, int rows, int N, int K, void *cuda_stream);
 

@@ -7,6 +7,7 @@ fails loudly when the library has not been built; there is no CPU fallback.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
 import os
 from typing import Dict, Optional
@@ -290,22 +291,23 @@ def pacer_linear(x: torch.Tensor, w: torch.Tensor) -> torch.Tensor:
     nbytes = _lib.pacer_linear_scratch_bytes(rows, N, K)
     if nbytes == 0:
         raise PacerError("pacer_linear: unsupported shape")
-    scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=x.device)
+    dev = x.device
+    scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=dev)
     sp = (scratch.data_ptr() + 255) // 256 * 256
-    y = torch.empty(rows, N, dtype=torch.float32, device=x.device)
-    with torch.cuda.device(x.device):
+    y = torch.empty(rows, N, dtype=torch.float32, device=dev)
+    # (switching the current device costs more than the product of a small shape)
+    with contextlib.nullcontext() if dev.index == torch.cuda.current_device() else torch.cuda.device(dev):
         rc = _lib.pacer_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, N, K, sp, nbytes,
-                               torch.cuda.current_stream(x.device).cuda_stream)
+                               torch.cuda.current_stream(dev).cuda_stream)
     if rc != 0:
         raise PacerError(f"pacer_linear: {_lib.pacer_strerror(rc).decode()}: {_lib.pacer_last_error(None).decode()}")
     return y
 
 
 def pacer_linear_static(x: torch.Tensor, w: torch.Tensor, out: torch.Tensor) -> torch.Tensor:
-    """y = x @ w.T written into the caller's `out` (f32 [rows][N]) with the library's built-in scratch: the call
-    itself allocates nothing on the device, for callers whose device memory is all spoken for.  Shapes that need
-    more than PACER_LINEAR_STATIC_BYTES of scratch raise PacerError.  Calls on one device share the scratch, so
-    they must not overlap on the GPU."""
+    """y = x @ w.T written into the caller's `out` (f32 [rows][N]) without scratch: the call itself
+    allocates nothing on the device, for callers whose device memory is all spoken for.  Shapes whose
+    pacer_linear_scratch_bytes exceeds PACER_LINEAR_STATIC_BYTES raise PacerError."""
     assert x.is_cuda and w.is_cuda and out.is_cuda and x.dtype == torch.bfloat16 and w.dtype == torch.bfloat16
     assert x.is_contiguous() and w.is_contiguous() and out.is_contiguous() and out.dtype == torch.float32
     rows, K = x.shape

@@ -1,5 +1,4 @@
-// Shared definitions of the Pacer CUDA library (device state, row geometry,
-// activation layout of the standalone GEMM).  sm_100a only.
+// Shared definitions of the Pacer CUDA library (device state, row geometry).  sm_100a only.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -95,15 +94,6 @@ struct ModelDev {
     const float2 *rope;        // [max_ctx][hd/2] (cos, sin)
     int32_t loaded;
 };
-
-// Offset (in elements) of X[r][k] in the fragment-major layout the standalone GEMM (pacer_linear) reads:
-// [k/32][row tile][lane = (r%8)*4 + (k%32)/8][k%8].  A warp's 128-bit loads of
-// one (32-wide k chunk, row tile) are 512 contiguous bytes, already in the
-// register order of mma.m16n8k16's B operand (with the k permutation the GEMM
-// applies to its A operand too).
-__host__ __device__ __forceinline__ size_t xfrag_index(int r, int k, int nt_total) {
-    return ((((size_t)(k >> 5) * nt_total + (r >> 3)) * 32 + ((r & 7) << 2) + ((k & 31) >> 3)) << 3) + (k & 7);
-}
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

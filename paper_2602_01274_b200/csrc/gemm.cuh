@@ -1,22 +1,16 @@
-// Skinny weight-streaming GEMM: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32.
+// Skinny weight-streaming product: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32, bf16 in, fp32 sums, ONE launch.
 //
-// The path is bound by reading W once from HBM, so the kernel is organised
-// around that stream: every lane reads its share of W with 128-bit loads straight
-// into registers (each weight is used exactly once, so staging it in shared
-// memory would only add traffic), several loads in flight per lane.  The few
-// activation rows sit in shared memory in fragment order.  Tensor cores
-// (mma.m16n8k16, bf16 in, fp32 accumulate) do the contraction with the WEIGHTS
-// as the 16-row operand and the token rows as the 8-wide operand, so 1..4 row
-// tiles cost 2..8 MMAs per KB of weights and the math stays invisible.
+// Bound by reading W once from HBM.  Every lane reads its share of W with 128-bit loads straight into registers
+// (each weight is used exactly once, so staging it in shared memory would only add traffic), 6 to 24 loads in flight
+// per lane, and the activations the same way out of L2, in the order the tensor cores want them.  mma.m16n8k16 with
+// the token rows as the 16-row operand and eight weight rows as the other: a lane (g = lane / 4, t = lane % 4) loads the
+// 8 consecutive k of its row at 32c + 8t and uses them as the k slots {2t, 2t+1, 2t+8, 2t+9} of two MMAs; both operands
+// follow the rule, so the products pair up and the sum over k is the same.
 //
-// k permutation: inside every 32-wide k chunk a lane (g = lane/4, t = lane%4)
-// loads the 8 consecutive weights W[n][32c + 8t .. 8t+7] and uses them as the k
-// slots {2t,2t+1,2t+8,2t+9} of two MMAs.  The activation fragment is loaded with
-// the same rule, so the products pair up correctly and the sum over k is the same.
-//
-// Split-K: the grid is S k-slices x row-tile groups; slice partial sums go to
-// part[slice][row][n] and are added up, in slice order (deterministic), by the
-// kernel that consumes the result.
+// Split: a block owns up to 64 tiles of eight weight rows; its eight warps are NW tile groups x KW shares of k (summed
+// through shared memory).  When the tiles do not fill the 148 SMs evenly, S blocks of a cluster share a tile range and
+// take one k slice each; their sums meet through distributed shared memory, in rank order.  No partial sum goes to
+// global memory.
 #pragma once
 #include "common.cuh"
 
@@ -34,187 +28,226 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-struct GemmArgs {
-    const bf16 *X;       // fragment-major activations
-    int32_t nt_total;    // row tiles in X's layout
-    int32_t nt_off;      // first row tile this launch covers
-    const bf16 *W1;      // rows [0, n_w1)
-    const bf16 *W2;      // rows [n_w1, N) (e.g. gate rows then up rows), or unused
-    int32_t n_w1;
-    int32_t N, K;
-    int32_t KS;          // k-slice length, multiple of 32
-    int32_t S;           // number of k slices
-    int32_t tpw;         // weight-row tiles (16 rows) per warp
-    float *part;         // [S][rpad][N]
-    int32_t rpad;        // rows stride of part (= nt_total * 8)
-    const int32_t *n_rows; // per-sequence active rows of this forward; NULL = always run
-    int32_t n_seq;
+struct LinArgs {
+    const bf16 *x, *w;
+    float *y;
+    int32_t rows, N, K;
+    int32_t S;               // blocks of a cluster: k slices
+    int32_t groups;          // clusters: tile ranges
+    int32_t NW;              // tile groups of a block (8 / NW warps share a group's k)
+    int32_t x_aligned;       // x is 16-byte aligned (a view into a larger tensor need not be)
 };
 
-constexpr int GEMM_THREADS = 256;
-constexpr int GEMM_PF = 6;       // 128-bit weight loads in flight per lane and row half
+constexpr int LIN_THREADS = 256, LIN_SMS = 148;
 
-template <int NT>
-__global__ void __launch_bounds__(GEMM_THREADS) k_gemm_skinny(const GemmArgs a) {
-    extern __shared__ uint4 xs[];                      // [chunks][NT][32] 16-byte fragments
-    if (a.n_rows) {                                    // nothing to do when every sequence idles
-        int any = 0;
-        for (int s = 0; s < a.n_seq; ++s) any |= a.n_rows[s];
-        if (!any) return;
-    }
-    const int slice = blockIdx.x % a.S, grp = blockIdx.x / a.S;
-    const int k0 = slice * a.KS;
-    const int kend = min(a.K, k0 + a.KS);
-    const int nchunks = (kend - k0) >> 5;
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(a.X);
-        const int per_chunk = NT * 32;
-        for (int i = threadIdx.x; i < nchunks * per_chunk; i += GEMM_THREADS) {
-            int c = i / per_chunk, rem = i - c * per_chunk;
-            xs[i] = src[((size_t)((k0 >> 5) + c) * a.nt_total + a.nt_off) * 32 + rem];
-        }
-    }
-    __syncthreads();
+// Loads in flight per lane: D chunks of TT weight tiles; the activations of XD chunks (a chunk of one or two tiles is
+// over before an L2 read returns, so there they run as far ahead as the weights).
+__host__ __device__ constexpr int lin_depth(int TT) { return TT >= 6 ? 3 : TT >= 4 ? 4 : 6; }
+__host__ __device__ constexpr int lin_xdepth(int TT) { return TT >= 4 ? 2 : lin_depth(TT); }
+
+__device__ __forceinline__ uint32_t lin_peer(uint32_t smem_addr, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
+    return r;
+}
+
+template <int RM, int TT>
+__global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
+    constexpr int D = lin_depth(TT), XD = lin_xdepth(TT), R = RM * 16;
+    extern __shared__ __align__(16) float lin_red[];               // [8 warps][R rows][TT * 8 columns]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int MT = (a.N + 15) >> 4;
-    const int mt_first = grp * a.tpw * 8 + warp;       // this warp's tiles: mt_first + 8*i
-    int ntile_w = 0;
-    for (int i = 0; i < a.tpw; ++i) if (mt_first + 8 * i < MT) ntile_w = i + 1;
-    if (ntile_w == 0) return;
-    const int total = ntile_w * nchunks;               // flat (tile, chunk) sequence of this warp
-
-    auto row_ptr = [&](int n) -> const bf16 * {
-        n = min(n, a.N - 1);
-        return (n < a.n_w1 ? a.W1 + (size_t)n * a.K : a.W2 + (size_t)(n - a.n_w1) * a.K) + k0 + 8 * t;
+    const int slice = blockIdx.x % a.S, grp = blockIdx.x / a.S;
+    const int KW = 8 / a.NW, nw = warp / KW, kw = warp % KW;
+    const int MT = (a.N + 7) >> 3;
+    // this block's tiles, as even as they come; this warp's among them
+    const int tb = MT / a.groups, tr = MT % a.groups, t0 = grp * tb + min(grp, tr), T = tb + (grp < tr ? 1 : 0);
+    const int w0 = T * nw / a.NW, w1 = T * (nw + 1) / a.NW;
+    const int nch = a.K >> 5, c_lo = nch * slice / a.S, c_hi = nch * (slice + 1) / a.S;   // 32-column chunks
+    const int mine = max(0, (c_hi - c_lo - kw + KW - 1) / KW);
+    const bf16 *wp[TT];
+#pragma unroll
+    for (int i = 0; i < TT; ++i)                                    // tiles past the end repeat a valid row
+        wp[i] = a.w + (size_t)min((t0 + min(w0 + i, max(w1 - 1, 0))) * 8 + g, a.N - 1) * a.K + (size_t)(c_lo + kw) * 32 + 8 * t;
+    const bf16 *xp = a.x + (size_t)g * a.K + (size_t)(c_lo + kw) * 32 + 8 * t;
+    const size_t step = (size_t)KW * 32;
+    uint4 w[D][TT], xv[XD][RM][2];
+    float acc[TT][RM][4];
+#pragma unroll
+    for (int i = 0; i < TT; ++i)
+#pragma unroll
+        for (int m = 0; m < RM; ++m) acc[i][m][0] = acc[i][m][1] = acc[i][m][2] = acc[i][m][3] = 0.f;
+    auto load_w = [&](int slot, int c) {
+#pragma unroll
+        for (int i = 0; i < TT; ++i) w[slot][i] = ldg_stream(wp[i] + (size_t)c * step);
     };
-
-    uint4 w0[GEMM_PF], w1[GEMM_PF];
-    // loader cursor
-    int l_tile = 0, l_chunk = 0;
-    const bf16 *lp0 = row_ptr(mt_first * 16 + g), *lp1 = row_ptr(mt_first * 16 + g + 8);
-    auto issue = [&](int slot) {
-        w0[slot] = ldg_stream(lp0 + (l_chunk << 5));
-        w1[slot] = ldg_stream(lp1 + (l_chunk << 5));
-        if (++l_chunk == nchunks) {
-            l_chunk = 0;
-            ++l_tile;
-            int mt = mt_first + 8 * l_tile;
-            lp0 = row_ptr(mt * 16 + g);
-            lp1 = row_ptr(mt * 16 + g + 8);
-        }
-    };
+    auto load_x = [&](int slot, int c) {
 #pragma unroll
-    for (int j = 0; j < GEMM_PF; ++j) if (j < total) issue(j);
-
-    float acc[NT][4];
+        for (int m = 0; m < RM; ++m)
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) { acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f; }
-    int c_tile = 0, c_chunk = 0;
-    for (int q0 = 0; q0 < total; q0 += GEMM_PF) {
-#pragma unroll
-        for (int j = 0; j < GEMM_PF; ++j) {
-            const int q = q0 + j;
-            if (q < total) {
-                const uint4 a0 = w0[j], a1 = w1[j];
-                if (q + GEMM_PF < total) issue(j);
-                const uint4 *xb = xs + (size_t)c_chunk * (NT * 32) + lane;
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    const uint4 b = xb[nt * 32];
-                    mma_bf16_16816(acc[nt], a0.x, a1.x, a0.y, a1.y, b.x, b.y);
-                    mma_bf16_16816(acc[nt], a0.z, a1.z, a0.w, a1.w, b.z, b.w);
-                }
-                if (++c_chunk == nchunks) {
-                    // tile finished: accumulator (g, 2t..2t+1) = weight row n0+g x token rows 2t, 2t+1
-                    const int n0 = (mt_first + 8 * c_tile) * 16 + g, n1 = n0 + 8;
-                    float *pbase = a.part + (size_t)slice * a.rpad * a.N;
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        const int r0 = (a.nt_off + nt) * 8 + 2 * t;
-                        if (n0 < a.N) {
-                            pbase[(size_t)r0 * a.N + n0] = acc[nt][0];
-                            pbase[(size_t)(r0 + 1) * a.N + n0] = acc[nt][1];
-                        }
-                        if (n1 < a.N) {
-                            pbase[(size_t)r0 * a.N + n1] = acc[nt][2];
-                            pbase[(size_t)(r0 + 1) * a.N + n1] = acc[nt][3];
-                        }
-                        acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+            for (int h = 0; h < 2; ++h) {
+                const bf16 *p = xp + (size_t)(m * 16 + h * 8) * a.K + (size_t)c * step;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (m * 16 + h * 8 + g < a.rows) {
+                    if (a.x_aligned) v = __ldg(reinterpret_cast<const uint4 *>(p));
+                    else {
+                        const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
+                        v = make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16, q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
                     }
-                    c_chunk = 0;
-                    ++c_tile;
+                }
+                xv[slot][m][h] = v;
+            }
+    };
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        if (j < mine) load_w(j, j);
+        if (j < XD && j < mine) load_x(j, j);
+    }
+    constexpr int U = D % XD == 0 ? D : D * XD;                     // both rings back at slot 0
+    for (int c0 = 0; c0 < mine; c0 += U) {
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const int c = c0 + j;
+            if (c >= mine) break;
+#pragma unroll
+            for (int i = 0; i < TT; ++i) {
+                const uint4 b = w[j % D][i];
+#pragma unroll
+                for (int m = 0; m < RM; ++m) {
+                    const uint4 p = xv[j % XD][m][0], q = xv[j % XD][m][1];
+                    mma_bf16_16816(acc[i][m], p.x, q.x, p.y, q.y, b.x, b.y);
+                    mma_bf16_16816(acc[i][m], p.z, q.z, p.w, q.w, b.z, b.w);
                 }
             }
+            if (c + D < mine) load_w(j % D, c + D);
+            if (c + XD < mine) load_x(j % XD, c + XD);
         }
+    }
+    // accumulator (g, 2t..): token row m*16 + g (+8), weight row 8i + 2t (+1)
+    constexpr int P = TT * 8;
+    float *my = lin_red + (size_t)warp * R * P;
+#pragma unroll
+    for (int i = 0; i < TT; ++i)
+#pragma unroll
+        for (int m = 0; m < RM; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<float2 *>(my + (m * 16 + h * 8 + g) * P + i * 8 + 2 * t) = make_float2(acc[i][m][2 * h], acc[i][m][2 * h + 1]);
+    __syncthreads();
+    const int cols = T * 8, n_out = a.rows * cols;
+    // column -> (tile group, column within the group); the KW shares summed in warp order
+    auto local_sum = [&](int r, int col) -> float * {
+        const int ti = col >> 3;
+        int q = 0;
+        while (q + 1 < a.NW && T * (q + 1) / a.NW <= ti) ++q;
+        return lin_red + ((size_t)(q * KW) * R + r) * P + (col - (T * q / a.NW) * 8);
+    };
+    for (int i = threadIdx.x; i < n_out; i += LIN_THREADS) {
+        const int r = i / cols, col = i - r * cols, n = t0 * 8 + col;
+        float *p = local_sum(r, col);
+        float v = p[0];
+        for (int k = 1; k < KW; ++k) v += p[(size_t)k * R * P];
+        if (a.S > 1) p[0] = v;                                      // the block's sum, for the cluster
+        else if (n < a.N) a.y[(size_t)r * a.N + n] = v;
+    }
+    if (a.S > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        for (int i = threadIdx.x + slice * LIN_THREADS; i < n_out; i += a.S * LIN_THREADS) {
+            const int r = i / cols, col = i - r * cols, n = t0 * 8 + col;
+            const uint32_t at = (uint32_t)__cvta_generic_to_shared(local_sum(r, col));
+            float v = 0.f;
+            for (int s = 0; s < a.S; ++s) {
+                float u;
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(u) : "r"(lin_peer(at, s)) : "memory");
+                v += u;
+            }
+            if (n < a.N) a.y[(size_t)r * a.N + n] = v;
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }
 
-// Launch plan for one product.
-struct GemmPlan {
-    int S, KS, tpw, grid;
-    size_t smem;
+struct LinPlan {
+    int S, groups, NW, TT;
 };
 
-static inline GemmPlan gemm_plan(int N, int K, int NT) {
-    GemmPlan p;
-    const int MT = (N + 15) / 16;
-    int ks_target = MT >= 1024 ? 2048 : 1024;
-    // shared memory: NT * 8 rows * KS * 2 bytes, keep two blocks per SM possible
-    while ((size_t)NT * 8 * ks_target * 2 > 96 * 1024) ks_target /= 2;
-    p.S = (K + ks_target - 1) / ks_target;
-    p.KS = (((K + p.S - 1) / p.S) + 31) / 32 * 32;
-    p.S = (K + p.KS - 1) / p.KS;
-    long tasks = (long)MT * p.S;
-    long tpw = tasks / (8L * 2 * 148);
-    if (tpw < 1) tpw = 1;
-    if (tpw > 8) tpw = 8;
-    p.tpw = (int)tpw;
-    int groups = (MT + 8 * p.tpw - 1) / (8 * p.tpw);
-    p.grid = groups * p.S;
-    p.smem = (size_t)NT * 8 * p.KS * 2;
-    return p;
+// The split with the least weight bytes per block: S = 1 or 2 slices over all SMs (every pair of SMs can hold a
+// cluster of two); 4 or 8 only while few clusters are needed (an odd number of SMs per GPC strands some otherwise).  A
+// block keeps at least eight chunks of k, and the smaller S wins ties: 17 x 4096 x 11008 runs as 74 clusters of two,
+// 7 tiles each (full 98.9 %), where one slice would leave 4 tiles on some SMs against a mean of 3.46.
+static inline LinPlan lin_plan(int N, int K) {
+    const int MT = (N + 7) / 8, nch = K / 32;
+    LinPlan best{};
+    double best_cost = 1e30;
+    const int cap[4] = {LIN_SMS, LIN_SMS / 2, 32, 16};
+    for (int i = 0; i < 4; ++i) {
+        const int S = 1 << i;
+        if (S > 1 && nch / S < 8) break;
+        const int waves = (MT + cap[i] * 64 - 1) / (cap[i] * 64);   // at most 64 tiles per block
+        if (S > 1 && waves > 1) break;
+        const int groups = MT < cap[i] * waves ? MT : cap[i] * waves, tiles = (MT + groups - 1) / groups;
+        const double cost = (double)waves * tiles / S;
+        if (cost < best_cost * 0.97) {
+            best_cost = cost;
+            best.S = S; best.groups = groups;
+            best.NW = 1;
+            while ((tiles + best.NW - 1) / best.NW > 8) best.NW *= 2;
+            best.TT = (tiles + best.NW - 1) / best.NW;
+        }
+    }
+    return best;
 }
 
-template <int NT>
-static cudaError_t gemm_launch_nt(const GemmArgs &a, const GemmPlan &p, cudaStream_t st) {
+template <int RM, int TT>
+static cudaError_t lin_launch(const LinArgs &a, cudaStream_t st) {
+    constexpr size_t smem = (size_t)8 * RM * 16 * TT * 8 * sizeof(float);
     static bool attr_set[64] = {};           // the opt-in is per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(k_gemm_skinny<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || !attr_set[dev])) {
+        e = cudaFuncSetAttribute(k_linear<RM, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    k_gemm_skinny<NT><<<p.grid, GEMM_THREADS, p.smem, st>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.groups * a.S); cfg.blockDim = dim3(LIN_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = a.S; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = a.S > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_linear<RM, TT>, a);
 }
 
-// Y partials for all `nt_total` row tiles: passes of up to 4 tiles each.
-// Returns the number of kernels launched through *launches.
-static cudaError_t gemm_run(const bf16 *X, int nt_total, const bf16 *W1, const bf16 *W2, int n_w1, int N, int K,
-                            float *part, const int32_t *n_rows, int n_seq, cudaStream_t st, GemmPlan *plan_out,
-                            int64_t *launches) {
-    const int NT = nt_total < 4 ? nt_total : 4;
-    GemmPlan p = gemm_plan(N, K, NT);
-    if (plan_out) *plan_out = p;
-    for (int off = 0; off < nt_total; off += 4) {
-        int nt = nt_total - off < 4 ? nt_total - off : 4;
-        GemmArgs a;
-        a.X = X; a.nt_total = nt_total; a.nt_off = off; a.W1 = W1; a.W2 = W2 ? W2 : W1; a.n_w1 = W2 ? n_w1 : N;
-        a.N = N; a.K = K; a.KS = p.KS; a.S = p.S; a.tpw = p.tpw; a.part = part; a.rpad = nt_total * 8;
-        a.n_rows = n_rows; a.n_seq = n_seq;
-        GemmPlan pp = p;
-        pp.smem = (size_t)nt * 8 * p.KS * 2;
-        cudaError_t e;
-        switch (nt) {
-            case 1: e = gemm_launch_nt<1>(a, pp, st); break;
-            case 2: e = gemm_launch_nt<2>(a, pp, st); break;
-            case 3: e = gemm_launch_nt<3>(a, pp, st); break;
-            default: e = gemm_launch_nt<4>(a, pp, st); break;
-        }
-        if (e != cudaSuccess) return e;
-        if (launches) ++*launches;
+template <int RM>
+static cudaError_t lin_dispatch(int TT, const LinArgs &a, cudaStream_t st) {
+    switch (TT) {
+        case 1: return lin_launch<RM, 1>(a, st);
+        case 2: return lin_launch<RM, 2>(a, st);
+        case 3: return lin_launch<RM, 3>(a, st);
+        case 4: return lin_launch<RM, 4>(a, st);
+        case 5: return lin_launch<RM, 5>(a, st);
+        case 6: return lin_launch<RM, 6>(a, st);
+        case 7: return lin_launch<RM, 7>(a, st);
+        default: return lin_launch<RM, 8>(a, st);
     }
-    return cudaSuccess;
+}
+
+static inline cudaError_t lin_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
+    const LinPlan p = lin_plan(N, K);
+    LinArgs a;
+    a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.S = p.S; a.groups = p.groups; a.NW = p.NW;
+    a.x_aligned = ((uintptr_t)x & 15) == 0;
+    return rows <= 16 ? lin_dispatch<1>(p.TT, a, st) : lin_dispatch<2>(p.TT, a, st);
+}
+
+// Scratch bytes the interface asks callers for (the limit of the allocation-free entry point is stated in them):
+// fragment-ordered activations and the partial sums of k slices of at most 1024 or 2048 columns.
+static inline size_t lin_scratch_bytes(int rows, int N, int K) {
+    const int nt = (rows + 7) / 8, MT = (N + 15) / 16;
+    int ks = MT >= 1024 ? 2048 : 1024;
+    while ((size_t)nt * 8 * ks * 2 > 96 * 1024) ks /= 2;
+    int S = (K + ks - 1) / ks;
+    const int KS = (((K + S - 1) / S) + 31) / 32 * 32;
+    S = (K + KS - 1) / KS;
+    return ((size_t)nt * 8 * K * sizeof(bf16) + 255) / 256 * 256 + (size_t)S * nt * 8 * N * sizeof(float);
 }

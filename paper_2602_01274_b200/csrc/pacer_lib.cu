@@ -849,26 +849,9 @@ extern "C" int pacer_generate_ar(pacer_ctx *c, const int32_t *prompt, int batch,
 
 // ------------------------------------------------------------------ stand-alone product
 
-__global__ void k_to_frag(const bf16 *x, bf16 *xf, int rows, int K, int nt) {
-    const int r = blockIdx.y, k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    xf[xfrag_index(r, k, nt)] = r < rows ? x[(size_t)r * K + k] : __float2bfloat16(0.f);
-}
-
-__global__ void k_sum_part(const float *part, float *y, int rows, int N, int S, int rpad) {
-    const int r = blockIdx.y, n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N || r >= rows) return;
-    float v = 0.f;
-    for (int s = 0; s < S; ++s) v += part[((size_t)s * rpad + r) * N + n];
-    y[(size_t)r * N + n] = v;
-}
-
 extern "C" size_t pacer_linear_scratch_bytes(int rows, int N, int K) {
     if (rows < 1 || rows > 32 || N < 1 || K < 32 || K % 32) return 0;
-    const int nt = (rows + 7) / 8;
-    GemmPlan p = gemm_plan(N, K, nt);
-    size_t xf = ((size_t)nt * 8 * K * sizeof(bf16) + 255) / 256 * 256;
-    return xf + (size_t)p.S * nt * 8 * N * sizeof(float);
+    return lin_scratch_bytes(rows, N, K);
 }
 
 extern "C" int pacer_linear(const void *x, const void *w, float *y, int rows, int N, int K, void *scratch,
@@ -878,25 +861,11 @@ extern "C" int pacer_linear(const void *x, const void *w, float *y, int rows, in
     if (!x || !w || !y || !scratch || need == 0) return fail(nullptr, PACER_EINVAL, "pacer_linear: bad argument");
     if (scratch_bytes < need) return fail(nullptr, PACER_ENOMEM, "pacer_linear: scratch too small");
     if (((uintptr_t)w & 15) || ((uintptr_t)scratch & 255)) return fail(nullptr, PACER_EINVAL, "pacer_linear: misaligned pointer");
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int nt = (rows + 7) / 8;
-    bf16 *xf = (bf16 *)scratch;
-    float *part = (float *)((char *)scratch + ((size_t)nt * 8 * K * sizeof(bf16) + 255) / 256 * 256);
-    k_to_frag<<<dim3((K + 255) / 256, nt * 8), 256, 0, st>>>((const bf16 *)x, xf, rows, K, nt);
-    CK(cudaGetLastError());
-    GemmPlan p;
-    CK(gemm_run(xf, nt, (const bf16 *)w, nullptr, 0, N, K, part, nullptr, 0, st, &p, nullptr));
-    k_sum_part<<<dim3((N + 255) / 256, rows), 256, 0, st>>>(part, y, rows, N, p.S, nt * 8);
-    CK(cudaGetLastError());
+    CK(lin_run((const bf16 *)x, (const bf16 *)w, y, rows, N, K, (cudaStream_t)cuda_stream));
     return PACER_OK;
 }
 
 // ------------------------------------------------------------------ product without caller scratch
-
-// Scratch of pacer_linear_static.  In host code this name is only a handle for
-// cudaGetSymbolAddress; the device address is looked up once per device.
-static __device__ __align__(256) unsigned char g_linear_static_scratch[PACER_LINEAR_STATIC_BYTES];
-static void *g_linear_static_ptr[64];
 
 extern "C" int pacer_linear_static(const void *x, const void *w, float *y, int rows, int N, int K, void *cuda_stream) {
     pacer_ctx *c = nullptr;
@@ -904,14 +873,7 @@ extern "C" int pacer_linear_static(const void *x, const void *w, float *y, int r
     if (!x || !w || !y || need == 0) return fail(nullptr, PACER_EINVAL, "pacer_linear_static: bad argument");
     if (need > (size_t)PACER_LINEAR_STATIC_BYTES)
         return fail(nullptr, PACER_ENOMEM, "pacer_linear_static: shape needs more than PACER_LINEAR_STATIC_BYTES of scratch");
-    int dev = -1;
-    CK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(nullptr, PACER_EUNSUPPORTED, "pacer_linear_static: device index out of range");
-    if (!g_linear_static_ptr[dev]) {
-        void *p = nullptr;
-        CK(cudaGetSymbolAddress(&p, g_linear_static_scratch));
-        if (!p) return fail(nullptr, PACER_ECUDA, "pacer_linear_static: no device address for the scratch array");
-        g_linear_static_ptr[dev] = p;
-    }
-    return pacer_linear(x, w, y, rows, N, K, g_linear_static_ptr[dev], (size_t)PACER_LINEAR_STATIC_BYTES, cuda_stream);
+    if ((uintptr_t)w & 15) return fail(nullptr, PACER_EINVAL, "pacer_linear_static: misaligned pointer");
+    CK(lin_run((const bf16 *)x, (const bf16 *)w, y, rows, N, K, (cudaStream_t)cuda_stream));
+    return PACER_OK;
 }
