@@ -128,7 +128,7 @@ def kernel_source_digest() -> str:
     h = hashlib.sha1()
     d = os.path.join(ROOT, "paper_2602_01274_b200", "csrc")
     for f in sorted(os.listdir(d)):
-        if f.endswith((".cu", ".cuh")):
+        if f.endswith((".cu", ".cuh", ".h")):
             h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()[:16]
 

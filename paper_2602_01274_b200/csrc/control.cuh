@@ -92,7 +92,7 @@ __device__ __forceinline__ void accept_greedy_seq(const DevPtrs &d, const Geom &
 
 // The same as a kernel of its own, for the stage-by-stage interface (the whole-loop entry points take the
 // decision in the tail of the verify forward).
-__global__ void k_accept_greedy(DevPtrs d, Geom g) {
+static __global__ void k_accept_greedy(DevPtrs d, Geom g) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < g.batch) accept_greedy_seq(d, g, s);
 }

@@ -97,13 +97,15 @@ struct Plan {
 
 // Device buffers of the forward kernel beyond DevPtrs (all in the workspace).
 struct FwdBufs {
-    float *qkv;              // [k slices][MAX_ROWS][qrows] fp32
+    float *qkv;              // [k slices][MAX_ROWS][qrows] fp32 (the rows of a q or k head as rotary pairs, see k_retile);
+                             // in the few-row kernel q alone, [row][H * hd], rotated and scaled
     bf16 *xg;                // x * gain of the next RMSNorm, split bf16 in operand order (its 1/rms comes later)
     float *ssq;              // [d/16][MAX_ROWS] sum of squares of x over the 16 columns of a tile
     float *part;             // k-slice partial tiles [S][d/16][row tiles * 8][16] of the two residual projections
     float *tile_top;         // [MT(head)][MAX_ROWS][4]: max, argmax (int bits), runner-up, unused
     float *attp;             // attention partials [seq*H + h][split][row][hd + 2]
-    int32_t *att_cnt;        // [batch * H]
+    float *attf;             // attention partials of the few-row kernel: [item][query row][hd + 2]
+    int32_t *att_cnt;        // arrivals of the key splits of an attention unit (few-row kernel)
     unsigned long long *bar; // grid barrier counter
     int32_t *abort_flag;     // [0] code of the first bounded wait that ran out, [1..3] its block, warp, detail
     unsigned long long *prof; // optional: every block stamps %globaltimer at its phase boundaries (NULL = off)

@@ -88,22 +88,32 @@ __device__ __forceinline__ void attention_rows(Ctx &c, const Args &a, int layer,
             if (GQA) { const int v = vbase + lv, hq = v / n_r; jq = v - hq * n_r; h = kh * group + hq; }
             const float *rowk = a.fb.qkv + (size_t)(r_base + (onk ? lv : 0)) * qrows;
             const float *rowq = GQA ? a.fb.qkv + (size_t)(r_base + (onq ? jq : 0)) * qrows : rowk;
-            const int col[6] = {h * HD + ii, h * HD + ii + half, (H + kh) * HD + ii, (H + kh) * HD + ii + half,
-                                (H + Hkv + kh) * HD + ii, (H + Hkv + kh) * HD + ii + half};
+            // channels ii and ii + half of q and k lie side by side (rotary pairs); of v they do not
+            const float *pq = rowq + h * HD + 2 * ii, *pk = rowk + (H + kh) * HD + 2 * ii, *pv = rowk + (H + Hkv + kh) * HD + ii;
             csq[u] = onq ? m.rope[(size_t)(pos0 + jq) * half + ii] : make_float2(0.f, 0.f);
             csk[u] = !GQA ? csq[u] : (onk ? m.rope[(size_t)(pos0 + lv) * half + ii] : make_float2(0.f, 0.f));
 #pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int e = 0; e < 6; ++e)
-                    part[u][s][e] = ((e < 2 ? onq : onk) && s < S) ? __ldcg((e < 2 ? rowq : rowk) + s * sl + col[e]) : 0.f;
+            for (int s = 0; s < 2; ++s) {
+                const float2 z = make_float2(0.f, 0.f);
+                const float2 q2 = onq && s < S ? __ldcg(reinterpret_cast<const float2 *>(pq + s * sl)) : z;
+                const float2 k2 = onk && s < S ? __ldcg(reinterpret_cast<const float2 *>(pk + s * sl)) : z;
+                part[u][s][0] = q2.x; part[u][s][1] = q2.y; part[u][s][2] = k2.x; part[u][s][3] = k2.y;
+                part[u][s][4] = onk && s < S ? __ldcg(pv + s * sl) : 0.f;
+                part[u][s][5] = onk && s < S ? __ldcg(pv + s * sl + half) : 0.f;
+            }
             if (S > 2) {                                         // slices 2, 3: a second wave of loads
 #pragma unroll
-                for (int e = 0; e < 6; ++e) {
-                    if (!(e < 2 ? onq : onk)) continue;
-                    const float *row = e < 2 ? rowq : rowk;
-                    const float p2 = __ldcg(row + 2 * sl + col[e]), p3 = S > 3 ? __ldcg(row + 3 * sl + col[e]) : 0.f;
-                    part[u][0][e] += p2; part[u][1][e] += p3;
+                for (int s = 2; s < 4; ++s) {
+                    if (s >= S) continue;
+                    if (onq) {
+                        const float2 q2 = __ldcg(reinterpret_cast<const float2 *>(pq + s * sl));
+                        part[u][s - 2][0] += q2.x; part[u][s - 2][1] += q2.y;
+                    }
+                    if (onk) {
+                        const float2 k2 = __ldcg(reinterpret_cast<const float2 *>(pk + s * sl));
+                        part[u][s - 2][2] += k2.x; part[u][s - 2][3] += k2.y;
+                        part[u][s - 2][4] += __ldcg(pv + s * sl); part[u][s - 2][5] += __ldcg(pv + s * sl + half);
+                    }
                 }
             }
         }
@@ -162,7 +172,7 @@ __device__ __forceinline__ void attention_append(Ctx &c, const Args &a, int laye
     for (int i = threadIdx.x; i < n_el; i += MMA_THREADS) {
         const int j = jbase + i / half, ii = i % half, pos = pos0 + j;
         const float *row = a.fb.qkv + (size_t)(r_base + j) * qrows;
-        const int col[4] = {(H + kh) * HD + ii, (H + kh) * HD + ii + half, (H + Hkv + kh) * HD + ii, (H + Hkv + kh) * HD + ii + half};
+        const int col[4] = {(H + kh) * HD + 2 * ii, (H + kh) * HD + 2 * ii + 1, (H + Hkv + kh) * HD + ii, (H + Hkv + kh) * HD + ii + half};
         float in[4] = {0.f, 0.f, 0.f, 0.f};
         for (int s_ = 0; s_ < S; ++s_)
 #pragma unroll

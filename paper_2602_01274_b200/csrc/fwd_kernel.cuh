@@ -1,142 +1,12 @@
-// The forward kernel itself, the tails that take the loop's decisions (Eq. 6 /
-// Eq. 7 / Algorithm 1) on the device, the host-side plan and the cooperative launch.
+// The forward kernel itself, the host-side plan and the cooperative launch.
 #pragma once
 #include <algorithm>
 #include <vector>
 
 #include "fwd_attention.cuh"
-#include "sampling.cuh"
+#include "fwd_tails.cuh"
 
 namespace fwd {
-
-// ------------------------------------------------------------------ tails (one block per sequence)
-
-__device__ __forceinline__ float hidden_at(const Args &a, const Ctx &c, int r, int i) {
-    return __ldcg(a.d.xres + (size_t)r * a.m.cfg.d_model + i) * c.inv_rms[r] * __bfloat162float(a.m.normf[i]);
-}
-
-// 1/rms of the final residual rows of sequence s, for the final RMSNorm the tails apply (MMA warps of one block).
-__device__ __forceinline__ void tail_inv_rms(Ctx &c, const Args &a, int s) {
-    const int dm = a.m.cfg.d_model;
-    float *red = reinterpret_cast<float *>(c.scratch);
-    for (int j = 0; j < c.n_rows[s]; ++j) {
-        const int r = s * a.g.rps + j;
-        float ss = 0.f;
-        for (int i = threadIdx.x; i < dm; i += MMA_THREADS) { const float v = __ldcg(a.d.xres + (size_t)r * dm + i); ss += v * v; }
-        ss = mma_block_sum(ss, red);
-        if (threadIdx.x == 0) c.inv_rms[r] = rsqrtf(ss / (float)dm + a.m.cfg.rms_eps);
-    }
-    bsync();
-}
-
-// End of one draft forward (Eq. 6): y_i, h_i queued for the pre-verification model, cache length.
-__device__ __forceinline__ void tail_draft(Ctx &c, const Args &a, int s) {
-    const DevPtrs &d = a.d;
-    SeqState &st = d.st[s];
-    const int n_in = c.n_rows[s], dm = a.m.cfg.d_model;
-    if (n_in == 0) return;
-    const int gamma = st.gamma, n_pend = st.n_pend, r_last = s * a.g.rps + n_in - 1;
-    int y_new = 0;
-    if (st.mode == PACER_SAMPLE)                          // y_i ~ q_i by the Gumbel-max rule at the token's position
-        y_new = gumbel_argmax(d.draft_logits + ((size_t)s * d.gamma_cap + gamma) * a.m.cfg.vocab, a.m.cfg.vocab, st.seed,
-                              st.P + gamma, s, TAG_DRAFT, MMA_THREADS, reinterpret_cast<BestD *>(c.scratch), true);
-    const bool queue = !st.sched;                        // with prescribed windows nothing is pre-verified
-    for (int jj = 0; queue && jj < n_in; ++jj) {
-        float *dst = d.hpend + ((size_t)s * (d.block_b + 1) + n_pend + jj) * dm;
-        for (int i = threadIdx.x; i < dm; i += MMA_THREADS) dst[i] = hidden_at(a, c, s * a.g.rps + jj, i);
-    }
-    bsync();
-    if (threadIdx.x == 0) {
-        for (int jj = 0; queue && jj < n_in; ++jj)
-            d.hpend_e[s * (d.block_b + 1) + n_pend + jj] = (jj == n_in - 1) ? gamma + 1 : 0;
-        d.y[(size_t)s * d.gamma_cap + gamma] = st.mode == PACER_SAMPLE ? y_new : d.row_arg[r_last];
-        if (queue) st.n_pend = n_pend + n_in;
-        st.gamma = gamma + 1;
-        st.len_D += n_in;
-        st.n_draft_fwd += 1;
-    }
-}
-
-// End of a pre-verification call (Eq. 7 + the block test of Algorithm 1).
-__device__ __forceinline__ void tail_mb(Ctx &c, const Args &a, int s) {
-    const DevPtrs &d = a.d;
-    SeqState &st = d.st[s];
-    const int n = c.n_rows[s], dm = a.m.cfg.d_model;
-    if (n == 0) return;
-    float *red = reinterpret_cast<float *>(c.scratch);
-    for (int j = 0; j < n; ++j) {
-        const int r = s * a.g.rps + j, e = c.row_tok[r];
-        if (e == 0) continue;
-        float z0 = 0.f, z1 = 0.f;
-        for (int i = threadIdx.x; i < dm; i += MMA_THREADS) {
-            const float hv = hidden_at(a, c, r, i);
-            z0 += hv * __bfloat162float(a.m.head_b[i]);
-            z1 += hv * __bfloat162float(a.m.head_b[dm + i]);
-        }
-        z0 = mma_block_sum(z0, red);
-        z1 = mma_block_sum(z1, red);
-        if (threadIdx.x == 0) d.alpha[(size_t)s * d.gamma_cap + e - 1] = 1.f / (1.f + expf(z0 - z1));
-    }
-    bsync();
-    if (threadIdx.x == 0) {
-        const int b = d.block_b, gamma = st.gamma;
-        const float *ab = d.alpha + (size_t)s * d.gamma_cap + (gamma - b);
-        float stat;
-        if (d.criterion == 1) { stat = ab[0]; for (int i = 1; i < b; ++i) stat = fminf(stat, ab[i]); }
-        else if (d.criterion == 2) stat = ab[b - 1];
-        else { stat = 0.f; for (int i = 0; i < b; ++i) stat += ab[i]; stat /= (float)b; }
-        int stop = 0;
-        if (st.t0 >= 0.f && stat <= st.t_k) stop = 1;
-        if (gamma + b > st.gamma_max) stop = 1;
-        if (stop) st.drafting = 0;
-        else { st.t_k = st.t_k * d.rho; st.k_round += 1; }
-        if (gamma == b) {                     // first call of the step: where its drafts begin in the cache
-            int n_hist = 0;
-            while (n_hist < n && c.row_tok[s * a.g.rps + n_hist] == 0) ++n_hist;
-            st.mb_start = st.len_B + n_hist;
-        }
-        st.len_B += n;
-        st.n_pend = 0;
-        st.n_mb_calls += 1;
-    }
-}
-
-// End of a prefill chunk: the caches grew; the draft's hidden rows are the
-// history rows the pre-verification model is prefilled with.
-__device__ __forceinline__ void tail_prefill(Ctx &c, const Args &a, int s, int which) {
-    const DevPtrs &d = a.d;
-    const int n = c.n_rows[s], dm = a.m.cfg.d_model;
-    if (n == 0) return;
-    if (which == PACER_DRAFT)
-        for (int j = 0; j < n; ++j) {
-            const int r = s * a.g.rps + j;
-            for (int i = threadIdx.x; i < dm; i += MMA_THREADS) d.hidden[(size_t)r * dm + i] = hidden_at(a, c, r, i);
-        }
-    if (threadIdx.x == 0) {
-        SeqState &st = d.st[s];
-        if (which == PACER_TARGET) st.len_T += n;
-        else if (which == PACER_DRAFT) st.len_D += n;
-        else st.len_B += n;
-    }
-}
-
-// End of one autoregressive target step (Eq. 1).
-__device__ __forceinline__ void tail_ar(Ctx &c, const Args &a, int s) {
-    if (c.n_rows[s] == 0) return;
-    const DevPtrs &d = a.d;
-    SeqState &st = d.st[s];
-    int tok = d.row_arg[s * a.g.rps];
-    if (st.mode == PACER_SAMPLE)
-        tok = gumbel_argmax(d.verify_logits + (size_t)s * (d.gamma_cap + 1) * a.m.cfg.vocab, a.m.cfg.vocab, st.seed, st.P, s,
-                            TAG_NEXT, MMA_THREADS, reinterpret_cast<BestD *>(c.scratch), true);
-    if (threadIdx.x != 0) return;
-    d.x[(size_t)s * d.max_ctx + st.P] = tok;
-    st.P += 1;
-    st.len_T += 1;
-    st.n_target_fwd += 1;
-    st.n_steps += 1;
-    if (st.P - st.n_prompt >= st.max_new) st.finished = 1;
-}
 
 // ------------------------------------------------------------------ the kernel
 
@@ -212,13 +82,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
         c.key_start[s] = ks;
     }
     __syncthreads();
-    int any = 0;
-    for (int s = 0; s < g.batch; ++s) any |= c.n_rows[s];
+    int live = 0;
+    for (int s = 0; s < g.batch; ++s) live += c.n_rows[s];
+    if (live <= a.few_max && a.few_max > 0) return;     // done by k_few already (the same decision in every block)
     if (c.cta == 0 && threadIdx.x < MAX_ROWS) {
         if (threadIdx.x < g.batch && threadIdx.x < MAX_SEQ) d.n_rows[threadIdx.x] = c.n_rows[threadIdx.x];
         if (threadIdx.x < g.rtot) { d.row_pos[threadIdx.x] = c.row_pos[threadIdx.x]; d.row_tok[threadIdx.x] = c.row_tok[threadIdx.x]; }
     }
-    if (!any) return;                       // every sequence idles: the same decision in every block
+    if (!live) return;                      // every sequence idles: the same decision in every block
 
     if (threadIdx.x < MAX_ROWS) {           // where the LM-head rows go
         const int r = threadIdx.x;
@@ -369,7 +240,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
         }
     }
     if (c.cta < g.batch && kind != KIND_VERIFY) {
-        if (kind != KIND_AR) tail_inv_rms(c, a, c.cta);     // the tails below apply the final RMSNorm themselves
+        // the final RMSNorm of the hidden rows the pre-verification model will read
+        if (kind == KIND_DRAFT || (kind == KIND_PREFILL && which == PACER_DRAFT)) tail_inv_rms(c, a, c.cta);
         if (kind == KIND_DRAFT) tail_draft(c, a, c.cta);
         else if (kind == KIND_MB) tail_mb(c, a, c.cta);
         else if (kind == KIND_AR) tail_ar(c, a, c.cta);
@@ -452,7 +324,7 @@ static inline Plan make_plan(const ModelDev &m, const DevPtrs &d, const FwdBufs 
 }
 
 template <int NT, bool TWO, bool BIG>
-static inline cudaError_t launch_nt(const Args &a, int which, int ncta, cudaStream_t st) {
+cudaError_t launch_nt(const Args &a, int which, int ncta, cudaStream_t st) {
     static bool attr_set[64] = {};           // the opt-in is per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -465,6 +337,17 @@ static inline cudaError_t launch_nt(const Args &a, int which, int ncta, cudaStre
     void *params[] = {(void *)&a, (void *)&which};
     return cudaLaunchCooperativeKernel((const void *)k_forward<NT, TWO, BIG>, dim3(ncta), dim3(THREADS), params, SMEM_BYTES, st);
 }
+
+// The variants are translation units of their own (fwd_nt*.cu): compiled together, their register allocation changes with
+// what else is there.
+#define FWD_VARIANT(NT, TWO, BIG) template cudaError_t launch_nt<NT, TWO, BIG>(const Args &, int, int, cudaStream_t)
+#ifndef FWD_INSTANTIATE
+extern FWD_VARIANT(1, false, false); extern FWD_VARIANT(1, true, false);
+extern FWD_VARIANT(2, false, false); extern FWD_VARIANT(2, true, false);
+extern FWD_VARIANT(3, false, false); extern FWD_VARIANT(3, true, false);
+extern FWD_VARIANT(4, false, false); extern FWD_VARIANT(4, true, false);
+extern FWD_VARIANT(6, false, true);
+extern FWD_VARIANT(8, false, true);
 
 // The variant with two accumulators runs the models in which some block has more than MMA_TILES tiles of a
 // projection; the wide variants (6 or 8 tiles per row group, up to three groups) the forwards with more than 32 rows.
@@ -480,5 +363,6 @@ static inline cudaError_t launch(const Args &a, int which, int ncta, cudaStream_
     }
     return cudaErrorInvalidValue;
 }
+#endif
 
 }  // namespace fwd

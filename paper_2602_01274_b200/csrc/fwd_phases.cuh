@@ -14,6 +14,7 @@ struct Args {
     Plan P;
     FwdBufs fb;
     int32_t kind, aux;
+    int32_t few_max;         // k_forward: a forward of at most this many live rows was k_few's
 };
 
 struct RowDesc {

@@ -14,6 +14,7 @@
 
 #include "common.cuh"
 #include "control.cuh"
+#include "fwd_few.h"
 #include "fwd_kernel.cuh"
 #include "gemm.cuh"
 
@@ -143,7 +144,7 @@ struct Carver {
 struct Layout {
     size_t st, x, y, alpha, hpend, hpend_e, draft_len, accept_len, sched_win, verify_logits, draft_logits;
     size_t row_pos, row_tok, n_rows, row_arg, row_margin, xres, att, act, hidden, part;
-    size_t att_cnt, bar, abort_flag, qkv, xg, ssq, tile_top, attp, prof;
+    size_t att_cnt, bar, abort_flag, qkv, xg, ssq, tile_top, attp, attf, prof;
     size_t kc[3], vc[3], rope[3];
     size_t wt[3][5], wt_bytes[3][5];   // the projections re-laid for the tensor cores
     size_t kv_bytes[3], rope_bytes[3];
@@ -194,7 +195,7 @@ static Layout make_layout(const pacer_cfg &c) {
     L.n_rows = cv.take(sizeof(int32_t) * fwd::MAX_SEQ);
     L.row_arg = cv.take(sizeof(int32_t) * fwd::MAX_ROWS);
     L.row_margin = cv.take(sizeof(float) * fwd::MAX_ROWS);
-    L.att_cnt = cv.take(sizeof(int32_t) * (size_t)B * h_max);
+    L.att_cnt = cv.take(sizeof(int32_t) * (size_t)(fwd::FEW_ROWS + 2) * fwd::FEW_ROWS * h_max);   // batch * kv heads * query chunks, at most 16 rows
     L.bar = cv.take(sizeof(unsigned long long));
     L.abort_flag = cv.take(sizeof(int32_t) * 4);
     L.prof = cv.take(sizeof(unsigned long long) * fwd::PROF_STAMPS * fwd::PROF_BLOCKS);
@@ -209,8 +210,9 @@ static Layout make_layout(const pacer_cfg &c) {
     L.act = cv.take(sizeof(bf16) * 2 * RP * f_max);
     L.qkv = cv.take(sizeof(float) * 4 * fwd::MAX_ROWS * qrows_max);     // up to four k slices, MAX_ROWS apart
     L.xg = cv.take(sizeof(bf16) * 2 * RP * d_max);
-    L.ssq = cv.take(sizeof(float) * fwd::MAX_ROWS * (d_max / 16 + 1));
-    L.tile_top = cv.take(sizeof(float) * 4 * fwd::MAX_ROWS * ((size_t)V / 16 + 1));
+    L.ssq = cv.take(sizeof(float) * std::max<size_t>(fwd::MAX_ROWS * (d_max / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
+    L.tile_top = cv.take(sizeof(float) * 4 * std::max<size_t>(fwd::MAX_ROWS * ((size_t)V / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
+    L.attf = cv.take(sizeof(float) * (size_t)fwd::FEW_ITEMS * fwd::FQ * (hd_max + 2));
     const int rps_all = std::max(rps_max, std::max(gc + 1, 128 / B));          // rows per sequence: verify, M_B, prompt chunks
     L.attp = cv.take(sizeof(float) * (size_t)B * h_max * fwd::MAX_SPLIT * rps_all * (hd_max + 2));
     L.part_bytes = sizeof(float) * 8 * (size_t)(d_max + 16) * RP;         // up to 8 k slices of [d/16][padded rows][16]
@@ -291,6 +293,7 @@ extern "C" int pacer_create(const pacer_cfg *cfg, void *dev_workspace, size_t wo
     c->fb.qkv = (float *)(w + L.qkv); c->fb.xg = (bf16 *)(w + L.xg); c->fb.ssq = (float *)(w + L.ssq);
     c->fb.part = (float *)(w + L.part);
     c->fb.tile_top = (float *)(w + L.tile_top); c->fb.attp = (float *)(w + L.attp);
+    c->fb.attf = (float *)(w + L.attf);
     c->fb.att_cnt = (int32_t *)(w + L.att_cnt); c->fb.bar = (unsigned long long *)(w + L.bar);
     c->fb.abort_flag = (int32_t *)(w + L.abort_flag);
     c->fb.prof = nullptr;
@@ -374,8 +377,9 @@ extern "C" int pacer_destroy(pacer_ctx *c) {
 // Re-lays one stack of [layers][N][K] row-major matrices into the order the forward kernel streams:
 // [layer][K/64][atoms][8 rows][64 k], an atom being 1 KB in the 128-byte swizzle layout of a K-major tensor-core
 // operand (the 16-byte chunk c of row r sits at chunk c ^ r).  Atom a holds rows 8a .. 8a+7 of W1, or, when W2 is
-// given (gate/up), rows 8(a/2) .. of W1 for even a and of W2 for odd a.  Rows past N are zeros.
-__global__ void k_retile(const bf16 *W1, const bf16 *W2, bf16 *out, int layers, int N, int K, int atoms) {
+// given (gate/up), rows 8(a/2) .. of W1 for even a and of W2 for odd a.  Rows past N are zeros.  The first `paired` rows
+// (the q and k heads, hd rows each) are stored as rotary pairs: rows 2i, 2i + 1 of a head are its channels i, i + hd/2.
+__global__ void k_retile(const bf16 *W1, const bf16 *W2, bf16 *out, int layers, int N, int K, int atoms, int paired, int hd) {
     const size_t total = (size_t)layers * (K / 64) * atoms * 64;          // 16-byte chunks
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int ch = (int)(i & 7), r = (int)((i >> 3) & 7);
@@ -386,6 +390,7 @@ __global__ void k_retile(const bf16 *W1, const bf16 *W2, bf16 *out, int layers, 
         const bf16 *src = W1;
         int row = a * 8 + r;
         if (W2) { row = (a >> 1) * 8 + r; if (a & 1) src = W2; }
+        if (row < paired) { const int w = row % hd; row += (w >> 1) + (w & 1) * (hd >> 1) - w; }
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (row < N) v = *reinterpret_cast<const uint4 *>(src + ((size_t)layer * N + row) * K + kb * 64 + ch * 8);
         *reinterpret_cast<uint4 *>(out + atom_lin * 512 + r * 64 + ((ch ^ r) << 3)) = v;
@@ -437,7 +442,8 @@ extern "C" int pacer_load_weights(pacer_ctx *c, int which, const pacer_tensor *t
         };
         for (const Job &jb : jobs) {
             if (!jb.w1 || !m.wt[jb.j]) continue;
-            k_retile<<<148 * 8, 256, 0, c->stream>>>(jb.w1, jb.w2, const_cast<bf16 *>(m.wt[jb.j]), jb.layers, jb.N, jb.K, jb.atoms);
+            k_retile<<<148 * 8, 256, 0, c->stream>>>(jb.w1, jb.w2, const_cast<bf16 *>(m.wt[jb.j]), jb.layers, jb.N, jb.K, jb.atoms,
+                                                        jb.j == 0 ? (k.n_heads + k.n_kv_heads) * m.hd : 0, m.hd);
             CK(cudaGetLastError());
         }
     }
@@ -478,8 +484,18 @@ static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux
     a.fb.prof = (c->prof_on && c->ncta <= fwd::PROF_BLOCKS) ? c->prof_stamps : nullptr;
     const bool prof = c->prof_on && which == PACER_TARGET && c->prof_used + 2 <= c->prof_ev.size();
     if (prof) CK(cudaEventRecord(c->prof_ev[c->prof_used], c->stream));
-    CK(fwd::launch(a, which, c->ncta, c->stream));
-    ++c->launches;
+    a.few_max = 0;
+    if (fwd::few_rows_ok(m, g, kind, c->ncta)) {
+        // The live rows are counted on the device: k_few takes the forward when they are at most 16, k_forward (launched
+        // behind it where the geometry allows more; a sequence that k_few has committed shows one row then) otherwise.
+        CK(fwd::launch_few(a, which, c->ncta, c->stream));
+        ++c->launches;
+        a.few_max = fwd::FEW_ROWS;
+    }
+    if (g.rtot > a.few_max) {
+        CK(fwd::launch(a, which, c->ncta, c->stream));
+        ++c->launches;
+    }
     if (prof) {
         CK(cudaEventRecord(c->prof_ev[c->prof_used + 1], c->stream));
         c->prof_used += 2;

@@ -118,7 +118,7 @@ constexpr int ACCEPT_THREADS = 1024;
 // kept while r_i <= p_i(y_i) / q_i(y_i) (tested as log r <= log p - log q); on the
 // first rejection the next token is drawn from norm(max(0, p - q)) of that
 // position, when all are kept from p_{gamma+1}; then commit, cache rollback, logs.
-__global__ void __launch_bounds__(ACCEPT_THREADS) k_accept_sample(DevPtrs d, Geom g, int V) {
+static __global__ void __launch_bounds__(ACCEPT_THREADS) k_accept_sample(DevPtrs d, Geom g, int V) {
     __shared__ double smd[32];
     __shared__ BestD smb[32];
     const int s = blockIdx.x;

@@ -1,0 +1,80 @@
+"""Forwards of few live rows (drafts, pre-verification calls, autoregressive steps, early-stopped windows) at the edges of
+their kernel: 1 to 17 live rows (8 and 16 are operand sizes, 17 is the other kernel's), fewer weight rows than blocks and
+several passes per block, grouped heads, both head sizes, contexts around the key splits.  The logits of every forward
+against the oracle's, 2e-2 as everywhere (the activations carry 16 mantissa bits: what is seen is below 1e-4)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import pacer_oracle as orc
+from paper_2602_01274_b200 import synth
+from tests.common import oracle_models
+
+pytestmark = pytest.mark.gpu
+TOL = 2e-2
+
+SHAPES = {
+    # head dimension 64, fewer two-row units than blocks in the residual projections, ragged vocabulary
+    "narrow": (synth.ModelShape(2, 128, 2, 1, 192, 1001), synth.ModelShape(1, 64, 1, 1, 64, 1001)),
+    # head dimension 128, three heads per kv head, several passes of the gate/up projection and the LM head
+    "passes": (synth.ModelShape(1, 768, 6, 2, 20480, 50000), synth.ModelShape(1, 256, 2, 2, 512, 50000)),
+}
+
+
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+@pytest.mark.parametrize("window,n_prompt", [(4, 2), (7, 33), (8, 97), (15, 40), (16, 300)])
+def test_verify_rows(shape, window, n_prompt):
+    from paper_2602_01274_b200 import binding as b
+    T, D = SHAPES[shape]
+    cfg = synth.PairConfig("few", T, D, agree=0.8, n_prompt=n_prompt, max_new=24, gamma_max=window, block_b=1 if window % 4 else 4)
+    gpu = synth.make_pair(cfg, seed=3, device="cuda:0")
+    cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
+    To, Do, Bo = oracle_models(cfg, cpu)
+    max_ctx = n_prompt + cfg.max_new + window + 2
+    ctx = b.Context(b.make_cfg(T, D, 1, max_ctx, window, cfg.block_b, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, gpu)
+    prompt = synth.make_prompts(T.vocab, 1, n_prompt, seed=9).numpy()
+    ctx.pacer_prefill(prompt, cfg.max_new, window, -1.0)
+    o = orc.Pacer(To, Do, Bo, max_ctx, b=cfg.block_b, gamma_cap=window, t0=-1.0, rho=cfg.rho)
+    o.prefill(prompt[0])
+    V, blocks = T.vocab, window // cfg.block_b
+    for k in range(blocks):
+        for _ in range(cfg.block_b):
+            ctx.pacer_draft_step()
+        ctx.pacer_preverify()
+        o.draft_block(); o.preverify()
+        if k not in (0, blocks - 1):
+            continue
+        ctx.pacer_verify()                          # 1 + the drafts so far live rows
+        if k == blocks - 1:
+            o.verify()
+            gamma = (k + 1) * cfg.block_b
+            got = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, (window + 1) * V).reshape(window + 1, V)[: gamma + 1]
+            y = ctx.pacer_read_buffer(b.BUF_DRAFTS, np.int32, window)[:gamma]
+            if o.stats()["min_margin_draft"] > 2 * TOL:
+                np.testing.assert_array_equal(y, o.y()[:gamma])
+                assert np.abs(got - o.plogits(gamma + 1)).max() < TOL
+                al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, window)[:gamma]
+                assert np.abs(al - o.alpha()[:gamma]).max() < 2e-3
+    ctx.close()
+
+
+@pytest.mark.parametrize("batch", [1, 9, 16, 17])
+def test_batched_autoregressive_rows(batch):
+    """One live row per sequence: packed rows of several sequences, and one sequence too many for the kernel."""
+    from paper_2602_01274_b200 import binding as b
+    T, D = SHAPES["narrow"]
+    cfg = synth.PairConfig("few", T, D, agree=0.8, n_prompt=21, max_new=6, gamma_max=4, batch=batch)
+    gpu = synth.make_pair(cfg, seed=4, device="cuda:0")
+    cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
+    To, _, _ = oracle_models(cfg, cpu)
+    ctx = b.Context(b.make_cfg(T, D, batch, 40, 4, 4, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, gpu)
+    prompts = synth.make_prompts(T.vocab, batch, cfg.n_prompt, seed=5).numpy()
+    tok, _ = ctx.pacer_generate_ar(prompts, cfg.max_new)
+    for s in range(batch):
+        out, margin = orc.generate_ar(To, prompts[s], cfg.max_new)
+        if margin > 2 * TOL:
+            np.testing.assert_array_equal(tok[s], out, err_msg=str(s))
+    ctx.close()
