@@ -17,6 +17,7 @@
 #include "fwd_few.h"
 #include "fwd_kernel.cuh"
 #include "gemm.cuh"
+#include "prefill.h"
 
 struct pacer_ctx {
     pacer_cfg cfg;
@@ -25,8 +26,10 @@ struct pacer_ctx {
     size_t ws_bytes;
     DevPtrs d;
     ModelDev model[3];
-    Geom g_draft, g_mb, g_verify, g_ar, g_prefill;
+    Geom g_draft, g_mb, g_verify, g_ar;
     fwd::FwdBufs fb;
+    pf::Bufs pf;
+    int pf_rows;
     int ncta;                  // blocks of the forward kernel (one per SM)
     std::map<int, fwd::Plan> plans;   // key: which * 2 + has_head
     unsigned long long *prof_stamps;
@@ -145,6 +148,8 @@ struct Layout {
     size_t st, x, y, alpha, hpend, hpend_e, draft_len, accept_len, sched_win, verify_logits, draft_logits;
     size_t row_pos, row_tok, n_rows, row_arg, row_margin, xres, att, act, hidden, part;
     size_t att_cnt, bar, abort_flag, qkv, xg, ssq, tile_top, attp, attf, prof;
+    size_t pf_x, pf_xg, pf_att, pf_act, pf_ssq;
+    int pf_rows;                       // rows of a prompt chunk at most
     size_t kc[3], vc[3], rope[3];
     size_t wt[3][5], wt_bytes[3][5];   // the projections re-laid for the tensor cores
     size_t kv_bytes[3], rope_bytes[3];
@@ -169,7 +174,7 @@ static Layout make_layout(const pacer_cfg &c) {
     const pacer_model_cfg *ms[3] = {&c.target, &c.draft, &mb};
     const int B = c.max_batch, gc = c.gamma_cap, V = c.target.vocab;
     const int rps_max = gc + 1 > c.block_b + 1 ? gc + 1 : c.block_b + 1;
-    L.rtot_max = std::max(B * rps_max, B * std::max(gc + 1, 128 / B));      // verify rows, prompt-chunk rows
+    L.rtot_max = std::max(B * rps_max, 32);                 // verify rows, prompts that go through the forward kernel
     L.nt_max = (L.rtot_max + 7) / 8;
     const size_t RP = std::min<size_t>(fwd::MAX_ROWS, make_geom(1, std::max(L.rtot_max, 32)).rpad);   // padded rows of the widest forward
     L.max_steps = c.max_ctx;
@@ -213,10 +218,13 @@ static Layout make_layout(const pacer_cfg &c) {
     L.ssq = cv.take(sizeof(float) * std::max<size_t>(fwd::MAX_ROWS * (d_max / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
     L.tile_top = cv.take(sizeof(float) * 4 * std::max<size_t>(fwd::MAX_ROWS * ((size_t)V / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
     L.attf = cv.take(sizeof(float) * (size_t)fwd::FEW_ITEMS * fwd::FQ * (hd_max + 2));
-    const int rps_all = std::max(rps_max, std::max(gc + 1, 128 / B));          // rows per sequence: verify, M_B, prompt chunks
+    const int rps_all = std::max(rps_max, 32);             // rows per sequence: verify, M_B, short prompts
     L.attp = cv.take(sizeof(float) * (size_t)B * h_max * fwd::MAX_SPLIT * rps_all * (hd_max + 2));
     L.part_bytes = sizeof(float) * 8 * (size_t)(d_max + 16) * RP;         // up to 8 k slices of [d/16][padded rows][16]
     L.part = cv.take(L.part_bytes);
+    L.pf_rows = (int)std::min<int64_t>(pf::ROWS, (int64_t)B * c.max_ctx);
+    const pf::Sizes ps = pf::sizes(d_max, d_max, f_max, L.pf_rows);
+    L.pf_x = cv.take(ps.x); L.pf_xg = cv.take(ps.xg); L.pf_att = cv.take(ps.att); L.pf_act = cv.take(ps.act); L.pf_ssq = cv.take(ps.ssq);
     for (int i = 0; i < 3; ++i) {
         const int hd = ms[i]->d_model / ms[i]->n_heads;
         L.kv_bytes[i] = 2 * sizeof(bf16) * (size_t)ms[i]->n_layers * B * ms[i]->n_kv_heads * c.max_ctx * hd;   // values + remainders
@@ -253,8 +261,6 @@ static void set_geoms(pacer_ctx *c, int batch, int draft_rows = 2) {
     c->g_mb = make_geom(batch, c->cfg.block_b + 1);
     c->g_verify = make_geom(batch, c->cfg.gamma_cap + 1);
     c->g_ar = make_geom(batch, 1);
-    // prompt chunks: as many rows per sequence as keep the forward at 128 rows (two full row groups)
-    c->g_prefill = make_geom(batch, std::max(c->cfg.gamma_cap + 1, 128 / batch));
 }
 
 extern "C" int pacer_create(const pacer_cfg *cfg, void *dev_workspace, size_t workspace_bytes, void *cuda_stream,
@@ -297,6 +303,9 @@ extern "C" int pacer_create(const pacer_cfg *cfg, void *dev_workspace, size_t wo
     c->fb.att_cnt = (int32_t *)(w + L.att_cnt); c->fb.bar = (unsigned long long *)(w + L.bar);
     c->fb.abort_flag = (int32_t *)(w + L.abort_flag);
     c->fb.prof = nullptr;
+    c->pf.x = (float *)(w + L.pf_x); c->pf.xg = (bf16 *)(w + L.pf_xg); c->pf.att = (bf16 *)(w + L.pf_att);
+    c->pf.act = (bf16 *)(w + L.pf_act); c->pf.q = (float *)(w + L.pf_act); c->pf.ssq = (float *)(w + L.pf_ssq);
+    c->pf_rows = L.pf_rows;
     c->prof_stamps = (unsigned long long *)(w + L.prof);
     c->ncta = sm_count_or_default();
     d.max_batch = cfg->max_batch; d.max_ctx = cfg->max_ctx; d.gamma_cap = cfg->gamma_cap; d.block_b = cfg->block_b;
@@ -563,18 +572,32 @@ static int start_run(pacer_ctx *c, const int32_t *prompt, int batch, int n_promp
     return PACER_OK;
 }
 
-static int prefill_models(pacer_ctx *c, int n_prompt, bool target, bool draft_and_mb, bool mb = true) {
-    const Geom &g = c->g_prefill;
-    for (int c0 = 0; c0 < n_prompt - 1; c0 += g.rps) {
-        int rc;
-        if (target) {
-            if ((rc = run_forward(c, PACER_TARGET, g, KIND_PREFILL, c0, false))) return rc;
-        }
-        if (draft_and_mb) {
-            if ((rc = run_forward(c, PACER_DRAFT, g, KIND_PREFILL, c0, false))) return rc;
-            if (mb && (rc = run_forward(c, PACER_PREVERIFY, g, KIND_PREFILL_B, c0, false))) return rc;
-        }
+// Prompt tokens 0 .. n_prompt-2 through the models.  Few rows in all: one forward of the forward kernel per model.  More:
+// chunks of up to pf_rows rows as tiled GEMMs (the weights are read once per chunk, the tensor cores are the bound).
+static int prefill_models(pacer_ctx *c, int n_prompt, bool target, bool draft, bool mb = true) {
+    const int n = n_prompt - 1, batch = c->batch;
+    int rc;
+    if (n < 1) return PACER_OK;
+    if ((int64_t)batch * n < pf::MIN_ROWS) {
+        const Geom g = make_geom(batch, n);
+        if (target && (rc = run_forward(c, PACER_TARGET, g, KIND_PREFILL, 0, false))) return rc;
+        if (draft && (rc = run_forward(c, PACER_DRAFT, g, KIND_PREFILL, 0, false))) return rc;
+        if (draft && mb && (rc = run_forward(c, PACER_PREVERIFY, g, KIND_PREFILL_B, 0, false))) return rc;
+        return PACER_OK;
     }
+    const int chunk = std::min(n, c->pf_rows / batch);
+    for (int c0 = 0; c0 < n; c0 += chunk) {
+        const int nj = std::min(chunk, n - c0);
+        auto model = [&](int which, pf::Input input, bool need_x) {
+            return pf::run(c->model[which], c->d, c->pf, c->fb.abort_flag, batch, nj, c0, input, c->model[PACER_DRAFT].normf, need_x, c->ncta,
+                           c->stream, &c->launches);
+        };
+        if (target) CK(model(PACER_TARGET, pf::EMBED, false));
+        if (draft) CK(model(PACER_DRAFT, pf::EMBED, mb));
+        if (draft && mb) CK(model(PACER_PREVERIFY, pf::HIDDEN, false));
+    }
+    CK(pf::set_lengths(c->d, batch, n, target, draft, draft && mb, c->stream));
+    LAUNCH_CHECK();
     return PACER_OK;
 }
 
