@@ -1,8 +1,9 @@
 // Skinny weight-streaming product: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32, bf16 in, fp32 sums, ONE launch.
 //
 // Bound by reading W once from HBM.  Every lane reads its share of W with 128-bit loads straight into registers
-// (each weight is used exactly once, so staging it in shared memory would only add traffic), 6 to 24 loads in flight
-// per lane, and the activations the same way out of L2, in the order the tensor cores want them.  mma.m16n8k16 with
+// (each weight is used exactly once, so staging it in shared memory would only add traffic), 8 to 32 loads in flight
+// per lane.  The activations come out of L2 through shared memory, eight chunks ahead: a lane copies exactly the 16-byte
+// pieces that it reads, so nothing is synchronised.  mma.m16n8k16 with
 // the token rows as the 16-row operand and eight weight rows as the other: a lane (g = lane / 4, t = lane % 4) loads the
 // 8 consecutive k of its row at 32c + 8t and uses them as the k slots {2t, 2t+1, 2t+8, 2t+9} of two MMAs; both operands
 // follow the rule, so the products pair up and the sum over k is the same.
@@ -40,10 +41,10 @@ struct LinArgs {
 
 constexpr int LIN_THREADS = 256, LIN_SMS = 148;
 
-// Loads in flight per lane: D chunks of TT weight tiles; the activations of XD chunks (a chunk of one or two tiles is
-// over before an L2 read returns, so there they run as far ahead as the weights).
-__host__ __device__ constexpr int lin_depth(int TT) { return TT >= 6 ? 3 : TT >= 4 ? 4 : 6; }
-__host__ __device__ constexpr int lin_xdepth(int TT) { return TT >= 4 ? 2 : lin_depth(TT); }
+// Weight loads in flight per lane: D chunks of TT tiles (about 100 KB per SM where registers allow); activations: LIN_XD
+// chunks.  (With the activations in registers, two chunks ahead, 17 x 4096 x 11008 took 30 us: every chunk waited for L2.)
+__host__ __device__ constexpr int lin_depth(int TT) { return TT >= 7 ? 4 : TT == 6 ? 5 : TT >= 4 ? 6 : 8; }
+constexpr int LIN_XD = 8;
 
 __device__ __forceinline__ uint32_t lin_peer(uint32_t smem_addr, int rank) {
     uint32_t r;
@@ -53,8 +54,9 @@ __device__ __forceinline__ uint32_t lin_peer(uint32_t smem_addr, int rank) {
 
 template <int RM, int TT>
 __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
-    constexpr int D = lin_depth(TT), XD = lin_xdepth(TT), R = RM * 16;
-    extern __shared__ __align__(16) float lin_red[];               // [8 warps][R rows][TT * 8 columns]
+    constexpr int D = lin_depth(TT), R = RM * 16;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    float *lin_red = reinterpret_cast<float *>(smem);              // [8 warps][R rows][TT * 8 columns], after the products
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int slice = blockIdx.x % a.S, grp = blockIdx.x / a.S;
     const int KW = 8 / a.NW, nw = warp / KW, kw = warp % KW;
@@ -68,9 +70,10 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
 #pragma unroll
     for (int i = 0; i < TT; ++i)                                    // tiles past the end repeat a valid row
         wp[i] = a.w + (size_t)min((t0 + min(w0 + i, max(w1 - 1, 0))) * 8 + g, a.N - 1) * a.K + (size_t)(c_lo + kw) * 32 + 8 * t;
-    const bf16 *xp = a.x + (size_t)g * a.K + (size_t)(c_lo + kw) * 32 + 8 * t;
+    const bf16 *xp = a.x + (size_t)min(g, a.rows - 1) * a.K + (size_t)(c_lo + kw) * 32 + 8 * t;
     const size_t step = (size_t)KW * 32;
-    uint4 w[D][TT], xv[XD][RM][2];
+    uint4 w[D][TT];
+    unsigned char *xs = smem + warp * (LIN_XD * R * 64) + lane * 16;   // [chunk][8-row half][lane] x 16 bytes
     float acc[TT][RM][4];
 #pragma unroll
     for (int i = 0; i < TT; ++i)
@@ -80,48 +83,54 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
 #pragma unroll
         for (int i = 0; i < TT; ++i) w[slot][i] = ldg_stream(wp[i] + (size_t)c * step);
     };
-    auto load_x = [&](int slot, int c) {
+    auto load_x = [&](int c) {                                      // a group per chunk, also when there is nothing to copy
+        if (c < mine) {
 #pragma unroll
-        for (int m = 0; m < RM; ++m)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const bf16 *p = xp + (size_t)(m * 16 + h * 8) * a.K + (size_t)c * step;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (m * 16 + h * 8 + g < a.rows) {
-                    if (a.x_aligned) v = __ldg(reinterpret_cast<const uint4 *>(p));
-                    else {
-                        const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
-                        v = make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16, q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
-                    }
+            for (int i = 0; i < 2 * RM; ++i) {
+                const bool in = i * 8 + g < a.rows;
+                const bf16 *p = xp + (in ? (size_t)(i * 8) * a.K : 0) + (size_t)c * step;    // (an idle row reads nothing)
+                unsigned char *dst = xs + ((c % LIN_XD) * 2 * RM + i) * 512;
+                if (a.x_aligned)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(p), "r"(in ? 16 : 0) : "memory");
+                else {
+                    const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
+                    *reinterpret_cast<uint4 *>(dst) = in ? make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16, q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16)
+                                                         : make_uint4(0u, 0u, 0u, 0u);
                 }
-                xv[slot][m][h] = v;
             }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
+    for (int j = 0; j < D; ++j)
         if (j < mine) load_w(j, j);
-        if (j < XD && j < mine) load_x(j, j);
-    }
-    constexpr int U = D % XD == 0 ? D : D * XD;                     // both rings back at slot 0
-    for (int c0 = 0; c0 < mine; c0 += U) {
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
+    for (int j = 0; j < LIN_XD - 1; ++j) load_x(j);
+    for (int c0 = 0; c0 < mine; c0 += D) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
             const int c = c0 + j;
             if (c >= mine) break;
+            load_x(c + LIN_XD - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(LIN_XD - 1) : "memory");
+            uint4 xv[RM][2];
+#pragma unroll
+            for (int i = 0; i < 2 * RM; ++i) xv[i >> 1][i & 1] = *reinterpret_cast<const uint4 *>(xs + ((c % LIN_XD) * 2 * RM + i) * 512);
 #pragma unroll
             for (int i = 0; i < TT; ++i) {
-                const uint4 b = w[j % D][i];
+                const uint4 b = w[j][i];
 #pragma unroll
                 for (int m = 0; m < RM; ++m) {
-                    const uint4 p = xv[j % XD][m][0], q = xv[j % XD][m][1];
+                    const uint4 p = xv[m][0], q = xv[m][1];
                     mma_bf16_16816(acc[i][m], p.x, q.x, p.y, q.y, b.x, b.y);
                     mma_bf16_16816(acc[i][m], p.z, q.z, p.w, q.w, b.z, b.w);
                 }
             }
-            if (c + D < mine) load_w(j % D, c + D);
-            if (c + XD < mine) load_x(j % XD, c + XD);
+            if (c + D < mine) load_w(j, c + D);
         }
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                                // the activations' bytes become the sums'
     // accumulator (g, 2t..): token row m*16 + g (+8), weight row 8i + 2t (+1)
     constexpr int P = TT * 8;
     float *my = lin_red + (size_t)warp * R * P;
@@ -199,7 +208,8 @@ static inline LinPlan lin_plan(int N, int K) {
 
 template <int RM, int TT>
 static cudaError_t lin_launch(const LinArgs &a, cudaStream_t st) {
-    constexpr size_t smem = (size_t)8 * RM * 16 * TT * 8 * sizeof(float);
+    constexpr size_t sums = (size_t)8 * RM * 16 * TT * 8 * sizeof(float), ring = (size_t)8 * LIN_XD * RM * 16 * 64;
+    constexpr size_t smem = sums > ring ? sums : ring;
     static bool attr_set[64] = {};           // the opt-in is per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
