@@ -74,6 +74,9 @@ struct FewCtx {
     float **row_dst;               // [FEW_ROWS] where an LM-head row goes, or NULL
     int32_t *bias_at;              // [FEW_ROWS] column of the planted bias, or -1
     Top2 *top;                     // [FEW_ROWS] best two logits of this block's columns so far
+    int32_t *draw_pos;             // [FEW_ROWS] position of the token that is drawn from an LM-head row (sampling), or -1
+    uint64_t *seed;                // [FEW_ROWS]
+    BestD *best;                   // [FEW_ROWS] best Gumbel score of this block's columns so far
     int x0, xc;                    // this block's columns of the residual stream
 };
 
@@ -263,6 +266,21 @@ __device__ __forceinline__ Top2 few_warp_top2(Top2 tp) {
     return tp;
 }
 
+__device__ __forceinline__ BestD few_warp_best(BestD t) {
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1) {
+        BestD u;
+        u.v = __shfl_xor_sync(0xffffffffu, t.v, x);
+        u.i = __shfl_xor_sync(0xffffffffu, t.i, x);
+        t = best_merge(t, u);
+    }
+    return t;
+}
+// the blocks' draws, behind their best logits: [block][FEW_ROWS]
+__device__ __forceinline__ BestD *few_best(const Args &a, const FewCtx &c) {
+    return reinterpret_cast<BestD *>(reinterpret_cast<float4 *>(a.fb.tile_top) + (size_t)c.ncta * FEW_ROWS);
+}
+
 // The row-wise step after a projection, weight rows [ra, rb) of live row i (one warp; red: the k groups' sums, column 0 =
 // weight row `off`, groups `ks` floats apart; last: the last pass).
 __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, int l, int i, int ra, int rb, int off, const float *red,
@@ -309,21 +327,38 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
         if (!dst) return;
         const int V = m.cfg.vocab, b = c.bias_at[i];
         Top2 tp{-INFINITY, 0x7fffffff, -INFINITY};
+        BestD bd{-INFINITY, 0x7fffffff};
+        const int dpos = c.draw_pos[i];
+        // a draw from the row's softmax by the Gumbel-max rule, every block on its own columns (one block over all of them
+        // took 0.08 ms at vocabulary 32 000: the noise is fp64)
+        auto draw = [&](int n, float v) {
+            if (dpos < 0) return;
+            const double sc = (double)v + gumbel_noise(c.seed[i], (uint32_t)n, (uint32_t)dpos, (uint32_t)(c.row_of[i] / a.g.rps), a.kind == KIND_DRAFT ? TAG_DRAFT : TAG_NEXT);
+            if (sc > bd.v) { bd.v = sc; bd.i = n; }
+        };
         for (int n = ra + 2 * c.lane; n < rb; n += 64) {
             const float2 s = few_sum(red + (n - off), ks);
             if (n < V) {
                 const float v = s.x * inv + (n == b ? d.succ_bias : 0.f);
                 dst[n] = v;
+                draw(n, v);
                 tp = top2_merge(tp, Top2{v, n, -INFINITY});
             }
             if (n + 1 < V) {
                 const float v = s.y * inv + (n + 1 == b ? d.succ_bias : 0.f);
                 dst[n + 1] = v;
+                draw(n + 1, v);
                 tp = top2_merge(tp, Top2{v, n + 1, -INFINITY});
             }
         }
         tp = few_warp_top2(tp);
+        if (dpos >= 0) bd = few_warp_best(bd);
         if (c.lane == 0) {
+            if (dpos >= 0) {
+                bd = best_merge(c.best[i], bd);
+                c.best[i] = bd;
+                if (last) few_best(a, c)[(size_t)c.cta * FEW_ROWS + i] = bd;
+            }
             tp = top2_merge(c.top[i], tp);               // (a block may have several passes of rows)
             c.top[i] = tp;
             if (last)
@@ -477,8 +512,10 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
     }
     if (o.npass == 0 && opi != OP_QKV && opi != OP_GU)   // fewer units than blocks: this one has no row, but its slots of
         for (int i = threadIdx.x; i < nlive; i += FC_THREADS) {              // the row statistics are read
-            if (opi == OP_HEAD) reinterpret_cast<float4 *>(a.fb.tile_top)[(size_t)c.cta * FEW_ROWS + i] = make_float4(-INFINITY, __int_as_float(0x7fffffff), -INFINITY, 0.f);
-            else a.fb.ssq[i * c.ncta + c.cta] = 0.f;
+            if (opi == OP_HEAD) {
+                reinterpret_cast<float4 *>(a.fb.tile_top)[(size_t)c.cta * FEW_ROWS + i] = make_float4(-INFINITY, __int_as_float(0x7fffffff), -INFINITY, 0.f);
+                few_best(a, c)[(size_t)c.cta * FEW_ROWS + i] = BestD{-INFINITY, 0x7fffffff};
+            } else a.fb.ssq[i * c.ncta + c.cta] = 0.f;
         }
 }
 
@@ -762,9 +799,12 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     c.bias_at = c.row_of + FEW_ROWS;
     c.inv = reinterpret_cast<float *>(c.bias_at + FEW_ROWS);
     c.top = reinterpret_cast<Top2 *>(c.inv + FEW_ROWS);                      // [FEW_ROWS]
-    c.flag = reinterpret_cast<int32_t *>(c.top + FEW_ROWS);                  // 4 words: attention's last arrival, live rows
+    c.best = reinterpret_cast<BestD *>(c.top + FEW_ROWS);                    // [FEW_ROWS]
+    c.seed = reinterpret_cast<uint64_t *>(c.best + FEW_ROWS);                // [FEW_ROWS]
+    c.draw_pos = reinterpret_cast<int32_t *>(c.seed + FEW_ROWS);             // [FEW_ROWS]
+    c.flag = c.draw_pos + FEW_ROWS;                                          // 4 words: attention's last arrival / the drawn token, live rows
     static_assert(8 * (2 * FNB + 2 * FXS + 1) + 4 * FNB + sizeof(FewOp) * N_OPS + 8 * FEW_ROWS + 4 * (3 * MAX_ROWS + 2 * MAX_SEQ + 3 * FEW_ROWS) +
-                  12 * FEW_ROWS + 16 <= F_MISC - F_XBYTES, "tables");
+                  (12 + 16 + 8 + 4) * FEW_ROWS + 16 <= F_MISC - F_XBYTES, "tables");
     static_assert(sizeof(FewOp) * N_OPS % 8 == 0, "alignment of the pointer table");
     c.xs = reinterpret_cast<float *>(misc + F_MISC - F_XBYTES);
     c.bar_target = 0; c.ok = true; c.stage = 0; c.xstage = 0; c.pass = 0;
@@ -857,6 +897,10 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
             if (m.succ) b = m.succ[c.row_tok[r]];
         }
         c.row_dst[i] = dst; c.bias_at[i] = b;
+        const SeqState &st = d.st[s];
+        c.draw_pos[i] = dst && st.mode == PACER_SAMPLE && kind != KIND_VERIFY ? st.P + (kind == KIND_DRAFT ? st.gamma : 0) : -1;
+        c.seed[i] = st.seed;
+        c.best[i] = BestD{-INFINITY, 0x7fffffff};
         c.top[i] = Top2{-INFINITY, 0x7fffffff, -INFINITY};
     }
     if (c.cta == 0 && threadIdx.x < MAX_ROWS) {
@@ -917,6 +961,15 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
             }
             tp = few_warp_top2(tp);
             if (c.lane == 0) { d.row_arg[r] = tp.i1; d.row_margin[r] = tp.v1 - tp.v2; }
+            if (c.draw_pos[i] >= 0) {           // (one row of the sequence at most)
+                BestD bd{-INFINITY, 0x7fffffff};
+                for (int b = c.lane; b < c.ncta; b += 32) {
+                    const BestD *p = few_best(a, c) + (size_t)b * FEW_ROWS + i;
+                    bd = best_merge(bd, BestD{__ldcg(&p->v), __ldcg(&p->i)});
+                }
+                bd = few_warp_best(bd);
+                if (c.lane == 0) c.flag[0] = bd.i;
+            }
         }
         fsync();
         if (kind == KIND_VERIFY && a.aux && threadIdx.x == 0) accept_greedy_seq(d, g, c.cta);
@@ -926,9 +979,9 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
         t.warp = c.warp; t.lane = c.lane; t.cta = c.cta; t.ncta = c.ncta;
         t.scratch = c.scratch; t.n_rows = c.n_rows; t.row_tok = c.row_tok; t.row_pos = c.row_pos;
         t.inv_rms = reinterpret_cast<float *>(c.scratch) + 1024;             // [MAX_ROWS], beside what the tails use
-        if (kind == KIND_DRAFT) { tail_inv_rms(t, a, t.cta); tail_draft(t, a, t.cta); }
+        if (kind == KIND_DRAFT) { tail_inv_rms(t, a, t.cta); tail_draft(t, a, t.cta, c.flag[0]); }
         else if (kind == KIND_MB) tail_mb(t, a, t.cta);
-        else if (kind == KIND_AR) tail_ar(t, a, t.cta);
+        else if (kind == KIND_AR) tail_ar(t, a, t.cta, c.flag[0]);
     }
     stamp();
 }

@@ -28,6 +28,7 @@ struct pacer_ctx {
     ModelDev model[3];
     Geom g_draft, g_mb, g_verify, g_ar;
     fwd::FwdBufs fb;
+    AcceptBufs acc;
     pf::Bufs pf;
     int pf_rows;
     int ncta;                  // blocks of the forward kernel (one per SM)
@@ -148,6 +149,7 @@ struct Layout {
     size_t st, x, y, alpha, hpend, hpend_e, draft_len, accept_len, sched_win, verify_logits, draft_logits;
     size_t row_pos, row_tok, n_rows, row_arg, row_margin, xres, att, act, hidden, part;
     size_t att_cnt, bar, abort_flag, qkv, xg, ssq, tile_top, attp, attf, prof;
+    size_t acc_lse, acc_pick, acc_arrived;
     size_t pf_x, pf_xg, pf_att, pf_act, pf_ssq;
     int pf_rows;                       // rows of a prompt chunk at most
     size_t kc[3], vc[3], rope[3];
@@ -201,10 +203,13 @@ static Layout make_layout(const pacer_cfg &c) {
     L.row_arg = cv.take(sizeof(int32_t) * fwd::MAX_ROWS);
     L.row_margin = cv.take(sizeof(float) * fwd::MAX_ROWS);
     L.att_cnt = cv.take(sizeof(int32_t) * (size_t)(fwd::FEW_ROWS + 2) * fwd::FEW_ROWS * h_max);   // batch * kv heads * query chunks, at most 16 rows
+    L.acc_arrived = cv.take(sizeof(int32_t) * B);
     L.bar = cv.take(sizeof(unsigned long long));
     L.abort_flag = cv.take(sizeof(int32_t) * 4);
     L.prof = cv.take(sizeof(unsigned long long) * fwd::PROF_STAMPS * fwd::PROF_BLOCKS);
     L.state_bytes = cv.off;                                   // zeroed at create
+    L.acc_lse = cv.take(sizeof(double2) * B * (2 * gc + 1) * LSE_PARTS);
+    L.acc_pick = cv.take(sizeof(BestD) * B * PICK_PARTS);
     L.hpend = cv.take(sizeof(float) * B * (c.block_b + 1) * c.draft.d_model);
     L.verify_logits = cv.take(sizeof(float) * B * (gc + 1) * V);
     L.draft_logits = cv.take(sizeof(float) * B * gc * V);
@@ -216,7 +221,7 @@ static Layout make_layout(const pacer_cfg &c) {
     L.qkv = cv.take(sizeof(float) * 4 * fwd::MAX_ROWS * qrows_max);     // up to four k slices, MAX_ROWS apart
     L.xg = cv.take(sizeof(bf16) * 2 * RP * d_max);
     L.ssq = cv.take(sizeof(float) * std::max<size_t>(fwd::MAX_ROWS * (d_max / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
-    L.tile_top = cv.take(sizeof(float) * 4 * std::max<size_t>(fwd::MAX_ROWS * ((size_t)V / 16 + 1), fwd::FEW_ROWS * sm_count_or_default()));
+    L.tile_top = cv.take(sizeof(float) * 4 * std::max<size_t>(fwd::MAX_ROWS * ((size_t)V / 16 + 1), 2 * fwd::FEW_ROWS * sm_count_or_default()));
     L.attf = cv.take(sizeof(float) * (size_t)fwd::FEW_ITEMS * fwd::FQ * (hd_max + 2));
     const int rps_all = std::max(rps_max, 32);             // rows per sequence: verify, M_B, short prompts
     L.attp = cv.take(sizeof(float) * (size_t)B * h_max * fwd::MAX_SPLIT * rps_all * (hd_max + 2));
@@ -303,6 +308,7 @@ extern "C" int pacer_create(const pacer_cfg *cfg, void *dev_workspace, size_t wo
     c->fb.att_cnt = (int32_t *)(w + L.att_cnt); c->fb.bar = (unsigned long long *)(w + L.bar);
     c->fb.abort_flag = (int32_t *)(w + L.abort_flag);
     c->fb.prof = nullptr;
+    c->acc.lse = (double2 *)(w + L.acc_lse); c->acc.pick = (BestD *)(w + L.acc_pick); c->acc.arrived = (int32_t *)(w + L.acc_arrived);
     c->pf.x = (float *)(w + L.pf_x); c->pf.xg = (bf16 *)(w + L.pf_xg); c->pf.att = (bf16 *)(w + L.pf_att);
     c->pf.act = (bf16 *)(w + L.pf_act); c->pf.q = (float *)(w + L.pf_act); c->pf.ssq = (float *)(w + L.pf_ssq);
     c->pf_rows = L.pf_rows;
@@ -632,8 +638,11 @@ extern "C" int pacer_verify(pacer_ctx *c) {
 extern "C" int pacer_accept_rollback(pacer_ctx *c) {
     int rc = need_ready(c, true);
     if (rc) return rc;
-    if (c->mode == PACER_SAMPLE) k_accept_sample<<<c->batch, ACCEPT_THREADS, 0, c->stream>>>(c->d, c->g_verify, c->cfg.target.vocab);
-    else k_accept_greedy<<<1, 64, 0, c->stream>>>(c->d, c->g_verify);
+    if (c->mode == PACER_SAMPLE) {
+        k_lse_parts<<<dim3(2 * c->cfg.gamma_cap + 1, LSE_PARTS, c->batch), LSE_THREADS, 0, c->stream>>>(c->d, c->acc, c->cfg.target.vocab);
+        LAUNCH_CHECK();
+        k_accept_sample<<<dim3(PICK_PARTS, c->batch), PICK_THREADS, 0, c->stream>>>(c->d, c->acc, c->cfg.target.vocab);
+    } else k_accept_greedy<<<1, 64, 0, c->stream>>>(c->d, c->g_verify);
     LAUNCH_CHECK();
     return PACER_OK;
 }

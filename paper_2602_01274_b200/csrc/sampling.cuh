@@ -77,7 +77,7 @@ __device__ __forceinline__ int gumbel_argmax(const float *logits, int V, uint64_
     return block_best(t, sm, named_barrier).i;
 }
 
-// Block-wide sum of doubles (plain __syncthreads version, for the acceptance kernel).
+// Block-wide sum of doubles (plain __syncthreads version, for the acceptance kernels).
 __device__ __forceinline__ double block_sum_d(double v, double *sm) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -89,78 +89,121 @@ __device__ __forceinline__ double block_sum_d(double v, double *sm) {
     __syncthreads();
     return s;
 }
-__device__ __forceinline__ double block_max_d(double v, double *sm) {
+__device__ __forceinline__ float block_max_f(float v, double *sm) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = (double)v;
     __syncthreads();
-    double s = -INFINITY;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s = fmax(s, sm[i]);
+    float s = -INFINITY;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s = fmaxf(s, (float)sm[i]);
     __syncthreads();
     return s;
 }
 
-// log-sum-exp of one logits row (fp64 accumulation), result in every thread.
-__device__ __forceinline__ double block_lse(const float *row, int V, double *sm) {
-    double mx = -INFINITY;
-    for (int v = threadIdx.x; v < V; v += blockDim.x) mx = fmax(mx, (double)__ldcg(row + v));
-    mx = block_max_d(mx, sm);
-    double s = 0.0;
-    for (int v = threadIdx.x; v < V; v += blockDim.x) s += exp((double)__ldcg(row + v) - mx);
-    s = block_sum_d(s, sm);
-    return mx + log(s);
+// Acceptance by rejection sampling (Eq. 5).  The transcendentals are fp64 (a step at vocabulary 32 000 and window 8 has
+// 17 rows of exponentials and one of logarithms), so they are spread over the device: k_lse_parts takes every row that the
+// acceptance may need in LSE_PARTS pieces, k_accept_sample the vocabulary of the resampling in PICK_PARTS pieces.  One
+// block per sequence for all of it took 0.3 to 0.6 ms a step, these two 0.03 ms.
+constexpr int LSE_PARTS = 4, LSE_THREADS = 512, PICK_PARTS = 32, PICK_THREADS = 256;
+
+struct AcceptBufs {
+    double2 *lse;              // [batch][2 * gamma_cap + 1 rows][LSE_PARTS] (max, sum of exponentials): p rows, then q rows
+    BestD *pick;               // [batch][PICK_PARTS]
+    int32_t *arrived;          // [batch], zero between launches
+};
+
+// Row blockIdx.x of sequence blockIdx.z (target rows 0 .. gamma, then draft rows), piece blockIdx.y of its vocabulary.
+static __global__ void __launch_bounds__(LSE_THREADS) k_lse_parts(DevPtrs d, AcceptBufs ab, int V) {
+    __shared__ double smd[32];
+    const int row = blockIdx.x, part = blockIdx.y, s = blockIdx.z, gc = d.gamma_cap;
+    const SeqState &st = d.st[s];
+    if (!st.active || st.finished || d.n_rows[s] == 0) return;
+    const bool q = row > gc;
+    const int j = q ? row - gc - 1 : row;
+    if (j > st.gamma - (q ? 1 : 0)) return;
+    const float *x = q ? d.draft_logits + ((size_t)s * gc + j) * V : d.verify_logits + ((size_t)s * (gc + 1) + j) * V;
+    const int v0 = (int)((long long)V * part / LSE_PARTS), v1 = (int)((long long)V * (part + 1) / LSE_PARTS);
+    float m = -INFINITY;
+    for (int v = v0 + threadIdx.x; v < v1; v += LSE_THREADS) m = fmaxf(m, __ldcg(x + v));
+    m = block_max_f(m, smd);
+    double e = 0.0;
+    for (int v = v0 + threadIdx.x; v < v1; v += LSE_THREADS) e += exp((double)__ldcg(x + v) - (double)m);
+    e = block_sum_d(e, smd);
+    if (threadIdx.x == 0) ab.lse[((size_t)s * (2 * gc + 1) + row) * LSE_PARTS + part] = make_double2((double)m, e);
+}
+__device__ __forceinline__ double row_lse(const double2 *p) {          // (a piece of an empty vocabulary range: -inf, 0)
+    double M = -INFINITY, e = 0.0;
+    for (int i = 0; i < LSE_PARTS; ++i) M = fmax(M, __ldcg(&p[i].x));
+    for (int i = 0; i < LSE_PARTS; ++i)
+        if (__ldcg(&p[i].y) > 0.0) e += __ldcg(&p[i].y) * exp(__ldcg(&p[i].x) - M);
+    return M + log(e);
 }
 
-constexpr int ACCEPT_THREADS = 1024;
-
-// Acceptance by rejection sampling (Eq. 5), one block per sequence: draft y_i is
-// kept while r_i <= p_i(y_i) / q_i(y_i) (tested as log r <= log p - log q); on the
-// first rejection the next token is drawn from norm(max(0, p - q)) of that
-// position, when all are kept from p_{gamma+1}; then commit, cache rollback, logs.
-static __global__ void __launch_bounds__(ACCEPT_THREADS) k_accept_sample(DevPtrs d, Geom g, int V) {
-    __shared__ double smd[32];
+// Draft y_i is kept while r_i <= p_i(y_i) / q_i(y_i) (tested as log r <= log p - log q); on the first rejection the next
+// token is drawn from norm(max(0, p - q)) of that position, when all are kept from p_{gamma+1}; the last block of a
+// sequence to arrive merges the draws of the pieces, commits and rolls the caches back.
+static __global__ void __launch_bounds__(PICK_THREADS) k_accept_sample(DevPtrs d, AcceptBufs ab, int V) {
     __shared__ BestD smb[32];
-    const int s = blockIdx.x;
+    __shared__ double ratio[160];                    // log r - (log p - log q) of every draft (at most 143)
+    __shared__ int last;
+    const int part = blockIdx.x, s = blockIdx.y, gc = d.gamma_cap;
     SeqState &st = d.st[s];
     if (!st.active || st.finished || d.n_rows[s] == 0) return;
     const int gamma = st.gamma, P = st.P;
     const uint64_t seed = st.seed;
-    const int32_t *y = d.y + (size_t)s * d.gamma_cap;
-    const float *plog = d.verify_logits + (size_t)s * (d.gamma_cap + 1) * V;
-    const float *qlog = d.draft_logits + (size_t)s * d.gamma_cap * V;
-    int n = 0;
-    double lsp = 0.0, lsq = 0.0;
-    for (; n < gamma; ++n) {
-        const float *p = plog + (size_t)n * V, *q = qlog + (size_t)n * V;
-        lsp = block_lse(p, V, smd);
-        lsq = block_lse(q, V, smd);
-        const double lp = (double)__ldcg(p + y[n]) - lsp, lq = (double)__ldcg(q + y[n]) - lsq;
-        const double lr = log(uniform01(seed, 0u, (uint32_t)(P + n), (uint32_t)s, TAG_ACCEPT));
-        if (lr > lp - lq) break;                     // r > p / q: reject (the same value in every thread)
+    const int32_t *y = d.y + (size_t)s * gc;
+    const float *plog = d.verify_logits + (size_t)s * (gc + 1) * V;
+    const float *qlog = d.draft_logits + (size_t)s * gc * V;
+    const double2 *lse = ab.lse + (size_t)s * (2 * gc + 1) * LSE_PARTS;
+    for (int i = threadIdx.x; i < gamma; i += PICK_THREADS) {
+        const double lp = (double)__ldcg(plog + (size_t)i * V + y[i]) - row_lse(lse + i * LSE_PARTS);
+        const double lq = (double)__ldcg(qlog + (size_t)i * V + y[i]) - row_lse(lse + (gc + 1 + i) * LSE_PARTS);
+        ratio[i] = log(uniform01(seed, 0u, (uint32_t)(P + i), (uint32_t)s, TAG_ACCEPT)) - (lp - lq);
     }
-    int next;
+    __syncthreads();
+    int n = 0;
+    while (n < gamma && !(ratio[n] > 0.0)) ++n;      // r > p / q: reject
+    const int v0 = (int)((long long)V * part / PICK_PARTS), v1 = (int)((long long)V * (part + 1) / PICK_PARTS);
+    const float *p = plog + (size_t)n * V, *q = qlog + (size_t)n * V;
+    BestD t{-INFINITY, 0x7fffffff};
     if (n == gamma) {
-        next = gumbel_argmax(plog + (size_t)gamma * V, V, seed, P + gamma, s, TAG_NEXT, ACCEPT_THREADS, smb, false);
+        for (int v = v0 + threadIdx.x; v < v1; v += PICK_THREADS) {
+            const double sc = (double)__ldcg(p + v) + gumbel_noise(seed, (uint32_t)v, (uint32_t)(P + gamma), (uint32_t)s, TAG_NEXT);
+            if (sc > t.v) { t.v = sc; t.i = v; }
+        }
     } else {
-        const float *p = plog + (size_t)n * V, *q = qlog + (size_t)n * V;
-        BestD t{-INFINITY, 0x7fffffff};
-        for (int v = threadIdx.x; v < V; v += ACCEPT_THREADS) {
+        const double lsp = row_lse(lse + n * LSE_PARTS), lsq = row_lse(lse + (gc + 1 + n) * LSE_PARTS);
+        for (int v = v0 + threadIdx.x; v < v1; v += PICK_THREADS) {
             const double res = exp((double)__ldcg(p + v) - lsp) - exp((double)__ldcg(q + v) - lsq);
             if (!(res > 0.0)) continue;
             const double sc = log(res) + gumbel_noise(seed, (uint32_t)v, (uint32_t)(P + n), (uint32_t)s, TAG_NEXT);
             if (sc > t.v) { t.v = sc; t.i = v; }
         }
-        t = block_best(t, smb, false);
-        next = t.i;
-        if (t.i == 0x7fffffff) {                     // p == q exactly: cannot be rejected in exact arithmetic
-            BestD a{-INFINITY, 0x7fffffff};
-            for (int v = threadIdx.x; v < V; v += ACCEPT_THREADS) {
-                const double pv = (double)__ldcg(p + v);
-                if (pv > a.v) { a.v = pv; a.i = v; }
-            }
-            next = block_best(a, smb, false).i;
-        }
     }
-    if (threadIdx.x == 0) commit_step(d, st, s, n, next);
+    t = block_best(t, smb, false);
+    BestD *pick = ab.pick + (size_t)s * PICK_PARTS;
+    if (threadIdx.x == 0) {
+        pick[part] = t;
+        __threadfence();
+        last = atomicAdd(ab.arrived + s, 1) == PICK_PARTS - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    t = BestD{-INFINITY, 0x7fffffff};
+    for (int i = 0; i < PICK_PARTS; ++i) t = best_merge(t, BestD{__ldcg(&pick[i].v), __ldcg(&pick[i].i)});
+    int next = t.i;
+    if (next == 0x7fffffff) {                        // p == q exactly: cannot be rejected in exact arithmetic
+        BestD a{-INFINITY, 0x7fffffff};
+        for (int v = threadIdx.x; v < V; v += PICK_THREADS) {
+            const double pv = (double)__ldcg(p + v);
+            if (pv > a.v) { a.v = pv; a.i = v; }
+        }
+        next = block_best(a, smb, false).i;
+    }
+    if (threadIdx.x == 0) {
+        ab.arrived[s] = 0;
+        commit_step(d, st, s, n, next);
+    }
 }
