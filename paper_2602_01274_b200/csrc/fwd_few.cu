@@ -535,15 +535,21 @@ __device__ __forceinline__ FewAtt few_att(const FewCtx &c, const Args &a) {
             rows = max(rows, c.n_rows[s]);
         }
     f.chunks = (group * rows + FQ - 1) / FQ;
-    const int base = a.g.batch * a.m.cfg.n_kv_heads * f.chunks, cap = max(1, min(len / 32, FEW_ITEMS / base));
-    if (base <= c.ncta) f.nsplit = max(1, min(c.ncta / base, cap));
-    else {
-        // several rounds: the split with the least rounds x (keys of an item + about 96 keys' worth of fixed cost)
-        long long best_cost = -1;
+    // Key splits: an item costs about 1.3 us per round of its ten warps (80 keys) and 3 us of fixed cost; splitting adds 3 us
+    // for the partials, the arrival and the merge.  Fewer items than blocks: the most splits that give every block one
+    // item, or none when a head is that short (96 keys of 4 heads: 4 us against 6).
+    const int base = a.g.batch * a.m.cfg.n_kv_heads * f.chunks;
+    const int cap = max(1, min(min((len + 79) / 80, 64), FEW_ITEMS / base));
+    if (base <= c.ncta) {
+        const int n = min(cap, c.ncta / base), rounds = ((len + n - 1) / n + 79) / 80, alone = (len + 79) / 80;
+        // (as many splits as leave the same number of rounds)
+        f.nsplit = 13 * alone <= 13 * rounds + 30 ? 1 : min(n, (len + 80 * rounds - 1) / (80 * rounds));
+    } else {
+        int best_cost = 1 << 30;
         f.nsplit = 1;
         for (int n = 1; n <= min(cap, 16); ++n) {
-            const long long cost = (long long)((base * n + c.ncta - 1) / c.ncta) * (len / n + 96);
-            if (best_cost < 0 || cost < best_cost) { best_cost = cost; f.nsplit = n; }
+            const int cost = ((base * n + c.ncta - 1) / c.ncta) * (13 * (((len + n - 1) / n + 79) / 80) + 30) + (n > 1 ? 30 : 0);
+            if (cost < best_cost) { best_cost = cost; f.nsplit = n; }
         }
     }
     f.items = base * f.nsplit;
