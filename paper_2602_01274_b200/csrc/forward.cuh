@@ -302,7 +302,6 @@ __device__ __forceinline__ void grid_barrier(Ctx &c, const FwdBufs &fb) {
                 break;
             }
         }
-        __threadfence();
     }
     bsync();
 }

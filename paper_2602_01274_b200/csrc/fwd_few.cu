@@ -8,7 +8,7 @@
 //     rows of bf16 values over their 8 rows of rounding remainders, so ONE m16n8k16 covers 8 split rows) they need 1
 //     MMA per 128 weights, 7 % to 20 % of what the SM can issue while HBM delivers them, and no tensor-memory round
 //     trip, commit or accumulator copy stands between the last weight and the epilogue;
-//   - ten warps share k (five groups) and the block's rows (two halves); their sums meet in shared memory.  A stage costs
+//   - ten warps share k (five or ten groups) and the block's rows; their sums meet in shared memory.  A stage costs
 //     a warp 0.5 us of waits and dependent instructions however little it computes, so the groups work on different ones
 //     (all ten warps on every stage, without groups: 37 us for a 7B gate/up projection against 26);
 //   - no projection is cut along k across blocks, so the two residual projections need no reduction pass; a block owns
@@ -32,7 +32,7 @@
 
 namespace fwd {
 
-constexpr int FW = 10, FKG = 5, FCG = 2;        // consumer warps = k groups x weight row groups (with the two producers
+constexpr int FW = 10;                          // consumer warps = k groups x weight row groups (with the two producers
 constexpr int FC_THREADS = 32 * FW;             // three warps per scheduler: 168 registers a thread)
 constexpr int FEW_THREADS = FC_THREADS + 64;
 constexpr int FNB = 32;                         // weight stages in flight (barrier pairs; one lane each in the producer)
@@ -49,6 +49,7 @@ constexpr int F_XBYTES = 5120;                  // of F_MISC: this block's colum
 struct FewOp {
     int r0, r1, atom0, span;       // rows; first 8-row atom and atoms touched
     int nkb, kbs, nst, npass;      // 64-column k blocks, of a weight stage, weight stages; passes over the atoms
+    int kgs, pad;                  // k groups: 10 (a warp takes all atoms of a stage) or 5 (two warps share them)
 };
 
 struct FewCtx {
@@ -98,7 +99,6 @@ __device__ __forceinline__ void few_grid_barrier(FewCtx &c, const FwdBufs &fb) {
                 break;
             }
         }
-        __threadfence();
     }
     fsync();
 }
@@ -130,11 +130,14 @@ __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int 
     o.span = o.r1 > o.r0 ? ((o.r1 + 7) >> 3) - o.atom0 : 0;
     o.nkb = op.K / KB;
     // a pass: what the accumulators and the buffer of the sums hold (an even number of atoms)
-    const int atoms = min(nlive <= 8 ? F_PASS : 16, F_SCRATCH / (FKG * nlive * 32)) & ~1;
+    // few atoms: ten k groups, so that a warp's chain of k blocks is as short as it can be (14 rows x 5504 columns: 18 k
+    // blocks a warp with five groups, 9 with ten)
+    o.kgs = o.span <= 3 ? FW : FW / 2;
+    const int atoms = min(nlive <= 8 ? F_PASS : 16, F_SCRATCH / (o.kgs * nlive * 32)) & ~1;
     o.npass = (o.span + atoms - 1) / atoms;
     // stage: F_STAGE bytes of weights, but work for every k group
     const int sp = o.npass ? (o.span + o.npass - 1) / o.npass : 1;
-    o.kbs = max(1, min(min(32, (F_STAGE / 1024) / sp), (o.nkb + FKG - 1) / FKG));
+    o.kbs = max(1, min(min(32, (F_STAGE / 1024) / sp), (o.nkb + o.kgs - 1) / o.kgs));
     o.nst = (o.nkb + o.kbs - 1) / o.kbs;
     return o;
 }
@@ -244,13 +247,19 @@ __device__ __forceinline__ float2 few_input(const Args &a, const FewCtx &c, int 
     return make_float2(__low2float(w), __high2float(w));
 }
 
-__device__ __forceinline__ float2 few_sum(const float *p, int kstride) {
+__device__ __forceinline__ float2 few_sum(const float *p, int kstride, int kgs) {
     float2 v = *reinterpret_cast<const float2 *>(p);
 #pragma unroll
-    for (int k = 1; k < FKG; ++k) {
+    for (int k = 1; k < FW / 2; ++k) {
         const float2 u = *reinterpret_cast<const float2 *>(p + k * kstride);
         v.x += u.x; v.y += u.y;
     }
+    if (kgs == FW)
+#pragma unroll
+        for (int k = FW / 2; k < FW; ++k) {
+            const float2 u = *reinterpret_cast<const float2 *>(p + k * kstride);
+            v.x += u.x; v.y += u.y;
+        }
     return v;
 }
 
@@ -282,9 +291,9 @@ __device__ __forceinline__ BestD *few_best(const Args &a, const FewCtx &c) {
 }
 
 // The row-wise step after a projection, weight rows [ra, rb) of live row i (one warp; red: the k groups' sums, column 0 =
-// weight row `off`, groups `ks` floats apart; last: the last pass).
+// weight row `off`, the kgs groups `ks` floats apart; last: the last pass).
 __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, int l, int i, int ra, int rb, int off, const float *red,
-                                             int ks, bool last) {
+                                             int ks, int kgs, bool last) {
     const DevPtrs &d = a.d;
     const ModelDev &m = a.m;
     const int dm = m.cfg.d_model, H = m.cfg.n_heads, Hkv = m.cfg.n_kv_heads, hd = m.hd, half = hd >> 1;
@@ -295,7 +304,7 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
         for (int n = ra + 2 * c.lane; n < rb; n += 64) {
             const int h = n >> hshift, w = n & (hd - 1), ii = w >> 1;
             const float2 cs = h < H + Hkv ? m.rope[(size_t)pos * half + ii] : make_float2(1.f, 0.f);
-            const float2 s = few_sum(red + (n - off), ks);
+            const float2 s = few_sum(red + (n - off), ks, kgs);
             const float v0 = s.x * inv, v1 = s.y * inv;
             if (h < H + Hkv) {                           // the pair (ii, ii + hd/2) of a q or k head: rotary embedding
                 const float y0 = v0 * cs.x - v1 * cs.y, y1 = v1 * cs.x + v0 * cs.y;
@@ -318,7 +327,7 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
     } else if (opi == OP_GU) {                           // whole gate/up atom pairs: columns f = ra / 2 ..
         for (int f = (ra >> 1) + 2 * c.lane; f < (rb >> 1); f += 64) {
             const int n = (f >> 3) * 16 + (f & 7);
-            const float2 gt = few_sum(red + (n - off), ks), up = few_sum(red + (n + 8 - off), ks);
+            const float2 gt = few_sum(red + (n - off), ks, kgs), up = few_sum(red + (n + 8 - off), ks, kgs);
             const float g0 = gt.x * inv, g1 = gt.y * inv;
             few_store(d.act, i, f, c.nlive, g0 / (1.f + expf(-g0)) * (up.x * inv), g1 / (1.f + expf(-g1)) * (up.y * inv));
         }
@@ -337,7 +346,7 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
             if (sc > bd.v) { bd.v = sc; bd.i = n; }
         };
         for (int n = ra + 2 * c.lane; n < rb; n += 64) {
-            const float2 s = few_sum(red + (n - off), ks);
+            const float2 s = few_sum(red + (n - off), ks, kgs);
             if (n < V) {
                 const float v = s.x * inv + (n == b ? d.succ_bias : 0.f);
                 dst[n] = v;
@@ -371,7 +380,7 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
         float ss = 0.f, *xr = d.xres + (size_t)c.row_of[i] * dm;
         for (int n = ra + 2 * c.lane; n < rb; n += 64) {
             const __nv_bfloat162 gn = *reinterpret_cast<const __nv_bfloat162 *>(gain + n);
-            const float2 s = few_sum(red + (n - off), ks);
+            const float2 s = few_sum(red + (n - off), ks, kgs);
             float *x = c.xs + i * c.xc + (n - c.x0);
             const float x0 = x[0] + s.x, x1 = x[1] + s.y;
             x[0] = x0; x[1] = x1;
@@ -394,7 +403,11 @@ __device__ __forceinline__ void few_inv(FewCtx &c, const Args &a) {
     }
 }
 
-// One warp's share of a pass: the weight stages kg, kg + 5, ... and N atoms of them from atom my_a on (my_n of them
+__device__ __forceinline__ void mbar_arrive_n(uint64_t *b, int count) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+
+// One warp's share of a pass: the weight stages kg, kg + kgs, ... and N atoms of them from atom my_a on (my_n of them
 // its own, the rest is computed and not stored), into the sum buffer.  N is a template parameter because a branch per atom
 // costs more than the atom's instructions.  (A lane of an operand row beyond the live ones reads live row 0.)
 template <int RT, int N>
@@ -423,7 +436,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
         xb = c.scratch + slot * (F_XROWS * 256) - xs * xk * nlive * 256;
         ++xs;
     };
-    for (int st = kg; st < nst; st += FKG) {
+    for (int st = kg; st < nst; st += o.kgs) {
         const int n = c.stage + st, slot = n & (FNB - 1), k_end = min((st + 1) * o.kbs, o.nkb);
         // first the activations: a warp that waited for weights inside an earlier activation stage would hold that stage
         // back from a warp whose weights must be read before its own can arrive
@@ -457,7 +470,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
             }
         }
         __syncwarp();
-        if (c.lane == 0) mbar_arrive(c.wempty + slot);
+        if (c.lane == 0) mbar_arrive_n(c.wempty + slot, o.kgs == FW ? 2 : 1);    // (two arrivals in all)
     }
     while (xs <= nxs) next_x();
     fsync();                                             // the activations' bytes become the sums'
@@ -473,16 +486,16 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
                         make_float2(acc[i][m][0] + acc[i][m][2], acc[i][m][1] + acc[i][m][3]);
 }
 
-// A projection of the forward.  Warp (kg, cg) takes a fifth of the k range and the cg-th half of the pass's atoms; the k
-// groups' sums go through shared memory; then warp w runs the epilogue for the live rows w, w + 10.
+// A projection of the forward.  Warp (kg, cg) takes its share of the k range and of the pass's atoms; the k groups' sums
+// go through shared memory; then warp w runs the epilogue for the live rows w, w + 10.
 __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int layer) {
     const FewOp o = c.ops[opi];
-    const int kg = c.warp / FCG, cg = c.warp % FCG, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
+    const int kg = o.kgs == FW ? c.warp : c.warp >> 1, cg = c.warp & 1, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
     float *red = reinterpret_cast<float *>(c.scratch);
     for (int p = 0; p < o.npass; ++p) {
         int pa, pn;
         few_pass(o, p, pa, pn);
-        const int h0 = (pn + 1) >> 1, my_a = cg ? h0 : 0, my_n = cg ? pn - h0 : h0;
+        const int h0 = (pn + 1) >> 1, my_a = o.kgs < FW && cg ? h0 : 0, my_n = o.kgs == FW ? pn : cg ? pn - h0 : h0;
         if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // the activations may be copied
         // (its loads travel with the first activations)
         if ((opi == OP_QKV || opi == OP_GU || opi == OP_HEAD) && p == 0) few_inv(c, a);
@@ -507,7 +520,7 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
         fsync();
         const int PC = pn * 8, ra = max(o.r0, (o.atom0 + pa) * 8), rb = min(o.r1, (o.atom0 + pa + pn) * 8), off = (o.atom0 + pa) * 8;
         for (int i = c.warp; i < nlive; i += FW)
-            few_epilogue(c, a, opi, layer, i, ra, rb, off, red + i * PC, nlive * PC, p == o.npass - 1);
+            few_epilogue(c, a, opi, layer, i, ra, rb, off, red + i * PC, nlive * PC, o.kgs, p == o.npass - 1);
         if (p + 1 < o.npass) fsync();
     }
     if (o.npass == 0 && opi != OP_QKV && opi != OP_GU)   // fewer units than blocks: this one has no row, but its slots of
@@ -830,7 +843,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
         c.row_pos[r] = pos; c.row_tok[r] = tok;
     }
     if (threadIdx.x == FC_THREADS) {
-        for (int i = 0; i < FNB; ++i) { mbar_init(c.wfull + i, 1); mbar_init(c.wempty + i, FCG); }
+        for (int i = 0; i < FNB; ++i) { mbar_init(c.wfull + i, 1); mbar_init(c.wempty + i, 2); }
         for (int i = 0; i < FXS; ++i) { mbar_init(c.xfull + i, 1); mbar_init(c.xempty + i, FW); }
         *c.ready = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
