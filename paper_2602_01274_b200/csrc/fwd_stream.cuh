@@ -91,12 +91,6 @@ __device__ __forceinline__ void weight_producer(Ctx &c, const FwdBufs &fb, const
     }
 }
 
-// Tiles of a pass in the first accumulator: all of them, or half when there are more than one MMA takes (an MMA of
-// N = 144 takes 33 ns, of N = 256 61 ns and of N = 16 30 ns: 17 tiles as 9 + 8 are 0.26 us per k block, as 16 + 1 they
-// were 0.36).
-template <bool TWO>
-__device__ __forceinline__ int first_tiles(int Tp) { return TWO && Tp > MMA_TILES ? (Tp + 1) >> 1 : Tp; }
-
 // Lane 0 of warp MMA_ISSUER: the tensor-core instructions of every stage.  Per k block four MMAs of K = 16 per row
 // group; the A operand is the group's part of the activation stage (128 rows are read from its base: values,
 // remainders, then whatever follows in shared memory, which only reaches accumulator lanes nobody reads), the B
@@ -117,7 +111,7 @@ __device__ __forceinline__ void mma_issuer(Ctx &c, const FwdBufs &fb, const Plan
             int p0, Tp;
             pass_range(T, p, P.max_tiles, p0, Tp);
             const int bytes = Tp * 2048;
-            const int T0 = first_tiles<TWO>(Tp), T1 = Tp - T0;               // tiles of the first / second accumulator
+            const int T0 = TWO ? min(Tp, MMA_TILES) : Tp, T1 = Tp - T0;      // tiles of the first / second accumulator
             const uint32_t idesc = umma_idesc(T0 * 16), idesc1 = umma_idesc(T1 ? T1 * 16 : 16);
             // the phase warps have copied the previous pass's accumulator out
             if (!wait_bar(fb, c.acc_empty, (((uint32_t)np) & 1u) ^ 1u, 11, np)) return;
@@ -268,8 +262,8 @@ __device__ __forceinline__ void gemm_op(Ctx &c, const FwdBufs &fb, const Plan &P
         const int n_acc = BIG ? G : ((TWO && Tp > MMA_TILES) ? 2 : 1);      // accumulators of this pass
         bool first = true;
         for (int ai = 0; ai < n_acc; ++ai) {
-            const int T0 = first_tiles<TWO>(Tp), a_t0 = (!BIG && ai) ? T0 : 0;    // first tile of the pass in this accumulator
-            const int a_T = BIG ? Tp : (ai ? Tp - T0 : T0);
+            const int a_t0 = (!BIG && ai) ? MMA_TILES : 0;                 // first tile of the pass in this accumulator
+            const int a_T = BIG ? Tp : (TWO ? min(MMA_TILES, Tp - a_t0) : Tp);
             const uint32_t a_col = BIG ? (uint32_t)(ai * P.acc_stride) : (ai ? ACC_COLS : 0);
             const int rb = BIG ? ai * 8 * NT : 0;
             for (int c0 = 0; c0 < a_T; c0 += CH) {
