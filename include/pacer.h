@@ -212,8 +212,8 @@ int pacer_read_buffer(pacer_ctx *ctx, int which, void *host_dst, size_t bytes);
  * stop of the drafting, acceptance, rollback, end of generation) is taken on the
  * device; the host enqueues whole steps (every block of the window, each a no-op
  * for a sequence that has stopped drafting) and stays two steps ahead of the device:
- * it reads the finished flags of an EARLIER step from pinned memory (copied there
- * behind an event) to know when to stop enqueuing, and never waits for the step it
+ * it reads the finished flags in pinned memory (the acceptance writes them) behind
+ * an event of an EARLIER step to know when to stop enqueuing, and never waits for the step it
  * has just enqueued.  The launches of one step (the draft forwards and pre-verification
  * calls of the whole window, the verify forward, the acceptance) are captured once
  * per context as a CUDA graph and replayed every step (not on the legacy default

@@ -71,6 +71,7 @@ struct DevPtrs {
     int32_t *row_pos;    // [rtot] cache position of row r, -1 = inactive
     int32_t *row_tok;    // [rtot] input token (or draft index for M_B rows)
     int32_t *n_rows;     // [max_batch] active rows per sequence in this forward
+    int32_t *fin_out;    // [max_batch] pinned host memory: set to 1 when a sequence has finished
     int32_t *row_arg;    // [rtot] argmax of the LM-head row
     float *row_margin;   // [rtot] top1 - top2
     float *xres;         // [rtot][d] fp32 residual stream

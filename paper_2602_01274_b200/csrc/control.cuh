@@ -74,7 +74,11 @@ __device__ __forceinline__ void commit_step(const DevPtrs &d, SeqState &st, int 
         st.gamma_max = w;
         st.drafting = w > 0;
     }
-    if (st.P - st.n_prompt >= st.max_new) { st.finished = 1; st.drafting = 0; }
+    if (st.P - st.n_prompt >= st.max_new) {
+        st.finished = 1; st.drafting = 0;
+        *(volatile int32_t *)(d.fin_out + s) = 1;         // (the host looks at it behind an event)
+        __threadfence_system();
+    }
 }
 
 // Greedy acceptance (Eq. 5 with one-hot distributions) of sequence s: the longest prefix of the drafts that equals

@@ -45,7 +45,7 @@ struct pacer_ctx {
     struct StepGraph { cudaGraph_t graph; cudaGraphExec_t exec; int64_t launches; };   // exec == NULL: seen once, not captured yet
     std::map<int64_t, StepGraph> step_graphs;
     int use_graphs;
-    int32_t *fin_host;         // pinned: finished flags of the sequences, one row per step in flight
+    int32_t *fin_host;         // pinned: finished flags of the sequences, written by the acceptance
     cudaEvent_t fin_ev[8];
     std::vector<float2> rope_host[3];
     std::string err;
@@ -363,7 +363,8 @@ extern "C" int pacer_create(const pacer_cfg *cfg, void *dev_workspace, size_t wo
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&c->ev[i]);
     for (int i = 0; i < 8 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&c->fin_ev[i], cudaEventDisableTiming);
     c->fin_host = nullptr;
-    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->fin_host, sizeof(int32_t) * 8 * cfg->max_batch, cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->fin_host, sizeof(int32_t) * cfg->max_batch, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&c->d.fin_out, c->fin_host, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         std::string msg = std::string("pacer_create: ") + cudaGetErrorString(e);
@@ -575,6 +576,7 @@ static int start_run(pacer_ctx *c, const int32_t *prompt, int batch, int n_promp
     CK(cudaMemcpy2DAsync(c->d.x, sizeof(int32_t) * k.max_ctx, prompt, sizeof(int32_t) * n_prompt, sizeof(int32_t) * n_prompt,
                          batch, cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));        // hs is a local
+    for (int s = 0; s < k.max_batch; ++s) c->fin_host[s] = 0;        // (nothing of an earlier run is in flight)
     return PACER_OK;
 }
 
@@ -777,9 +779,9 @@ static int launch_step(pacer_ctx *c, int gamma_max) {
 }
 
 // Enqueues steps until every sequence is finished.  The end of generation is decided on the device; the host only
-// learns of it, without ever waiting for the step it has just enqueued: after each step the finished flags are
-// copied to pinned memory behind an event, and the host looks at the flags of the step it enqueued RUN_AHEAD steps
-// ago.  Steps enqueued after the last real one are no-ops on the device.
+// learns of it, without ever waiting for the step it has just enqueued: the acceptance sets a flag in pinned memory, and
+// the host looks at the flags behind the event of the step it enqueued RUN_AHEAD steps ago (a copy of the flags after
+// every step cost the stream about 8 us).  Steps enqueued after the last real one are no-ops on the device.
 template <class Enqueue>
 static int run_steps(pacer_ctx *c, int batch, int max_steps, Enqueue enqueue) {
     constexpr int RUN_AHEAD = 2, SLOTS = 8;
@@ -787,14 +789,12 @@ static int run_steps(pacer_ctx *c, int batch, int max_steps, Enqueue enqueue) {
         int rc = enqueue(step);
         if (rc) return rc;
         const int slot = step % SLOTS;
-        CK(cudaMemcpy2DAsync(c->fin_host + (size_t)slot * c->cfg.max_batch, sizeof(int32_t), &c->d.st[0].finished, sizeof(SeqState),
-                             sizeof(int32_t), batch, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaEventRecord(c->fin_ev[slot], c->stream));
         if (step >= RUN_AHEAD) {
             const int seen = (step - RUN_AHEAD) % SLOTS;
             CK(cudaEventSynchronize(c->fin_ev[seen]));
             bool all = true;
-            for (int q = 0; q < batch; ++q) all = all && c->fin_host[(size_t)seen * c->cfg.max_batch + q];
+            for (int q = 0; q < batch; ++q) all = all && ((volatile int32_t *)c->fin_host)[q];
             if (all) break;
         }
     }
