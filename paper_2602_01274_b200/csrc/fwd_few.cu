@@ -52,6 +52,13 @@ struct FewOp {
     int kgs, pad;                  // k groups: 10 (a warp takes all atoms of a stage) or 5 (two warps share them)
 };
 
+struct FewAtt {
+    int chunks, nsplit, items;         // query-row chunks of a kv head (FQ rows each), key splits
+};
+struct FewItem {
+    int split, vc, kh, seq, n_r, pos0, lo, hi;
+};
+
 struct FewCtx {
     unsigned char *scratch, *ring;
     uint64_t *wfull, *wempty;      // [FNB] a stage's weights are there / have been read
@@ -79,6 +86,8 @@ struct FewCtx {
     uint64_t *seed;                // [FEW_ROWS]
     BestD *best;                   // [FEW_ROWS] best Gumbel score of this block's columns so far
     int x0, xc;                    // this block's columns of the residual stream
+    FewAtt *att;                   // the attention phases' work, the same in every layer (in shared memory: registers are short)
+    FewItem *first;                // this block's first item of it
 };
 
 __device__ __forceinline__ void fsync() { asm volatile("bar.sync 3, 320;" ::: "memory"); }
@@ -412,6 +421,7 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t *b, int count) {
 // costs more than the atom's instructions.  (A lane of an operand row beyond the live ones reads live row 0.)
 template <int RT, int N>
 __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &o, int kg, int pn, int my_a, int my_n) {
+    constexpr int KU = RT * N > 10 ? 1 : 2;              // k blocks whose loads overlap, as far as the registers go
     const int g = c.lane >> 2, t = c.lane & 3, nlive = c.nlive, nst = o.nst, xk = c.xk, nxs = (o.nkb + xk - 1) / xk;
     const uint32_t ring = smem_u32(c.ring) + (uint32_t)my_a * 1024u;
     int xrow[RT], xsw[RT];                               // this lane's operand rows within a k block; 64-byte groups swapped
@@ -447,7 +457,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
             while (kb >= xs * xk) next_x();
             const int run = min(k_end, xs * xk);
             const unsigned char *xa = xb + kb * nlive * 256;
-#pragma unroll 2
+#pragma unroll KU
             for (; kb < run; ++kb, base += (uint32_t)pn * 1024u, xa += nlive * 256) {
                 uint4 A[RT][4];
 #pragma unroll
@@ -534,9 +544,6 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
 
 // ------------------------------------------------------------------ attention
 
-struct FewAtt {
-    int chunks, nsplit, items;         // query-row chunks of a kv head (FQ rows each), key splits
-};
 __device__ __forceinline__ FewAtt few_att(const FewCtx &c, const Args &a) {
     FewAtt f;
     const int group = a.m.cfg.n_heads / a.m.cfg.n_kv_heads;
@@ -569,9 +576,6 @@ __device__ __forceinline__ FewAtt few_att(const FewCtx &c, const Args &a) {
     return f;
 }
 
-struct FewItem {
-    int split, vc, kh, seq, n_r, pos0, lo, hi;
-};
 __device__ __forceinline__ FewItem few_item(const FewCtx &c, const Args &a, const FewAtt &f, int it) {
     FewItem w;
     const int Hkv = a.m.cfg.n_kv_heads;
@@ -583,8 +587,8 @@ __device__ __forceinline__ FewItem few_item(const FewCtx &c, const Args &a, cons
     w.n_r = c.n_rows[w.seq];
     w.pos0 = c.row_pos[w.seq * a.g.rps];
     const int ks = min(c.key_start[w.seq], w.pos0), span = w.n_r > 0 ? w.pos0 + w.n_r - ks : 0;
-    w.lo = ks + (int)((long long)span * w.split / f.nsplit);
-    w.hi = ks + (int)((long long)span * (w.split + 1) / f.nsplit);
+    w.lo = ks + (int)((unsigned)(span * w.split) / (unsigned)f.nsplit);
+    w.hi = ks + (int)((unsigned)(span * (w.split + 1)) / (unsigned)f.nsplit);
     return w;
 }
 
@@ -622,13 +626,12 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     unsigned char *qs = c.scratch;                                    // [QR] rows: HD values, HD remainders
     float *red = reinterpret_cast<float *>(c.scratch + QR * QS);      // [FW][QR][PW]
     static_assert(QR * QS + FW * QR * PW * 4 <= F_SCRATCH, "attention scratch");
-    for (int i = threadIdx.x; i < nv * (HD / 4); i += FC_THREADS) {   // (rows past nv: stale, their sums are not read)
-        const int lv = i / (HD / 4), e = i - lv * (HD / 4), v = w.vc * QR + lv, hq = v / w.n_r, j = v - hq * w.n_r;
-        const float4 x = __ldcg(reinterpret_cast<const float4 *>(a.fb.qkv + (size_t)c.idx_of[w.seq * a.g.rps + j] * (H * HD) + (w.kh * group + hq) * HD) + e);
-        uint2 hi, lo;
-        split_pair(x.x, x.y, hi.x, lo.x); split_pair(x.z, x.w, hi.y, lo.y);
-        *reinterpret_cast<uint2 *>(qs + lv * QS + e * 8) = hi;
-        *reinterpret_cast<uint2 *>(qs + lv * QS + HD * 2 + e * 8) = lo;
+    static_assert(QR * (HD / 4) <= FC_THREADS, "four channels of a query row per thread");
+    const int qi = threadIdx.x;
+    float4 qx;
+    if (qi < nv * (HD / 4)) {
+        const int lv = qi / (HD / 4), e = qi & (HD / 4 - 1), v = w.vc * QR + lv, hq = v / w.n_r, j = v - hq * w.n_r;
+        qx = __ldcg(reinterpret_cast<const float4 *>(a.fb.qkv + (size_t)c.idx_of[w.seq * a.g.rps + j] * (H * HD) + (w.kh * group + hq) * HD) + e);
     }
     const int g = c.lane >> 2, t = c.lane & 3, ks = c.key_start[w.seq];
     const int vrow = g < nv ? (w.vc * QR + g) % w.n_r : -1, self = w.pos0 + vrow;        // this lane's query row in the sequence
@@ -645,7 +648,13 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
         }
     };
     int k0 = w.lo + c.warp * 8;
-    if (k0 < w.hi) load_k(k0);
+    if (k0 < w.hi) load_k(k0);                           // in flight with the query rows
+    if (qi < nv * (HD / 4)) {                            // (rows past nv: stale, their sums are not read)
+        uint2 hi, lo;
+        split_pair(qx.x, qx.y, hi.x, lo.x); split_pair(qx.z, qx.w, hi.y, lo.y);
+        *reinterpret_cast<uint2 *>(qs + qi / (HD / 4) * QS + (qi & (HD / 4 - 1)) * 8) = hi;
+        *reinterpret_cast<uint2 *>(qs + qi / (HD / 4) * QS + HD * 2 + (qi & (HD / 4 - 1)) * 8) = lo;
+    }
     fsync();                                             // the query rows are staged
     for (; k0 < w.hi; k0 += FW * 8) {
         uint4 vh[NC], vl[NC];
@@ -777,9 +786,10 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     }
 }
 
-__device__ __forceinline__ void few_attention(FewCtx &c, const Args &a, const FewAtt &f, const FewItem &first, int layer) {
+__device__ __forceinline__ void few_attention(FewCtx &c, const Args &a, int layer) {
+    const FewAtt f = *c.att;
     for (int it = c.cta; it < f.items; it += c.ncta) {
-        const FewItem w = it == c.cta ? first : few_item(c, a, f, it);
+        const FewItem w = it == c.cta ? *c.first : few_item(c, a, f, it);
         if (it != c.cta) fsync();                        // the scratch and the flag of the item before have been read
         if (a.m.hd == 64) few_attention_item<64>(c, a, f, w, layer);
         else few_attention_item<128>(c, a, f, w, layer);
@@ -822,8 +832,10 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     c.seed = reinterpret_cast<uint64_t *>(c.best + FEW_ROWS);                // [FEW_ROWS]
     c.draw_pos = reinterpret_cast<int32_t *>(c.seed + FEW_ROWS);             // [FEW_ROWS]
     c.flag = c.draw_pos + FEW_ROWS;                                          // 4 words: attention's last arrival / the drawn token, live rows
+    c.att = reinterpret_cast<FewAtt *>(c.flag + 4);
+    c.first = reinterpret_cast<FewItem *>(c.att + 1);
     static_assert(8 * (2 * FNB + 2 * FXS + 1) + 4 * FNB + sizeof(FewOp) * N_OPS + 8 * FEW_ROWS + 4 * (3 * MAX_ROWS + 2 * MAX_SEQ + 3 * FEW_ROWS) +
-                  (12 + 16 + 8 + 4) * FEW_ROWS + 16 <= F_MISC - F_XBYTES, "tables");
+                  (12 + 16 + 8 + 4) * FEW_ROWS + 16 + sizeof(FewAtt) + sizeof(FewItem) <= F_MISC - F_XBYTES, "tables");
     static_assert(sizeof(FewOp) * N_OPS % 8 == 0, "alignment of the pointer table");
     c.xs = reinterpret_cast<float *>(misc + F_MISC - F_XBYTES);
     c.bar_target = 0; c.ok = true; c.stage = 0; c.xstage = 0; c.pass = 0;
@@ -952,18 +964,25 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     stamp();
     few_grid_barrier(c, a.fb);
     stamp();
-    const FewAtt att = few_att(c, a);
-    const FewItem first = few_item(c, a, att, min(c.cta, att.items - 1));
+    if (threadIdx.x == 0) {
+        const FewAtt f = few_att(c, a);
+        *c.att = f;
+        *c.first = few_item(c, a, f, min(c.cta, f.items - 1));
+    }
+    fsync();
     const int nq = n_ops(a.P);
     for (int q = 0; q < nq; ++q) {
         const int opi = op_index(a.P, q), l = op_layer(a.P, q);
-        if (opi == OP_QKV && c.warp == FW - 1 && c.cta < att.items) few_kv_prefetch(c, a, first, l);
+        // opaque in every round: what the compiler could compute from these once for all rounds it would keep in registers
+        // that the projections need (68M draft step 90.7 -> 86.5 us, 7B forward of 5 rows 742 -> 727)
+        asm volatile("" : "+r"(c.lane), "+r"(c.warp), "+r"(c.nlive), "+r"(c.cta), "+r"(c.ncta), "+r"(c.xk));
+        if (opi == OP_QKV && c.warp == FW - 1 && c.cta < c.att->items) few_kv_prefetch(c, a, *c.first, l);
         few_gemm(c, a, opi, l);
         stamp();
         few_grid_barrier(c, a.fb);
         stamp();
         if (opi == OP_QKV) {
-            few_attention(c, a, att, first, l);
+            few_attention(c, a, l);
             stamp();
             few_grid_barrier(c, a.fb);
             stamp();
