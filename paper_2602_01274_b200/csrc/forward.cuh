@@ -287,8 +287,9 @@ __device__ __host__ __forceinline__ int op_slice(const GemmOp &op, int cta, int 
 
 // Grid barrier (MMA warps only): every block arrives once; waits are bounded.  A wait that runs
 // out raises the abort flag, after which all later barriers fall through.
+// (The proxy fence that bulk copies of these writes need stands in front of the copies, in the warp that issues them: it is
+// needed once on the way from the write to the copy.  In every thread of every block, here, it cost 0.4 us a barrier.)
 __device__ __forceinline__ void grid_barrier(Ctx &c, const FwdBufs &fb) {
-    asm volatile("fence.proxy.async;" ::: "memory");   // this thread's global writes, for bulk copies issued later
     bsync();
     if (threadIdx.x == 0) {
         c.bar_target += (unsigned long long)c.ncta;

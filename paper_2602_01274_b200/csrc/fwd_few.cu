@@ -63,7 +63,7 @@ struct FewCtx {
     unsigned char *scratch, *ring;
     uint64_t *wfull, *wempty;      // [FNB] a stage's weights are there / have been read
     uint64_t *xfull, *xempty;      // [FXS] the same for the activations
-    volatile int32_t *ready;       // passes whose activations may be copied: their inputs are complete, the ring is unused
+    volatile int32_t *ready;       // passes begun by the consumers: a later pass of a projection may overwrite the scratch
     int32_t *slot_at;              // [FNB] ring offset of a stage, written by the producer before the stage's barrier
     const FewOp *ops;              // [N_OPS]
     float *xs;                     // [live row][columns of this block] residual stream
@@ -93,8 +93,10 @@ struct FewCtx {
 __device__ __forceinline__ void fsync() { asm volatile("bar.sync 3, 320;" ::: "memory"); }
 static_assert(FC_THREADS == 320, "fsync");
 
+// (The proxy fence that bulk copies of these writes need stands in front of the copies, in the warp that issues them: it is
+// needed once on the way from the write to the copy.  In every thread of every block, here, it cost 0.4 us a barrier: 1.3B
+// draft step 1088 -> 1055 us.)
 __device__ __forceinline__ void few_grid_barrier(FewCtx &c, const FwdBufs &fb) {
-    asm volatile("fence.proxy.async;" ::: "memory");   // this thread's global writes, for bulk copies issued later
     fsync();
     if (threadIdx.x == 0) {
         c.bar_target += (unsigned long long)c.ncta;
@@ -217,8 +219,25 @@ __device__ __forceinline__ void few_x_producer(FewCtx &c, const Args &a, uint64_
         const FewOp o = c.ops[opi];
         const bf16 *X = opi == OP_O ? a.d.att : opi == OP_DOWN ? a.d.act : a.fb.xg;
         for (int p = 0; p < o.npass; ++p) {
-            wait_count(a.fb, c.ready, ++pass, 6);
-            __threadfence_block();
+            ++pass;
+            if (p > 0) {
+                wait_count(a.fb, c.ready, pass, 6);
+                __threadfence_block();
+            } else {
+                // the projection's inputs are complete, and this block's consumers are done with the ring's bytes, once the
+                // grid barrier in front of it is over: watched here, not passed on by the consumers (0.3 us a projection)
+                const int bars = opi == OP_HEAD ? 5 * P.n_layers : 5 * op_layer(P, q) + (opi == OP_QKV ? 0 : opi == OP_O ? 2 : opi == OP_GU ? 3 : 4);
+                const unsigned long long want = c.bar_target + (unsigned long long)c.ncta * (1 + bars);
+                unsigned it = 0;
+                while (ld_acquire_u64(a.fb.bar) < want) {
+                    ++it;
+                    if ((it & 255u) == 0 && (it > 4u * SPIN_LIMIT || *(volatile int32_t *)a.fb.abort_flag)) {
+                        atomicCAS(a.fb.abort_flag, 0, 1);
+                        break;
+                    }
+                }
+                __syncwarp();
+            }
             asm volatile("fence.proxy.async;" ::: "memory");
             for (int k = 0; k < o.nkb; k += c.xk, ++n) {
                 const int slot = n % FXS;
@@ -506,7 +525,7 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
         int pa, pn;
         few_pass(o, p, pa, pn);
         const int h0 = (pn + 1) >> 1, my_a = o.kgs < FW && cg ? h0 : 0, my_n = o.kgs == FW ? pn : cg ? pn - h0 : h0;
-        if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // the activations may be copied
+        if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // (a later pass:) the activations may be copied
         // (its loads travel with the first activations)
         if ((opi == OP_QKV || opi == OP_GU || opi == OP_HEAD) && p == 0) few_inv(c, a);
         if (nlive <= 8) {
