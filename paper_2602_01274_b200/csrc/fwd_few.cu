@@ -761,11 +761,10 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     if (f.nsplit > 1) {
         fsync();
         if (threadIdx.x == 0) {
-            __threadfence();
-            const int n = atomicAdd(a.fb.att_cnt + unit, 1);
+            int n;                                       // releases this split's partial and acquires the others'
+            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(n) : "l"(a.fb.att_cnt + unit) : "memory");
             const bool last = n == f.nsplit - 1;
             if (last) a.fb.att_cnt[unit] = 0;            // for the next layer (all splits have arrived)
-            __threadfence();
             *c.flag = last;
         }
         fsync();
@@ -774,10 +773,10 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
                 const int lv = i / (HD / 2), ch = 2 * (i - lv * (HD / 2));
                 const float *pp = part + (size_t)lv * PW;
                 float M = -INFINITY, L = 0.f, v0 = 0.f, v1 = 0.f;
-                for (int s0 = 0; s0 < f.nsplit; s0 += 8) {             // eight splits' loads in flight
-                    float2 ml[8], vv[8];
+                for (int s0 = 0; s0 < f.nsplit; s0 += 16) {             // sixteen splits' loads in flight
+                    float2 ml[16], vv[16];
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
+                    for (int x = 0; x < 16; ++x) {
                         const bool in = s0 + x < f.nsplit;
                         const float *sp = pp + (size_t)(in ? s0 + x : 0) * QR * PW;
                         ml[x] = __ldcg(reinterpret_cast<const float2 *>(sp + HD));
@@ -785,7 +784,7 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
                     }
                     float Mn = M;
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
+                    for (int x = 0; x < 16; ++x) {
                         if (s0 + x >= f.nsplit) ml[x] = make_float2(-INFINITY, 0.f);
                         Mn = fmaxf(Mn, ml[x].x);
                     }
@@ -793,7 +792,7 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
                     L *= fo; v0 *= fo; v1 *= fo;
                     M = Mn;
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
+                    for (int x = 0; x < 16; ++x) {
                         const float fc = ml[x].x == -INFINITY ? 0.f : __expf(ml[x].x - M);
                         L += ml[x].y * fc; v0 += vv[x].x * fc; v1 += vv[x].y * fc;
                     }
