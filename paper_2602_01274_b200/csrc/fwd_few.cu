@@ -41,7 +41,8 @@ constexpr int F_PASS = 28;                      // 8-row weight atoms of a pass 
 constexpr int FXS = 3, F_XROWS = 52;            // activation stages, and 256-byte (row, k block) pieces of one
 constexpr int F_SCRATCH = 47 * 1024;            // activation ring; the sums of a pass and attention use the same bytes
 constexpr int F_MISC = 9 * 1024;
-constexpr int F_RING = (227 * 1024 - F_SCRATCH - F_MISC) / 1024 * 1024;
+constexpr int F_GUARD = 1024;                   // before the ring: the rows of an atom ahead of the first one are read, not used
+constexpr int F_RING = (227 * 1024 - F_SCRATCH - F_MISC - F_GUARD) / 1024 * 1024;
 static_assert(FNB == 32 && F_SCRATCH % 1024 == 0 && FXS * F_XROWS * 256 <= F_SCRATCH && F_RING >= 5 * F_PASS * 1024, "layout");
 constexpr int F_XBYTES = 5120;                  // of F_MISC: this block's columns of the residual stream
 // Weight rows [r0, r1) of a block in a projection: units of two rows (gate/up: 16, a gate atom and its up atom), as even
@@ -146,9 +147,12 @@ __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int 
     o.kgs = o.span <= 3 ? FW : FW / 2;
     const int atoms = min(nlive <= 8 ? F_PASS : 16, F_SCRATCH / (o.kgs * nlive * 32)) & ~1;
     o.npass = (o.span + atoms - 1) / atoms;
-    // stage: F_STAGE bytes of weights, but work for every k group
+    // stage: F_STAGE bytes of weights, but work for every k group.  Only the block's own rows count: a block's 10 to 14 rows
+    // of a d_model-wide projection touch two or three atoms, and with whole atoms in the ring the ten stages of a 1.3B
+    // down projection did not fit it (6.5 us, now 4.7)
     const int sp = o.npass ? (o.span + o.npass - 1) / o.npass : 1;
-    o.kbs = max(1, min(min(32, (F_STAGE / 1024) / sp), (o.nkb + o.kgs - 1) / o.kgs));
+    const int rows = max(1, o.npass == 1 ? o.r1 - o.r0 : sp * 8);
+    o.kbs = max(1, min(min(32, F_STAGE / (rows * 128)), (o.nkb + o.kgs - 1) / o.kgs));
     o.nst = (o.nkb + o.kbs - 1) / o.kbs;
     return o;
 }
@@ -185,9 +189,9 @@ __device__ __forceinline__ void few_weight_producer(FewCtx &c, const FwdBufs &fb
             const int ra = max(o.r0, (o.atom0 + pa) * 8), rb = min(o.r1, (o.atom0 + pa + pn) * 8);
             const uint32_t kbytes = (uint32_t)(rb - ra) * 128u;
             const bf16 *src = wl + ((size_t)c.lane * (2 * op.MT) + o.atom0 + pa) * 512 + (ra & 7) * 64;
-            unsigned char *dst = c.ring + c.lane * pn * 1024 + (ra & 7) * 128;
+            unsigned char *dst = c.ring + c.lane * kbytes;
             for (int k = 0; k < o.nkb; k += o.kbs, ++n) {
-                const int nk = min(o.kbs, o.nkb - k), bytes = nk * pn * 1024;
+                const int nk = min(o.kbs, o.nkb - k), bytes = nk * (int)kbytes;
                 if (at + bytes > F_RING) { head += F_RING - at; at = 0; }
                 while (tail < n && (tail <= n - FNB || head + bytes > tail_v + F_RING)) {
                     if (!wait_bar(fb, c.wempty + (tail & (FNB - 1)), ((uint32_t)(tail / FNB)) & 1u, 5, tail)) { alive = false; break; }
@@ -435,14 +439,17 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t *b, int count) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
 }
 
-// One warp's share of a pass: the weight stages kg, kg + kgs, ... and N atoms of them from atom my_a on (my_n of them
+// One warp's share of a pass (weight rows ra .. ra + rows): the weight stages kg, kg + kgs, ... and N atoms of them from atom my_a on (my_n of them
 // its own, the rest is computed and not stored), into the sum buffer.  N is a template parameter because a branch per atom
 // costs more than the atom's instructions.  (A lane of an operand row beyond the live ones reads live row 0.)
 template <int RT, int N>
-__device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &o, int kg, int pn, int my_a, int my_n) {
+__device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &o, int kg, int pn, int ra, int rows, int my_a,
+                                         int my_n) {
     constexpr int KU = RT * N > 10 ? 1 : 2;              // k blocks whose loads overlap, as far as the registers go
     const int g = c.lane >> 2, t = c.lane & 3, nlive = c.nlive, nst = o.nst, xk = c.xk, nxs = (o.nkb + xk - 1) / xk;
-    const uint32_t ring = smem_u32(c.ring) + (uint32_t)my_a * 1024u;
+    // where atom my_a of a stage's first k block would begin: the ring holds the rows from ra on, a k block behind the other
+    // (the swizzle goes by the row's place in its atom, not by its address); other rows of an atom are whatever lies there
+    const uint32_t ring = smem_u32(c.ring) + (uint32_t)my_a * 1024u - (uint32_t)(ra & 7) * 128u, kbytes = (uint32_t)rows * 128u;
     int xrow[RT], xsw[RT];                               // this lane's operand rows within a k block; 64-byte groups swapped
 #pragma unroll
     for (int m = 0; m < RT; ++m) {
@@ -477,7 +484,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
             const int run = min(k_end, xs * xk);
             const unsigned char *xa = xb + kb * nlive * 256;
 #pragma unroll KU
-            for (; kb < run; ++kb, base += (uint32_t)pn * 1024u, xa += nlive * 256) {
+            for (; kb < run; ++kb, base += kbytes, xa += nlive * 256) {
                 uint4 A[RT][4];
 #pragma unroll
                 for (int m = 0; m < RT; ++m)
@@ -524,30 +531,31 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
     for (int p = 0; p < o.npass; ++p) {
         int pa, pn;
         few_pass(o, p, pa, pn);
+        const int ra = max(o.r0, (o.atom0 + pa) * 8), rb = min(o.r1, (o.atom0 + pa + pn) * 8);
         const int h0 = (pn + 1) >> 1, my_a = o.kgs < FW && cg ? h0 : 0, my_n = o.kgs == FW ? pn : cg ? pn - h0 : h0;
         if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // (a later pass:) the activations may be copied
         // (its loads travel with the first activations)
         if ((opi == OP_QKV || opi == OP_GU || opi == OP_HEAD) && p == 0) few_inv(c, a);
         if (nlive <= 8) {
-            if (my_n <= 1) few_main<1, 1>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 2) few_main<1, 2>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 3) few_main<1, 3>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 4) few_main<1, 4>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 6) few_main<1, 6>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 8) few_main<1, 8>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 10) few_main<1, 10>(c, a, o, kg, pn, my_a, my_n);
-            else few_main<1, 14>(c, a, o, kg, pn, my_a, my_n);
+            if (my_n <= 1) few_main<1, 1>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 2) few_main<1, 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 3) few_main<1, 3>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 4) few_main<1, 4>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 6) few_main<1, 6>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 8) few_main<1, 8>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 10) few_main<1, 10>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else few_main<1, 14>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
         } else {
-            if (my_n <= 1) few_main<2, 1>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 2) few_main<2, 2>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 3) few_main<2, 3>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 4) few_main<2, 4>(c, a, o, kg, pn, my_a, my_n);
-            else if (my_n <= 6) few_main<2, 6>(c, a, o, kg, pn, my_a, my_n);
-            else few_main<2, 8>(c, a, o, kg, pn, my_a, my_n);
+            if (my_n <= 1) few_main<2, 1>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 2) few_main<2, 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 3) few_main<2, 3>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 4) few_main<2, 4>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 6) few_main<2, 6>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else few_main<2, 8>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
         }
         c.stage += o.nst; c.xstage += nxs;
         fsync();
-        const int PC = pn * 8, ra = max(o.r0, (o.atom0 + pa) * 8), rb = min(o.r1, (o.atom0 + pa + pn) * 8), off = (o.atom0 + pa) * 8;
+        const int PC = pn * 8, off = (o.atom0 + pa) * 8;
         for (int i = c.warp; i < nlive; i += FW)
             few_epilogue(c, a, opi, layer, i, ra, rb, off, red + i * PC, nlive * PC, o.kgs, p == o.npass - 1);
         if (p + 1 < o.npass) fsync();
@@ -824,10 +832,10 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     }
     FewCtx c;
     c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31; c.cta = blockIdx.x; c.ncta = gridDim.x;
-    c.ring = smem;
-    c.scratch = smem + F_RING;
+    c.ring = smem + F_GUARD;
+    c.scratch = c.ring + F_RING;
     static_assert(F_RING % 1024 == 0, "ring");
-    unsigned char *misc = smem + F_RING + F_SCRATCH;
+    unsigned char *misc = c.scratch + F_SCRATCH;
     c.wfull = reinterpret_cast<uint64_t *>(misc);
     c.wempty = c.wfull + FNB;
     c.xfull = c.wempty + FNB;
@@ -1052,7 +1060,7 @@ bool few_rows_ok(const ModelDev &m, const Geom &g, int kind, int ncta) {
 
 cudaError_t launch_few(const Args &a, int which, int ncta, cudaStream_t st) {
     static bool attr_set[64] = {};           // the opt-in is per device
-    constexpr int smem = F_RING + F_SCRATCH + F_MISC;
+    constexpr int smem = F_GUARD + F_RING + F_SCRATCH + F_MISC;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
