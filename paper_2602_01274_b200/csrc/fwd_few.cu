@@ -636,12 +636,15 @@ __device__ __forceinline__ uint32_t movmatrix(uint32_t v) {         // transpose
 }
 
 // One item: FQ query rows (head within the group x row of the sequence) of a kv head over the keys [lo, hi), eight keys
-// per warp and step on mma.sync.  The 16-row operand holds the 8 rows' values over their remainders, for q and for the
-// probabilities; a lane (g, t) reads 8 consecutive channels of key g, of k as the k slots {2t, 2t+1, 2t+8, 2t+9} of two
-// MMAs (q is read by the same rule), of v as four 8 x 8 blocks that movmatrix turns into the other operand: its k slots
-// are the 8 keys' values, then their remainders, and its columns channels 8t + 2i of each 32.  Nothing is staged in
-// shared memory but q.  Bound by the latency of its K and V reads (8 KB per warp in flight); on the ordinary ALUs in fp32
-// a step of eight rows took 4 us, four times as long.
+// per warp and step on mma.sync.  A lane (g, t) reads 8 consecutive channels of key g.  Scores: the 16-row operand holds the
+// 8 query rows' values over their remainders, the keys are the columns, and the lane's channels are the k slots {2t, 2t+1,
+// 2t+8, 2t+9} of two MMAs (q is read by the same rule).  Values: transposed, 16 channels x 8 query rows, so that the
+// accumulators take half the registers (with the query rows over their remainders as rows, 64 a lane at head dimension
+// 128); movmatrix turns the lane's four 8 x 8 blocks of v into the row operand (rows: channels 8 (g / 2) + 2i + g % 2 of
+// each 32; k slots: the 8 keys' values, then their remainders), the probabilities and then their remainders are the
+// columns.  Nothing is staged in shared memory but q.  Bound by the latency of its K and V reads (8 KB per warp in
+// flight): 12.6 us for 16 heads over 2048 keys (14.8 before the transposition); on the ordinary ALUs in fp32 a step of
+// eight rows took 4 us, four times as long.
 template <int HD>
 __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, const FewAtt &f, const FewItem &w, int layer) {
     constexpr int NC = HD / 32, PW = HD + 2, QS = HD * 4 + 64, QR = FQ;
@@ -662,12 +665,13 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     }
     const int g = c.lane >> 2, t = c.lane & 3, ks = c.key_start[w.seq];
     const int vrow = g < nv ? (w.vc * QR + g) % w.n_r : -1, self = w.pos0 + vrow;        // this lane's query row in the sequence
-    float mx = -INFINITY, ls = 0.f, o[NC * 4][4];
+    float mx = -INFINITY, ls = 0.f, o[NC * 2][4];
 #pragma unroll
-    for (int e = 0; e < NC * 4; ++e) o[e][0] = o[e][1] = o[e][2] = o[e][3] = 0.f;
-    uint4 kh[NC], kl[NC];
+    for (int e = 0; e < NC * 2; ++e) o[e][0] = o[e][1] = o[e][2] = o[e][3] = 0.f;
+    uint4 kh[NC], kl[NC], vh[NC], vl[NC];
+    // (no condition around the loads, only around the row: it would keep a second set of the registers)
     auto load_k = [&](int k0) {
-        const bf16 *kp = m.kcache + cbase + (size_t)min(k0 + g, w.hi - 1) * HD + t * 8;
+        const bf16 *kp = m.kcache + cbase + (size_t)max(min(k0 + g, w.hi - 1), 0) * HD + t * 8;
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
             kh[n] = __ldcg(reinterpret_cast<const uint4 *>(kp + n * 32));
@@ -675,7 +679,15 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
         }
     };
     int k0 = w.lo + c.warp * 8;
-    if (k0 < w.hi) load_k(k0);                           // in flight with the query rows
+    auto load_v = [&](int k0) {
+        const bf16 *vp = m.vcache + cbase + (size_t)max(min(k0 + g, w.hi - 1), 0) * HD + t * 8;
+#pragma unroll
+        for (int n = 0; n < NC; ++n) {
+            vh[n] = __ldcg(reinterpret_cast<const uint4 *>(vp + n * 32));
+            vl[n] = __ldcg(reinterpret_cast<const uint4 *>(vp + m.kv_lo + n * 32));
+        }
+    };
+    load_k(k0);           // in flight with the query rows
     if (qi < nv * (HD / 4)) {                            // (rows past nv: stale, their sums are not read)
         uint2 hi, lo;
         split_pair(qx.x, qx.y, hi.x, lo.x); split_pair(qx.z, qx.w, hi.y, lo.y);
@@ -684,15 +696,7 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     }
     fsync();                                             // the query rows are staged
     for (; k0 < w.hi; k0 += FW * 8) {
-        uint4 vh[NC], vl[NC];
-        {
-            const bf16 *vp = m.vcache + cbase + (size_t)min(k0 + g, w.hi - 1) * HD + t * 8;
-#pragma unroll
-            for (int n = 0; n < NC; ++n) {
-                vh[n] = __ldcg(reinterpret_cast<const uint4 *>(vp + n * 32));
-                vl[n] = __ldcg(reinterpret_cast<const uint4 *>(vp + m.kv_lo + n * 32));
-            }
-        }
+        load_v(k0);
         float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
@@ -703,7 +707,7 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
             mma16816(sa, qh.x, ql.x, qh.y, ql.y, kl[n].x, kl[n].y);
             mma16816(sb, qh.z, ql.z, qh.w, ql.w, kl[n].z, kl[n].w);
         }
-        if (k0 + FW * 8 < w.hi) load_k(k0 + FW * 8);
+        load_k(k0 + FW * 8);
         // scores of row g, keys 2t, 2t + 1: a row sees the keys of its context up to its own position; a row before a
         // restricted context sees itself
         float s0 = (sa[0] + sb[0]) + (sa[2] + sb[2]), s1 = (sa[1] + sb[1]) + (sa[3] + sb[3]);
@@ -720,26 +724,30 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
         ls = ls * corr + p0 + p1;
         uint32_t ph, pl;
         split_pair(p0, p1, ph, pl);
+        const float c0 = __shfl_sync(0xffffffffu, corr, 8 * t), c1 = __shfl_sync(0xffffffffu, corr, 8 * t + 4);
 #pragma unroll
-        for (int e = 0; e < NC * 4; ++e) { o[e][0] *= corr; o[e][1] *= corr; o[e][2] *= corr; o[e][3] *= corr; }
+        for (int e = 0; e < NC * 2; ++e) { o[e][0] *= c0; o[e][1] *= c1; o[e][2] *= c0; o[e][3] *= c1; }
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
-            mma16816(o[n * 4 + 0], ph, pl, ph, pl, movmatrix(vh[n].x), movmatrix(vl[n].x));
-            mma16816(o[n * 4 + 1], ph, pl, ph, pl, movmatrix(vh[n].y), movmatrix(vl[n].y));
-            mma16816(o[n * 4 + 2], ph, pl, ph, pl, movmatrix(vh[n].z), movmatrix(vl[n].z));
-            mma16816(o[n * 4 + 3], ph, pl, ph, pl, movmatrix(vh[n].w), movmatrix(vl[n].w));
+            uint32_t a0 = movmatrix(vh[n].x), a1 = movmatrix(vh[n].y), a2 = movmatrix(vl[n].x), a3 = movmatrix(vl[n].y);
+            mma16816(o[n * 2], a0, a1, a2, a3, ph, ph);
+            mma16816(o[n * 2], a0, a1, a2, a3, pl, pl);
+            a0 = movmatrix(vh[n].z); a1 = movmatrix(vh[n].w); a2 = movmatrix(vl[n].z); a3 = movmatrix(vl[n].w);
+            mma16816(o[n * 2 + 1], a0, a1, a2, a3, ph, ph);
+            mma16816(o[n * 2 + 1], a0, a1, a2, a3, pl, pl);
         }
     }
     ls += __shfl_xor_sync(0xffffffffu, ls, 1);
     ls += __shfl_xor_sync(0xffffffffu, ls, 2);
     {
-        float *my = red + (c.warp * QR + g) * PW;
+        // rows 2t, 2t + 1; channel of block i, column g: 8 (g / 2) + 2 i + g % 2
+        float *my = red + (c.warp * QR + 2 * t) * PW + 8 * (g >> 1) + (g & 1);
 #pragma unroll
-        for (int n = 0; n < NC; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                *reinterpret_cast<float2 *>(my + n * 32 + 8 * t + 2 * i) = make_float2(o[n * 4 + i][0] + o[n * 4 + i][2], o[n * 4 + i][1] + o[n * 4 + i][3]);
-        if (t == 0) { my[HD] = mx; my[HD + 1] = ls; }
+        for (int e = 0; e < NC * 2; ++e) {
+            float *p = my + (e >> 1) * 32 + (e & 1) * 4;
+            p[0] = o[e][0]; p[PW] = o[e][1]; p[2] = o[e][2]; p[PW + 2] = o[e][3];
+        }
+        if (t == 0) { float *st = red + (c.warp * QR + g) * PW + HD; st[0] = mx; st[1] = ls; }
     }
     fsync();
     // the warps' shares -> the item's, two channels per thread
