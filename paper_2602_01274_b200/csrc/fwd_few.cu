@@ -830,6 +830,39 @@ __device__ __forceinline__ void few_attention(FewCtx &c, const Args &a, int laye
     }
 }
 
+// End of one draft forward (Eq. 6), as tail_draft: the rows' 1/rms is the LM head's, and all warps copy the hidden rows while
+// warp 0 still looks for the best logit (the arg-max, 1/rms, copy and state one after the other: 4.5 us of a 68M draft step
+// and 9.5 of a 1.3B one; now 3.3 and 4.5).
+__device__ __forceinline__ void few_tail_draft_rows(const FewCtx &c, const Args &a, int s) {
+    const DevPtrs &d = a.d;
+    const int n_in = c.n_rows[s], half = a.m.cfg.d_model >> 1;
+    if (d.st[s].sched) return;                           // with prescribed windows nothing is pre-verified
+    float2 *dst = reinterpret_cast<float2 *>(d.hpend + ((size_t)s * (d.block_b + 1) + d.st[s].n_pend) * (2 * half));
+    for (int j = 0; j < n_in; ++j) {
+        const int r = s * a.g.rps + j;
+        const float inv = c.inv[c.idx_of[r]];
+        const float2 *x = reinterpret_cast<const float2 *>(d.xres + (size_t)r * (2 * half));
+#pragma unroll 4
+        for (int i = threadIdx.x; i < half; i += FC_THREADS) {
+            const float2 v = __ldcg(x + i), gn = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162 *>(a.m.normf)[i]);
+            dst[(size_t)j * half + i] = make_float2(v.x * inv * gn.x, v.y * inv * gn.y);
+        }
+    }
+}
+__device__ __forceinline__ void few_tail_draft(const FewCtx &c, const Args &a, int s, int pick) {      // one thread
+    const DevPtrs &d = a.d;
+    SeqState &st = d.st[s];
+    const int n_in = c.n_rows[s], gamma = st.gamma, n_pend = st.n_pend;
+    if (!st.sched) {
+        for (int j = 0; j < n_in; ++j) d.hpend_e[s * (d.block_b + 1) + n_pend + j] = j == n_in - 1 ? gamma + 1 : 0;
+        st.n_pend = n_pend + n_in;
+    }
+    d.y[(size_t)s * d.gamma_cap + gamma] = pick;
+    st.gamma = gamma + 1;
+    st.len_D += n_in;
+    st.n_draft_fwd += 1;
+}
+
 // ------------------------------------------------------------------ the kernel
 
 __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ Args a, const int which) {
@@ -1032,7 +1065,10 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
                 tp = top2_merge(tp, Top2{v.x, __float_as_int(v.y), v.z});
             }
             tp = few_warp_top2(tp);
-            if (c.lane == 0) { d.row_arg[r] = tp.i1; d.row_margin[r] = tp.v1 - tp.v2; }
+            if (c.lane == 0) {
+                d.row_arg[r] = tp.i1; d.row_margin[r] = tp.v1 - tp.v2;
+                if (kind == KIND_DRAFT && c.draw_pos[i] < 0) c.flag[0] = tp.i1;
+            }
             if (c.draw_pos[i] >= 0) {           // (one row of the sequence at most)
                 BestD bd{-INFINITY, 0x7fffffff};
                 for (int b = c.lane; b < c.ncta; b += 32) {
@@ -1043,17 +1079,18 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
                 if (c.lane == 0) c.flag[0] = bd.i;
             }
         }
+        if (kind == KIND_DRAFT) few_tail_draft_rows(c, a, c.cta);
         fsync();
+        if (kind == KIND_DRAFT && c.n_rows[c.cta] > 0 && threadIdx.x == 0) few_tail_draft(c, a, c.cta, c.flag[0]);
         if (kind == KIND_VERIFY && a.aux && threadIdx.x == 0) accept_greedy_seq(d, g, c.cta);
     }
-    if (c.cta < g.batch && kind != KIND_VERIFY && c.warp < MMA_WARPS) {
+    if (c.cta < g.batch && (kind == KIND_MB || kind == KIND_AR) && c.warp < MMA_WARPS) {
         Ctx t;                                  // what the tails look at
         t.warp = c.warp; t.lane = c.lane; t.cta = c.cta; t.ncta = c.ncta;
         t.scratch = c.scratch; t.n_rows = c.n_rows; t.row_tok = c.row_tok; t.row_pos = c.row_pos;
         t.inv_rms = reinterpret_cast<float *>(c.scratch) + 1024;             // [MAX_ROWS], beside what the tails use
-        if (kind == KIND_DRAFT) { tail_inv_rms(t, a, t.cta); tail_draft(t, a, t.cta, c.flag[0]); }
-        else if (kind == KIND_MB) tail_mb(t, a, t.cta);
-        else if (kind == KIND_AR) tail_ar(t, a, t.cta, c.flag[0]);
+        if (kind == KIND_MB) tail_mb(t, a, t.cta);
+        else tail_ar(t, a, t.cta, c.flag[0]);
     }
     stamp();
 }
