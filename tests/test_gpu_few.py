@@ -78,3 +78,9 @@ def test_batched_autoregressive_rows(batch):
         if margin > 2 * TOL:
             np.testing.assert_array_equal(tok[s], out, err_msg=str(s))
     ctx.close()
+
+
+@pytest.mark.parametrize("n_prompt", [1279, 2600])
+def test_many_key_splits(n_prompt):
+    """One kv head, so that its keys are cut into 17 and 33 splits: they are merged sixteen at a time."""
+    test_verify_rows("narrow", 4, n_prompt)
