@@ -528,14 +528,14 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
     const FewOp o = c.ops[opi];
     const int kg = o.kgs == FW ? c.warp : c.warp >> 1, cg = c.warp & 1, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
     float *red = reinterpret_cast<float *>(c.scratch);
+    // (its loads travel with the first activations; also in a block without rows: it may end a sequence's draft step)
+    if (opi == OP_QKV || opi == OP_GU || opi == OP_HEAD) few_inv(c, a);
     for (int p = 0; p < o.npass; ++p) {
         int pa, pn;
         few_pass(o, p, pa, pn);
         const int ra = max(o.r0, (o.atom0 + pa) * 8), rb = min(o.r1, (o.atom0 + pa + pn) * 8);
         const int h0 = (pn + 1) >> 1, my_a = o.kgs < FW && cg ? h0 : 0, my_n = o.kgs == FW ? pn : cg ? pn - h0 : h0;
         if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // (a later pass:) the activations may be copied
-        // (its loads travel with the first activations)
-        if ((opi == OP_QKV || opi == OP_GU || opi == OP_HEAD) && p == 0) few_inv(c, a);
         if (nlive <= 8) {
             if (my_n <= 1) few_main<1, 1>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
             else if (my_n <= 2) few_main<1, 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);

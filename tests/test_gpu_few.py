@@ -84,3 +84,38 @@ def test_batched_autoregressive_rows(batch):
 def test_many_key_splits(n_prompt):
     """One kv head, so that its keys are cut into 17 and 33 splits: they are merged sixteen at a time."""
     test_verify_rows("narrow", 4, n_prompt)
+
+
+@pytest.mark.parametrize("vocab,batch,d_ffn", [(4, 3, 64), (16, 9, 2432), (16, 16, 64), (30, 16, 2432)])
+def test_small_vocabulary_hidden_rows(vocab, batch, d_ffn):
+    """Fewer LM-head rows than twice the sequences: the block that ends a sequence's draft step has none of them, without or
+    with rows of the gate/up projection.  The hidden rows queued for the pre-verification model and its scores against the
+    oracle's (an entry of a normalised row is a few units and passes about ten roundings to 16 mantissa bits, 2^-17 each:
+    1e-4 per unit, 1e-3 is three times that for the largest)."""
+    from paper_2602_01274_b200 import binding as b
+    T, D = synth.ModelShape(1, 64, 1, 1, 64, vocab), synth.ModelShape(2, 64, 1, 1, d_ffn, vocab)
+    cfg = synth.PairConfig("few", T, D, agree=0.8, n_prompt=7, max_new=8, gamma_max=4, batch=batch)
+    gpu = synth.make_pair(cfg, seed=3, device="cuda:0", std=0.1)
+    cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
+    To, Do, Bo = oracle_models(cfg, cpu)
+    ctx = b.Context(b.make_cfg(T, D, batch, 32, 4, 4, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, gpu)
+    prompts = synth.make_prompts(vocab, batch, cfg.n_prompt, seed=3).numpy()
+    ctx.pacer_prefill(prompts, cfg.max_new, 4, -1.0)
+    for _ in range(4):
+        ctx.pacer_draft_step()
+    y = ctx.pacer_read_buffer(b.BUF_DRAFTS, np.int32, batch * 4).reshape(batch, 4)
+    h = ctx.pacer_read_buffer(b.BUF_HPEND, np.float32, batch * 5 * D.d_model).reshape(batch, 5, D.d_model)
+    ctx.pacer_preverify()
+    al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, batch * 4).reshape(batch, 4)
+    for s in range(batch):
+        o = orc.Pacer(To, Do, Bo, 32, b=4, gamma_cap=4, t0=-1.0, rho=cfg.rho)
+        o.prefill(prompts[s])
+        o.draft_block()
+        want = o.hpend()
+        o.preverify()
+        assert o.stats()["min_margin_draft"] > 1.0, s
+        np.testing.assert_array_equal(y[s], o.y(), err_msg=str(s))
+        assert np.abs(h[s, :4] - want).max() < 1e-3, s
+        assert np.abs(al[s] - o.alpha()).max() < 1e-3, s
+    ctx.close()
