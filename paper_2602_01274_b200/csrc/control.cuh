@@ -9,6 +9,10 @@ struct Top2 {
     float v1; int i1; float v2;
 };
 
+// One logit as a candidate.  A NaN ranks lowest, as -inf: a NaN would lose to the empty candidate (column 0x7fffffff) of a lane
+// or block without columns, and the next forward would look that column up as a token.
+__device__ __forceinline__ Top2 top2_one(float v, int i) { return Top2{fmaxf(v, -INFINITY), i, -INFINITY}; }
+
 __device__ __forceinline__ Top2 top2_merge(Top2 a, Top2 b) {
     // larger value wins; equal values keep the lower index
     Top2 r;

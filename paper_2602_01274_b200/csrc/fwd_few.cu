@@ -383,13 +383,13 @@ __device__ __forceinline__ void few_epilogue(FewCtx &c, const Args &a, int opi, 
                 const float v = s.x * inv + (n == b ? d.succ_bias : 0.f);
                 dst[n] = v;
                 draw(n, v);
-                tp = top2_merge(tp, Top2{v, n, -INFINITY});
+                tp = top2_merge(tp, top2_one(v, n));
             }
             if (n + 1 < V) {
                 const float v = s.y * inv + (n + 1 == b ? d.succ_bias : 0.f);
                 dst[n + 1] = v;
                 draw(n + 1, v);
-                tp = top2_merge(tp, Top2{v, n + 1, -INFINITY});
+                tp = top2_merge(tp, top2_one(v, n + 1));
             }
         }
         tp = few_warp_top2(tp);
@@ -1076,7 +1076,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
                     bd = best_merge(bd, BestD{__ldcg(&p->v), __ldcg(&p->i)});
                 }
                 bd = few_warp_best(bd);
-                if (c.lane == 0) c.flag[0] = bd.i;
+                if (c.lane == 0) c.flag[0] = drawn_token(bd);
             }
         }
         if (kind == KIND_DRAFT) few_tail_draft_rows(c, a, c.cta);

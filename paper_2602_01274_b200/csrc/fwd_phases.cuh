@@ -284,12 +284,12 @@ __device__ __forceinline__ void epi_head(Ctx &c, const Args &a, float *const *ro
                 if (n0 < V) {
                     const float v = acc[nt][i] * inv + (n0 == b ? a.d.succ_bias : 0.f);
                     dst[n0] = v;
-                    tp.v1 = v; tp.i1 = n0;
+                    tp = top2_one(v, n0);
                 }
                 if (n1 < V) {
                     const float v = acc[nt][2 + i] * inv + (n1 == b ? a.d.succ_bias : 0.f);
                     dst[n1] = v;
-                    tp = top2_merge(tp, Top2{v, n1, -INFINITY});
+                    tp = top2_merge(tp, top2_one(v, n1));
                 }
             }
 #pragma unroll

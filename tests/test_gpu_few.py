@@ -119,3 +119,45 @@ def test_small_vocabulary_hidden_rows(vocab, batch, d_ffn):
         assert np.abs(h[s, :4] - want).max() < 1e-3, s
         assert np.abs(al[s] - o.alpha()).max() < 1e-3, s
     ctx.close()
+
+
+@pytest.mark.parametrize("vocab,batch", [(5000, 1), (5000, 3), (1001, 16), (1001, 17), (30, 2)])
+@pytest.mark.parametrize("mode", ["greedy", "sample"])
+def test_rows_without_a_largest_logit(vocab, batch, mode):
+    """Logits that are all NaN (a NaN gain of the final norm): the tokens stay inside the vocabulary (they are looked up by the
+    next forward), and the loop ends.  Vocabularies at which lanes, blocks or threads have no column of a row, in the few-row
+    kernel and, from 17 sequences on, in the other one."""
+    from paper_2602_01274_b200 import binding as b
+    shape = synth.ModelShape(1, 64, 1, 1, 64, vocab)
+    cfg = synth.PairConfig("few", shape, shape, agree=0.8, n_prompt=5, max_new=6, gamma_max=4, batch=batch)
+    pair = synth.make_pair(cfg, seed=3, device="cuda:0")
+    for which in ("target", "draft"):
+        pair[which]["normf"][3] = float("nan")
+    ctx = b.Context(b.make_cfg(shape, shape, batch, 24, 4, 4, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, pair)
+    prompts = synth.make_prompts(vocab, batch, cfg.n_prompt, seed=3).numpy()
+    m = b.PACER_SAMPLE if mode == "sample" else b.PACER_GREEDY
+    tok, *_ = ctx.pacer_generate(prompts, cfg.max_new, 4, 0.5, m, 7)
+    np.testing.assert_array_equal(tok, 0)
+    tok, _ = ctx.pacer_generate_ar(prompts, cfg.max_new, m, 7)
+    np.testing.assert_array_equal(tok, 0)
+    ctx.close()
+
+
+def test_nan_logit_is_never_the_largest():
+    """One column of the LM head is NaN: the other columns decide, as in the oracle (which compares with `>`)."""
+    from paper_2602_01274_b200 import binding as b
+    T, D = SHAPES["narrow"]
+    cfg = synth.PairConfig("few", T, D, agree=0.8, n_prompt=21, max_new=8, gamma_max=4)
+    gpu = synth.make_pair(cfg, seed=4, device="cuda:0")
+    gpu["target"]["head"][777, 5] = float("nan")
+    cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
+    To, _, _ = oracle_models(cfg, cpu)
+    prompt = synth.make_prompts(T.vocab, 1, cfg.n_prompt, seed=5).numpy()
+    out, margin = orc.generate_ar(To, prompt[0], cfg.max_new)
+    assert margin > 2 * TOL
+    ctx = b.Context(b.make_cfg(T, D, 1, 40, 4, 4, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, gpu)
+    tok, _ = ctx.pacer_generate_ar(prompt, cfg.max_new)
+    np.testing.assert_array_equal(tok[0], out)
+    ctx.close()
