@@ -132,15 +132,16 @@ static __global__ void __launch_bounds__(LSE_THREADS) k_lse_parts(DevPtrs d, Acc
     for (int v = v0 + threadIdx.x; v < v1; v += LSE_THREADS) m = fmaxf(m, __ldcg(x + v));
     m = block_max_f(m, smd);
     double e = 0.0;
-    for (int v = v0 + threadIdx.x; v < v1; v += LSE_THREADS) e += exp((double)__ldcg(x + v) - (double)m);
+    const double base = m == -INFINITY ? 0.0 : (double)m;      // (a piece of -inf only: a sum of 0, as in the whole row's sum)
+    for (int v = v0 + threadIdx.x; v < v1; v += LSE_THREADS) e += exp((double)__ldcg(x + v) - base);
     e = block_sum_d(e, smd);
     if (threadIdx.x == 0) ab.lse[((size_t)s * (2 * gc + 1) + row) * LSE_PARTS + part] = make_double2((double)m, e);
 }
-__device__ __forceinline__ double row_lse(const double2 *p) {          // (a piece of an empty vocabulary range: -inf, 0)
+__device__ __forceinline__ double row_lse(const double2 *p) {          // (an empty piece: -inf, 0; a NaN logit: its piece's sum)
     double M = -INFINITY, e = 0.0;
     for (int i = 0; i < LSE_PARTS; ++i) M = fmax(M, __ldcg(&p[i].x));
     for (int i = 0; i < LSE_PARTS; ++i)
-        if (__ldcg(&p[i].y) > 0.0) e += __ldcg(&p[i].y) * exp(__ldcg(&p[i].x) - M);
+        if (__ldcg(&p[i].y) != 0.0) e += __ldcg(&p[i].y) * exp(__ldcg(&p[i].x) - M);
     return M + log(e);
 }
 

@@ -127,3 +127,24 @@ def test_sampled_speculative_output_follows_the_target_distribution():
             chi += (o_ - e) ** 2 / e
             dof += 1
     assert chi < stats.chi2.ppf(1 - 1e-5, dof), (chi, dof)
+
+
+@pytest.mark.parametrize("column", [0, 1500, 2047])
+def test_nan_logit_keeps_the_drafts(column):
+    """One target logit is NaN: the row's log-sum-exp is NaN, no draft compares as rejected, and none is, whichever piece of the
+    vocabulary the column is in (the oracle compares the same way)."""
+    from paper_2602_01274_b200 import binding as b
+    shape = synth.ModelShape(1, 64, 1, 1, 64, 2048)
+    cfg = synth.PairConfig("nan", shape, shape, agree=0.3, n_prompt=9, max_new=16, gamma_max=4)
+    pair = synth.make_pair(cfg, seed=5, device="cuda:0")
+    max_ctx = cfg.n_prompt + cfg.max_new + cfg.gamma_cap + 2
+    prompt = synth.make_prompts(shape.vocab, 1, cfg.n_prompt, seed=9).numpy()
+    rejects = []
+    for value in (0.0, float("nan")):
+        pair["target"]["head"][column, 5] = value
+        ctx = b.Context(b.make_cfg(shape, shape, 1, max_ctx, cfg.gamma_cap, cfg.block_b, cfg.rho, 0, cfg.succ_bias))
+        b.load_pair(ctx, pair)
+        _, ns, dl, al, _ = ctx.pacer_generate(prompt, cfg.max_new, 4, -1.0, mode=b.PACER_SAMPLE, seed=3)
+        rejects.append(int((al[0, : ns[0]] < dl[0, : ns[0]]).sum()))
+        ctx.close()
+    assert rejects[0] > 0 and rejects[1] == 0, rejects
