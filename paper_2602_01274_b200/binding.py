@@ -10,6 +10,8 @@ from __future__ import annotations
 import contextlib
 import ctypes as C
 import os
+import threading
+import weakref
 from typing import Dict, Optional
 
 import numpy as np
@@ -128,6 +130,25 @@ def _i32(a) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
 
+# Logits of a window are read into page-locked memory, which is filled at the link's rate: fresh pageable memory took 0.33 ms
+# for 3.2 MB, a twelfth of the forward that made them.  A program may keep what it reads, so the total alive is bounded.
+_PINNED_MAX = 64 << 20
+_pinned_lock = threading.Lock()
+_pinned_alive: list = []                        # weak references to the arrays (every view keeps its array alive)
+
+
+def _pinned_array(nbytes: int) -> Optional[np.ndarray]:
+    """A page-locked byte array, or None where it would exceed the bound."""
+    global _pinned_alive
+    with _pinned_lock:
+        alive = [a for a in (r() for r in _pinned_alive) if a is not None]
+        if sum(a.nbytes for a in alive) + nbytes > _PINNED_MAX:
+            return None
+        out = torch.empty(nbytes, dtype=torch.uint8, pin_memory=True).numpy()
+        _pinned_alive = [weakref.ref(a) for a in alive] + [weakref.ref(out)]
+    return out
+
+
 class Context:
     """One pacer_ctx.  Methods carry the names of the C entry points."""
 
@@ -216,13 +237,12 @@ class Context:
         return [a.as_dict() for a in arr]
 
     def pacer_read_buffer(self, which: int, dtype, count: int) -> np.ndarray:
+        """The first `count` elements of a device buffer.  Arrays of 256 KB to 64 MB are page-locked while at most 64 MB of
+        such arrays are alive in the process (their memory goes back to PyTorch's host cache, which reuses it); others are
+        ordinary memory.  As with any page-locked array, keep it until an asynchronous copy out of a part of it has ended."""
         nbytes = count * np.dtype(dtype).itemsize
-        if (256 << 10) <= nbytes <= (64 << 20):
-            # logits of a window: page-locked memory (PyTorch's caching allocator takes it back with the array) is filled at
-            # the link's rate; fresh pageable memory took 0.33 ms for 3.2 MB, a twelfth of the forward that made them
-            out = torch.empty(nbytes, dtype=torch.uint8, pin_memory=True).numpy().view(dtype)
-        else:
-            out = np.empty(count, dtype=dtype)
+        out = _pinned_array(nbytes) if (256 << 10) <= nbytes <= _PINNED_MAX else None
+        out = np.empty(count, dtype=dtype) if out is None else out.view(dtype)
         with torch.cuda.device(self.device):
             self._check(_lib.pacer_read_buffer(self._h, which, out.ctypes.data, out.nbytes))
         return out

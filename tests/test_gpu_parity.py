@@ -199,3 +199,24 @@ def test_bad_arguments_are_refused_before_any_launch(tiny):
         ctx.pacer_generate(bad, cfg.max_new, cfg.gamma_max, 0.5)                # token id out of range
     bcfg = b.make_cfg(cfg.target, cfg.draft, 1, 64, 6, 4)                       # gamma_cap not a multiple of b
     assert b.pacer_workspace_bytes(bcfg) == 0
+
+
+def test_page_locked_reads_are_bounded():
+    """A program that keeps every window's logits: at most 64 MB of them are page-locked, also through views, and the arrays it
+    has dropped make room again.  What is read is the same in both kinds of memory."""
+    from paper_2602_01274_b200 import binding as b
+    shape = synth.ModelShape(1, 64, 1, 1, 64, 120000)
+    ctx = b.Context(b.make_cfg(shape, shape, 1, 40, 16, 4, 1.05, 0, 8.0))
+    count = 17 * 120000                                      # 8.2 MB; what the untouched buffer holds does not matter
+    def pinned(arrays):
+        return [a for a in arrays if torch.from_numpy(a).is_pinned()]
+    ctx.pacer_read_buffer(b.BUF_TOKENS, np.int32, 4)
+    kept = [ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, count)[5:] for _ in range(12)]
+    assert 0 < len(pinned(kept)) < 12 and sum(a.nbytes for a in pinned(kept)) <= 64 << 20
+    for a in kept[1:]:
+        np.testing.assert_array_equal(a.view(np.int32), kept[0].view(np.int32))
+    del kept, a
+    assert len(pinned([ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, count)])) == 1
+    small = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, 1000)
+    assert small.shape == (1000,) and not pinned([small])
+    ctx.close()
