@@ -142,35 +142,49 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
             for (int h = 0; h < 2; ++h)
                 *reinterpret_cast<float2 *>(my + (m * 16 + h * 8 + g) * P + i * 8 + 2 * t) = make_float2(acc[i][m][2 * h], acc[i][m][2 * h + 1]);
     __syncthreads();
-    const int cols = T * 8, n_out = a.rows * cols;
-    // column -> (tile group, column within the group); the KW shares summed in warp order
-    auto local_sum = [&](int r, int col) -> float * {
-        const int ti = col >> 3;
-        int q = 0;
-        while (q + 1 < a.NW && T * (q + 1) / a.NW <= ti) ++q;
-        return lin_red + ((size_t)(q * KW) * R + r) * P + (col - (T * q / a.NW) * 8);
-    };
-    for (int i = threadIdx.x; i < n_out; i += LIN_THREADS) {
-        const int r = i / cols, col = i - r * cols, n = t0 * 8 + col;
-        float *p = local_sum(r, col);
-        float v = p[0];
-        for (int k = 1; k < KW; ++k) v += p[(size_t)k * R * P];
-        if (a.S > 1) p[0] = v;                                      // the block's sum, for the cluster
-        else if (n < a.N) a.y[(size_t)r * a.N + n] = v;
-    }
-    if (a.S > 1) {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-        for (int i = threadIdx.x + slice * LIN_THREADS; i < n_out; i += a.S * LIN_THREADS) {
-            const int r = i / cols, col = i - r * cols, n = t0 * 8 + col;
-            const uint32_t at = (uint32_t)__cvta_generic_to_shared(local_sum(r, col));
-            float v = 0.f;
-            for (int s = 0; s < a.S; ++s) {
-                float u;
-                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(u) : "r"(lin_peer(at, s)) : "memory");
-                v += u;
-            }
-            if (n < a.N) a.y[(size_t)r * a.N + n] = v;
+    // The sums: a tile group's KW warps share its rows, CL lanes a row's columns; the KW shares are added in warp order.  (An
+    // element at a time over the whole block, with the divisions that find its group, this took up to 18 us: 32 x 12210 x 512 in
+    // all 27.0 us, now 16.2; 32 x 32000 x 256 22.5, now 12.1; 5 x 2304 x 768 4.1, now 4.0.)
+    constexpr int CL = TT == 1 ? 8 : TT == 2 ? 16 : 32, RL = 32 / CL, CH = (P + CL - 1) / CL;
+    const int qc = (w1 - w0) * 8, n0 = (t0 + w0) * 8, lc = lane & (CL - 1);
+    float *sums = lin_red + (size_t)(nw * KW) * R * P + lc;
+#pragma unroll 4
+    for (int r = kw * RL + lane / CL; r < a.rows; r += KW * RL)
+#pragma unroll
+        for (int h = 0; h < CH; ++h) {
+            const int col = lc + CL * h;
+            if (col >= qc) continue;
+            float *p = sums + r * P + CL * h;
+            float v = p[0];
+            for (int k = 1; k < KW; ++k) v += p[(size_t)k * R * P];
+            if (a.S > 1) p[0] = v;                                  // the block's sum, for the cluster
+            else if (n0 + col < a.N) a.y[(size_t)r * a.N + n0 + col] = v;
         }
+    if (a.S > 1) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        // the blocks share the rows; all slices' loads in flight
+        for (int r = (slice * KW + kw) * RL + lane / CL; r < a.rows; r += a.S * KW * RL) {
+            float u[CH][8];
+#pragma unroll
+            for (int h = 0; h < CH; ++h) {
+                const uint32_t at = (uint32_t)__cvta_generic_to_shared(sums + r * P + CL * h);
+#pragma unroll
+                for (int s = 0; s < 8; ++s)
+                    if (s < a.S && lc + CL * h < qc)
+                        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(u[h][s]) : "r"(lin_peer(at, s)) : "memory");
+            }
+#pragma unroll
+            for (int h = 0; h < CH; ++h) {
+                const int col = lc + CL * h;
+                float v = 0.f;
+#pragma unroll
+                for (int s = 0; s < 8; ++s)
+                    if (s < a.S) v += u[h][s];
+                if (col < qc && n0 + col < a.N) a.y[(size_t)r * a.N + n0 + col] = v;
+            }
+        }
+        __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }

@@ -21,6 +21,11 @@ pytestmark = pytest.mark.gpu
     (2, 32000, 1024, 0),        # 28 tiles per block: four tile groups
     (32, 8 * 148 * 64 + 3, 32, 0),   # more than one wave of 64-tile blocks
     (17, 1000, 512, 1), (16, 300, 2080, 3),
+    (31, 8 * 148 * 2 - 5, 256, 0),   # the sums: two tiles a block (16 lanes a row), rows that do not fill the warps
+    (29, 8 * 148 * 3 + 1, 96, 0),    # four tiles in some blocks, three in the others
+    (13, 8 * 148 * 5 + 3, 288, 0),   # six tiles: two columns a lane, the second past the end
+    (32, 12210, 512, 0),             # 21 tiles in four groups, a cluster of two
+    (25, 1016, 2048, 0),             # one tile a block: eight lanes a row
 ])
 def test_linear_split_edges(rows, N, K, offset):
     from paper_2602_01274_b200 import binding as b
