@@ -196,7 +196,9 @@ struct LinPlan {
 // The split with the least weight bytes per block: S = 1 or 2 slices over all SMs (every pair of SMs can hold a
 // cluster of two); 4 or 8 only while few clusters are needed (an odd number of SMs per GPC strands some otherwise).  A
 // block keeps at least eight chunks of k, and the smaller S wins ties: 17 x 4096 x 11008 runs as 74 clusters of two,
-// 7 tiles each (full 98.9 %), where one slice would leave 4 tiles on some SMs against a mean of 3.46.
+// 7 tiles each (full 98.9 %), where one slice would leave 4 tiles on some SMs against a mean of 3.46.  More than eight tiles a
+// block without slices: slices could even out 5 % at most, and the sums of twice the tiles through the cluster cost 1 to 7 us
+// (32 x 12210 x 512 16.2 us with two slices, 9.5 without; 32 x 11008 x 4096 33.3, 26.9).
 static inline LinPlan lin_plan(int N, int K) {
     const int MT = (N + 7) / 8, nch = K / 32;
     LinPlan best{};
@@ -204,7 +206,7 @@ static inline LinPlan lin_plan(int N, int K) {
     const int cap[4] = {LIN_SMS, LIN_SMS / 2, 32, 16};
     for (int i = 0; i < 4; ++i) {
         const int S = 1 << i;
-        if (S > 1 && nch / S < 8) break;
+        if (S > 1 && (nch / S < 8 || best.NW > 1)) break;           // (NW > 1: more than eight tiles a block without slices)
         const int waves = (MT + cap[i] * 64 - 1) / (cap[i] * 64);   // at most 64 tiles per block
         if (S > 1 && waves > 1) break;
         const int groups = MT < cap[i] * waves ? MT : cap[i] * waves, tiles = (MT + groups - 1) / groups;

@@ -24,7 +24,8 @@ pytestmark = pytest.mark.gpu
     (31, 8 * 148 * 2 - 5, 256, 0),   # the sums: two tiles a block (16 lanes a row), rows that do not fill the warps
     (29, 8 * 148 * 3 + 1, 96, 0),    # four tiles in some blocks, three in the others
     (13, 8 * 148 * 5 + 3, 288, 0),   # six tiles: two columns a lane, the second past the end
-    (32, 12210, 512, 0),             # 21 tiles in four groups, a cluster of two
+    (32, 8880, 512, 0),              # 15 tiles in two groups, a cluster of two
+    (32, 12210, 512, 0),             # eleven tiles: no cluster
     (25, 1016, 2048, 0),             # one tile a block: eight lanes a row
 ])
 def test_linear_split_edges(rows, N, K, offset):
