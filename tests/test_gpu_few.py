@@ -1,7 +1,9 @@
 """Forwards of few live rows (drafts, pre-verification calls, autoregressive steps, early-stopped windows) at the edges of
 their kernel: 1 to 17 live rows (8 and 16 are operand sizes, 17 is the other kernel's), fewer weight rows than blocks and
-several passes per block, grouped heads, both head sizes, contexts around the key splits.  The logits of every forward
-against the oracle's, 2e-2 as everywhere (the activations carry 16 mantissa bits: what is seen is below 1e-4)."""
+several passes per block, grouped heads, both head sizes, contexts around the key splits.  The logits of every forward (draft
+steps and verify forwards of short and full windows) against the oracle's.  The activations carry 16 mantissa bits; what is
+seen is at most 2.2e-5 on logits and 2.3e-6 on alpha_hat, the tolerance about four times that.  One lost remainder plane moves
+the logits of these shapes by 5e-4 to 6e-3 (fp64 model with one site rounded to 8 bits; q and k of the narrow shape 3e-5)."""
 import dataclasses
 
 import numpy as np
@@ -12,7 +14,7 @@ from paper_2602_01274_b200 import synth
 from tests.common import oracle_models
 
 pytestmark = pytest.mark.gpu
-TOL = 2e-2
+TOL, ALPHA_TOL = 1e-4, 1e-5
 
 SHAPES = {
     # head dimension 64, fewer two-row units than blocks in the residual projections, ragged vocabulary
@@ -38,25 +40,27 @@ def test_verify_rows(shape, window, n_prompt):
     ctx.pacer_prefill(prompt, cfg.max_new, window, -1.0)
     o = orc.Pacer(To, Do, Bo, max_ctx, b=cfg.block_b, gamma_cap=window, t0=-1.0, rho=cfg.rho)
     o.prefill(prompt[0])
-    V, blocks = T.vocab, window // cfg.block_b
+    V, blocks, rows = T.vocab, window // cfg.block_b, {}
     for k in range(blocks):
         for _ in range(cfg.block_b):
             ctx.pacer_draft_step()
         ctx.pacer_preverify()
         o.draft_block(); o.preverify()
-        if k not in (0, blocks - 1):
-            continue
-        ctx.pacer_verify()                          # 1 + the drafts so far live rows
-        if k == blocks - 1:
-            o.verify()
-            gamma = (k + 1) * cfg.block_b
-            got = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, (window + 1) * V).reshape(window + 1, V)[: gamma + 1]
-            y = ctx.pacer_read_buffer(b.BUF_DRAFTS, np.int32, window)[:gamma]
-            if o.stats()["min_margin_draft"] > 2 * TOL:
-                np.testing.assert_array_equal(y, o.y()[:gamma])
-                assert np.abs(got - o.plogits(gamma + 1)).max() < TOL
-                al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, window)[:gamma]
-                assert np.abs(al - o.alpha()[:gamma]).max() < 2e-3
+        if k in (0, blocks - 1):
+            ctx.pacer_verify()                      # 1 + the drafts so far live rows
+            rows[k] = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, (window + 1) * V).reshape(window + 1, V)
+    o.verify()
+    gamma = blocks * cfg.block_b
+    assert o.stats()["min_margin_draft"] > 2 * TOL
+    np.testing.assert_array_equal(ctx.pacer_read_buffer(b.BUF_DRAFTS, np.int32, window)[:gamma], o.y()[:gamma])
+    p, q = o.plogits(gamma + 1), o.qlogits(gamma)
+    for k, got in rows.items():                     # a row depends on the drafts before it only
+        n = (k + 1) * cfg.block_b + 1
+        assert np.abs(got[:n] - p[:n]).max() < TOL, k
+    got = ctx.pacer_read_buffer(b.BUF_DRAFT_LOGITS, np.float32, window * V).reshape(window, V)[:gamma]
+    assert np.abs(got - q).max() < TOL
+    al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, window)[:gamma]
+    assert np.abs(al - o.alpha()[:gamma]).max() < ALPHA_TOL
     ctx.close()
 
 
@@ -75,8 +79,8 @@ def test_batched_autoregressive_rows(batch):
     tok, _ = ctx.pacer_generate_ar(prompts, cfg.max_new)
     for s in range(batch):
         out, margin = orc.generate_ar(To, prompts[s], cfg.max_new)
-        if margin > 2 * TOL:
-            np.testing.assert_array_equal(tok[s], out, err_msg=str(s))
+        assert margin > 2 * TOL, s
+        np.testing.assert_array_equal(tok[s], out, err_msg=str(s))
     ctx.close()
 
 
