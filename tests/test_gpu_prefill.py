@@ -1,8 +1,9 @@
 """Prompt prefill at the edges of its tiles and chunks: the last prompt through the forward kernel and the first through the
 tiled GEMMs (32 / 33 rows), 128-row tiles with remainders, a batch whose sequences share a tile, more rows than a chunk,
 grouped heads and both head sizes.  Everything that later steps read of a prefill (the three models' caches) is checked
-through what they compute from it: target logits, drafts and alpha_hat of one block against the oracle's, 2e-2 / 2e-3 as
-everywhere."""
+through what they compute from it: target logits, drafts and alpha_hat of one block against the oracle's.  What is seen is at
+most 2.2e-5 on logits and 2.3e-6 on alpha_hat, the tolerance about four times that.  One lost remainder plane moves the logits of
+these shapes by 4e-4 to 7e-3 (fp64 model with one site rounded to 8 bits; q and k of the narrowest shape 1e-4)."""
 import numpy as np
 import pytest
 
@@ -11,10 +12,12 @@ from paper_2602_01274_b200 import synth
 from tests.common import oracle_models
 
 pytestmark = pytest.mark.gpu
-TOL, ALPHA_TOL = 2e-2, 2e-3
+TOL, ALPHA_TOL = 1e-4, 1e-5
 
 SHAPES = {
     "hd64": (synth.ModelShape(2, 256, 4, 4, 320, 2048), synth.ModelShape(2, 128, 2, 1, 192, 2048)),
+    # 10 and 65 blocks of 64 columns: the sums that leave the tensor cores every eight blocks end in a remainder
+    "long_k": (synth.ModelShape(2, 640, 5, 5, 4160, 2048), synth.ModelShape(2, 320, 5, 1, 2112, 2048)),
     "hd128_gqa": (synth.ModelShape(2, 512, 4, 2, 1088, 2048), synth.ModelShape(1, 256, 2, 2, 512, 2048)),
 }
 
@@ -22,7 +25,7 @@ SHAPES = {
 @pytest.mark.parametrize("shape,batch,n_prompt", [
     ("hd64", 1, 33), ("hd64", 1, 34), ("hd64", 2, 18), ("hd64", 3, 44), ("hd64", 1, 129), ("hd64", 1, 130),
     ("hd64", 1, 2050), ("hd64", 5, 500), ("hd128_gqa", 1, 65), ("hd128_gqa", 1, 300), ("hd128_gqa", 4, 97),
-    ("hd128_gqa", 1, 2305),
+    ("hd128_gqa", 1, 2305), ("long_k", 1, 140), ("long_k", 2, 50),
 ])
 def test_prefill_edges(shape, batch, n_prompt):
     from paper_2602_01274_b200 import binding as b
