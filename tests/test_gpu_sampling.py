@@ -148,3 +148,42 @@ def test_nan_logit_keeps_the_drafts(column):
         rejects.append(int((al[0, : ns[0]] < dl[0, : ns[0]]).sum()))
         ctx.close()
     assert rejects[0] > 0 and rejects[1] == 0, rejects
+
+
+@pytest.mark.parametrize("batch,window,t0", [(3, 16, 0.5), (12, 8, 0.5), (12, 8, -1.0), (17, 4, -1.0)])
+def test_sampled_batch_matches_oracle(batch, window, t0):
+    """Several sampled sequences at once, each against the oracle's run of it alone: windows that stop at different blocks,
+    different numbers of steps (a sequence that has finished idles beside the others), packed rows of several sequences in the
+    few-row kernel and more of them than it takes.  A sequence counts where the oracle's decisions are ten times what logits of
+    these shapes differ by (below 1e-4) clear of a tie."""
+    from paper_2602_01274_b200 import binding as b
+    margin = 1e-3
+    T, D = synth.ModelShape(2, 128, 2, 1, 192, 1001), synth.ModelShape(1, 64, 1, 1, 64, 1001)
+    cfg = synth.PairConfig("batch", T, D, agree=0.7, n_prompt=11, max_new=16, gamma_max=window, batch=batch)
+    gpu = synth.make_pair(cfg, seed=4, device="cuda:0", std=0.08)
+    cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
+    To, Do, Bo = oracle_models(cfg, cpu)
+    max_ctx = cfg.n_prompt + cfg.max_new + window + 2
+    ctx = b.Context(b.make_cfg(T, D, batch, max_ctx, window, cfg.block_b, cfg.rho, 0, cfg.succ_bias))
+    b.load_pair(ctx, gpu)
+    prompts = synth.make_prompts(T.vocab, batch, cfg.n_prompt, seed=5).numpy()
+    tok, ns, dl, al, _ = ctx.pacer_generate(prompts, cfg.max_new, window, t0, mode=b.PACER_SAMPLE, seed=22)
+    ar, _ = ctx.pacer_generate_ar(prompts, cfg.max_new, mode=b.PACER_SAMPLE, seed=22)
+    ctx.close()
+    comparable, comparable_ar, steps = 0, 0, set()
+    for s in range(batch):
+        o = orc.Pacer(To, Do, Bo, max_ctx, b=cfg.block_b, gamma_cap=window, t0=t0, rho=cfg.rho, mode=1, seed=22, seq_id=s)
+        out_o, dl_o, al_o, st = o.generate(prompts[s], cfg.max_new)
+        if min(st["min_margin_target"], st["min_margin_draft"], st["min_margin_accept"]) > 2 * margin and \
+                (t0 < 0 or st["min_margin_stop"] > margin / 10):
+            comparable += 1
+            steps.add(len(dl_o))
+            np.testing.assert_array_equal(tok[s], out_o, err_msg=f"sequence {s}")
+            assert ns[s] == len(dl_o), s
+            np.testing.assert_array_equal(dl[s, : ns[s]], dl_o, err_msg=f"sequence {s}")
+            np.testing.assert_array_equal(al[s, : ns[s]], al_o, err_msg=f"sequence {s}")
+        out_o, m = orc.generate_ar(To, prompts[s], cfg.max_new, mode=1, seed=22, seq=s)
+        if m > 2 * margin:
+            comparable_ar += 1
+            np.testing.assert_array_equal(ar[s], out_o, err_msg=f"sequence {s} (autoregressive)")
+    assert min(comparable, comparable_ar) >= batch - batch // 4 and len(steps) > 1, (comparable, comparable_ar, steps)
