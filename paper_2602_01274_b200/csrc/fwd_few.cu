@@ -865,7 +865,7 @@ __device__ __forceinline__ void few_tail_draft(const FewCtx &c, const Args &a, i
 
 // ------------------------------------------------------------------ the kernel
 
-__global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ Args a, const int which) {
+__global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     if (smem_u32(smem) & 1023u) {               // the swizzled weight atoms need this alignment (the same in every block)
         if (threadIdx.x == 0) atomicCAS(a.fb.abort_flag, 0, 13);
@@ -1103,7 +1103,7 @@ bool few_rows_ok(const ModelDev &m, const Geom &g, int kind, int ncta) {
     return FEW_ROWS * xc * 4 <= F_XBYTES && xc + 16 <= 8 * 16;
 }
 
-cudaError_t launch_few(const Args &a, int which, int ncta, cudaStream_t st) {
+cudaError_t launch_few(const Args &a, int ncta, cudaStream_t st) {
     static bool attr_set[64] = {};           // the opt-in is per device
     constexpr int smem = F_GUARD + F_RING + F_SCRATCH + F_MISC;
     int dev = 0;
@@ -1114,7 +1114,7 @@ cudaError_t launch_few(const Args &a, int which, int ncta, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    void *params[] = {(void *)&a, (void *)&which};
+    void *params[] = {(void *)&a};
     return cudaLaunchCooperativeKernel((const void *)k_few, dim3(ncta), dim3(FEW_THREADS), params, smem, st);
 }
 

@@ -13,6 +13,6 @@ constexpr int FEW_ITEMS = 1024;                 // attention partials kept: item
 // Whether a forward of these dimensions can take the kernel (when its live rows turn out to be few): the residual columns
 // of a block fit its shared memory and one pass.
 bool few_rows_ok(const ModelDev &m, const Geom &g, int kind, int ncta);
-cudaError_t launch_few(const Args &a, int which, int ncta, cudaStream_t st);
+cudaError_t launch_few(const Args &a, int ncta, cudaStream_t st);
 
 }  // namespace fwd

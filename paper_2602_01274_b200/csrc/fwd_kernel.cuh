@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
     if (c.cta < g.batch && kind != KIND_VERIFY) {
         // the final RMSNorm of the hidden rows the pre-verification model will read
         if (kind == KIND_DRAFT || (kind == KIND_PREFILL && which == PACER_DRAFT)) tail_inv_rms(c, a, c.cta);
-        if (kind == KIND_DRAFT) tail_draft(c, a, c.cta, -1);
+        if (kind == KIND_DRAFT) tail_draft(c, a, c.cta);
         else if (kind == KIND_MB) tail_mb(c, a, c.cta);
         else if (kind == KIND_AR) tail_ar(c, a, c.cta, -1);
         else if (kind == KIND_PREFILL || kind == KIND_PREFILL_B) tail_prefill(c, a, c.cta, which);

@@ -27,16 +27,15 @@ __device__ __forceinline__ void tail_inv_rms(Ctx &c, const Args &a, int s) {
     bsync();
 }
 
-// End of one draft forward (Eq. 6): y_i, h_i queued for the pre-verification model, cache length.  pick: the sampled
-// token when the forward has drawn it already, else -1.
-__device__ __forceinline__ void tail_draft(Ctx &c, const Args &a, int s, int pick) {
+// End of one draft forward (Eq. 6): y_i, h_i queued for the pre-verification model, cache length.
+__device__ __forceinline__ void tail_draft(Ctx &c, const Args &a, int s) {
     const DevPtrs &d = a.d;
     SeqState &st = d.st[s];
     const int n_in = c.n_rows[s], dm = a.m.cfg.d_model;
     if (n_in == 0) return;
     const int gamma = st.gamma, n_pend = st.n_pend, r_last = s * a.g.rps + n_in - 1;
-    int y_new = pick;
-    if (st.mode == PACER_SAMPLE && pick < 0)              // y_i ~ q_i by the Gumbel-max rule at the token's position
+    int y_new = 0;
+    if (st.mode == PACER_SAMPLE)                          // y_i ~ q_i by the Gumbel-max rule at the token's position
         y_new = gumbel_argmax(d.draft_logits + ((size_t)s * d.gamma_cap + gamma) * a.m.cfg.vocab, a.m.cfg.vocab, st.seed,
                               st.P + gamma, s, TAG_DRAFT, MMA_THREADS, reinterpret_cast<BestD *>(c.scratch), true);
     const bool queue = !st.sched;                        // with prescribed windows nothing is pre-verified
@@ -122,7 +121,7 @@ __device__ __forceinline__ void tail_prefill(Ctx &c, const Args &a, int s, int w
     }
 }
 
-// End of one autoregressive target step (Eq. 1).
+// End of one autoregressive target step (Eq. 1).  pick: the sampled token when the forward has drawn it already, else -1.
 __device__ __forceinline__ void tail_ar(Ctx &c, const Args &a, int s, int pick) {
     if (c.n_rows[s] == 0) return;
     const DevPtrs &d = a.d;

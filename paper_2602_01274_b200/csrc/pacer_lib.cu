@@ -504,7 +504,7 @@ static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux
     if (fwd::few_rows_ok(m, g, kind, c->ncta)) {
         // The live rows are counted on the device: k_few takes the forward when they are at most 16, k_forward (launched
         // behind it where the geometry allows more; a sequence that k_few has committed shows one row then) otherwise.
-        CK(fwd::launch_few(a, which, c->ncta, c->stream));
+        CK(fwd::launch_few(a, c->ncta, c->stream));
         ++c->launches;
         a.few_max = fwd::FEW_ROWS;
     }
