@@ -250,12 +250,12 @@ int pacer_generate_ar(pacer_ctx *ctx, const int32_t *prompt, int batch, int n_pr
                       uint64_t seed, int32_t *out_tokens, pacer_stats *stats);
 
 /* Kernel-level timing for roofline reports.  Between pacer_profile_begin and
- * pacer_profile_end every forward of the TARGET model (one launch of the
- * persistent forward kernel) is bracketed by a pair of CUDA events on the
- * context's stream (at most 4096 launches are recorded; later ones run untimed)
- * and every block of every forward (any model) stamps the device clock at its phase
+ * pacer_profile_end every forward of the TARGET model (a decoding forward, which is
+ * one launch or two, or one chunk of a prompt) is bracketed by a pair of CUDA events
+ * on the context's stream (at most 4096 forwards are recorded; later ones run untimed)
+ * and every block of every decoding forward (any model) stamps the device clock at its phase
  * boundaries (PACER_BUF_PHASE_NS keeps the last forward's).  pacer_profile_end [sync] returns the summed device time
- * of those launches (ms), the bf16 weight bytes they streamed and their count.
+ * of those forwards (ms), the bf16 weight bytes they streamed and their count.
  * Whole-loop timings are taken without it. */
 int pacer_profile_begin(pacer_ctx *ctx);
 int pacer_profile_end(pacer_ctx *ctx, double *fwd_ms, double *fwd_weight_bytes, int64_t *fwd_launches);

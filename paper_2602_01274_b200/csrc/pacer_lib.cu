@@ -32,7 +32,7 @@ struct pacer_ctx {
     pf::Bufs pf;
     int pf_rows;
     int ncta;                  // blocks of the forward kernel (one per SM)
-    std::map<int, fwd::Plan> plans;   // key: which * 2 + has_head
+    std::map<int, fwd::Plan> plans;   // key: model, head or not, row tiles and groups (run_forward)
     unsigned long long *prof_stamps;
     int batch;                 // sequences of the current run
     int mode;                  // PACER_GREEDY / PACER_SAMPLE of the current run
@@ -486,8 +486,22 @@ static double model_weight_bytes(const ModelDev &m, bool head) {
     return 2.0 * (k.n_layers * per_layer + (head ? (double)k.vocab * k.d_model : 0.0));
 }
 
-// Runs model `which` on the rows `kind` selects: ONE cooperative launch of the
-// persistent forward kernel, which also takes the stage's decisions in its tail.
+// Events around one forward of the target (pacer_profile_begin).
+static int prof_start(pacer_ctx *c, int which, bool *on) {
+    *on = c->prof_on && which == PACER_TARGET && c->prof_used + 2 <= c->prof_ev.size();
+    if (*on) CK(cudaEventRecord(c->prof_ev[c->prof_used], c->stream));
+    return PACER_OK;
+}
+static int prof_stop(pacer_ctx *c, bool on, double weight_bytes) {
+    if (!on) return PACER_OK;
+    CK(cudaEventRecord(c->prof_ev[c->prof_used + 1], c->stream));
+    c->prof_used += 2;
+    c->prof_bytes += weight_bytes;
+    return PACER_OK;
+}
+
+// Runs model `which` on the rows `kind` selects: one cooperative launch of k_few or k_forward, or one of each (see below); the
+// kernel that does the work also takes the stage's decisions in its tail.
 static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux, bool head) {
     ModelDev &m = c->model[which];
     if (g.rtot > fwd::MAX_ROWS || g.batch > fwd::MAX_SEQ) return fail(c, PACER_EUNSUPPORTED, "too many rows or sequences in one forward");
@@ -498,8 +512,9 @@ static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux
     fwd::Args a;
     a.d = c->d; a.m = m; a.g = g; a.P = it->second; a.fb = c->fb; a.kind = kind; a.aux = aux;
     a.fb.prof = (c->prof_on && c->ncta <= fwd::PROF_BLOCKS) ? c->prof_stamps : nullptr;
-    const bool prof = c->prof_on && which == PACER_TARGET && c->prof_used + 2 <= c->prof_ev.size();
-    if (prof) CK(cudaEventRecord(c->prof_ev[c->prof_used], c->stream));
+    bool prof;
+    int rc;
+    if ((rc = prof_start(c, which, &prof))) return rc;
     a.few_max = 0;
     if (fwd::few_rows_ok(m, g, kind, c->ncta)) {
         // The live rows are counted on the device: k_few takes the forward when they are at most 16, k_forward (launched
@@ -512,12 +527,7 @@ static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux
         CK(fwd::launch(a, which, c->ncta, c->stream));
         ++c->launches;
     }
-    if (prof) {
-        CK(cudaEventRecord(c->prof_ev[c->prof_used + 1], c->stream));
-        c->prof_used += 2;
-        c->prof_bytes += model_weight_bytes(m, head);
-    }
-    return PACER_OK;
+    return prof_stop(c, prof, model_weight_bytes(m, head));
 }
 
 static int need_ready(pacer_ctx *c, bool prefilled) {
@@ -600,7 +610,14 @@ static int prefill_models(pacer_ctx *c, int n_prompt, bool target, bool draft, b
             return pf::run(c->model[which], c->d, c->pf, c->fb.abort_flag, batch, nj, c0, input, c->model[PACER_DRAFT].normf, need_x, c->ncta,
                            c->stream, &c->launches);
         };
-        if (target) CK(model(PACER_TARGET, pf::EMBED, false));
+        if (target) {
+            const ModelDev &m = c->model[PACER_TARGET];
+            const double rest = 2.0 * ((double)m.cfg.d_model * m.cfg.n_heads * m.hd + 3.0 * m.cfg.d_model * m.cfg.d_ffn);
+            bool prof;
+            if ((rc = prof_start(c, PACER_TARGET, &prof))) return rc;
+            CK(model(PACER_TARGET, pf::EMBED, false));
+            if ((rc = prof_stop(c, prof, model_weight_bytes(m, false) - rest))) return rc;    // (the last layer ends with q, k, v)
+        }
         if (draft) CK(model(PACER_DRAFT, pf::EMBED, mb));
         if (draft && mb) CK(model(PACER_PREVERIFY, pf::HIDDEN, false));
     }

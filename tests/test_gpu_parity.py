@@ -220,3 +220,21 @@ def test_page_locked_reads_are_bounded():
     small = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, 1000)
     assert small.shape == (1000,) and not pinned([small])
     ctx.close()
+
+
+def test_profile_counts_the_prompt(tiny):
+    """Every forward of the target is bracketed, also a prompt's (one for a few rows, one per chunk for many)."""
+    cfg, b = tiny["cfg"], tiny["b"]
+    layer = cfg.target.streamed_weight_bytes() - 2 * cfg.target.vocab * cfg.target.d_model
+    for batch, n_prompt in ((1, 9), (1, 300), (3, 2000)):
+        ctx = b.Context(b.make_cfg(cfg.target, cfg.draft, batch, n_prompt + 40, 8, 4, cfg.rho, 0, cfg.succ_bias))
+        b.load_pair(ctx, synth.make_pair(cfg, seed=0, device="cuda:0"))
+        prompts = synth.make_prompts(cfg.target.vocab, batch, n_prompt, seed=1).numpy()
+        ctx.pacer_profile_begin()
+        ctx.pacer_prefill(prompts, 8, 8, -1.0)
+        ms, nbytes, n = ctx.pacer_profile_end()
+        chunks = -(-(n_prompt - 1) // (2048 // batch))
+        assert n == chunks and ms > 0
+        # a prompt through the tiled path does not run the last layer's other projections
+        assert 0.5 * chunks * layer < nbytes <= chunks * layer, (nbytes, layer)
+        ctx.close()
