@@ -218,8 +218,8 @@ int pacer_read_buffer(pacer_ctx *ctx, int which, void *host_dst, size_t bytes);
  * calls of the whole window, the verify forward, the acceptance) are captured once
  * per context as a CUDA graph and replayed every step (not on the legacy default
  * stream, which cannot be captured: there the launches are issued one by one).  Greedy runs take the
- * acceptance (Eq. 5) in the tail of the verify forward; sampling runs in a kernel of
- * its own.
+ * acceptance (Eq. 5) in the tail of the verify forward; sampling runs in two kernels
+ * of its own.
  * Outputs, all host, caller-owned:
  *   out_tokens     int32 [batch][max_new]
  *   out_n_steps    int32 [batch]
@@ -238,7 +238,7 @@ int pacer_generate(pacer_ctx *ctx, const int32_t *prompt, int batch, int n_promp
  * decoding with the optimal draft length gamma* of Section 3.1 (the upper bound an
  * oracle-knowledge window reaches).  M_B is not run.  The draft model catches up, in
  * the first forward of its next window, on the rows it has not seen; such a forward
- * holds at most 16 rows per sequence (32 / batch if that is less), and when the
+ * holds at most 16 rows per sequence (144 / batch if that is less), and when the
  * backlog reaches that number a prescribed 0 becomes 1.  Outputs as pacer_generate. */
 int pacer_generate_sched(pacer_ctx *ctx, const int32_t *prompt, int batch, int n_prompt, int max_new,
                          const int32_t *windows, int n_windows, int mode, uint64_t seed, int32_t *out_tokens,
@@ -261,8 +261,9 @@ int pacer_profile_begin(pacer_ctx *ctx);
 int pacer_profile_end(pacer_ctx *ctx, double *fwd_ms, double *fwd_weight_bytes, int64_t *fwd_launches);
 
 /* Y[r][n] = sum_k X[r][k] * W[n][k]: a stand-alone skinny weight-streaming product
- * (ONE kernel on mma.sync with plain bf16 activations; the projections inside
- * the forwards run on a different, tcgen05 path with split activations).  x: device bf16
+ * (ONE kernel on mma.sync with plain bf16 activations; the projections inside the
+ * forwards are other kernels, with split activations: mma.sync up to 16 live rows,
+ * tcgen05 beyond and for prompts).  x: device bf16
  * [rows][K] row-major; w: device bf16 [N][K], 16-byte aligned; y: device f32 [rows][N];
  * scratch: device, at least pacer_linear_scratch_bytes(rows, N, K) bytes (part of the
  * interface; the kernel keeps its partial sums on chip and leaves it untouched).

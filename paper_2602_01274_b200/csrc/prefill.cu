@@ -372,7 +372,7 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t a) {
 }
 
 // Query rows j0 .. j0+63 of one head over the keys 0 .. c0 + j, from the cache (the chunk's own keys are there already).
-// Bound by the mma.sync rate: 48 MMAs per 16 rows and 8 keys.
+// Bound by the mma.sync rate: 48 MMAs per 16 rows and 8 keys at head dimension 128, 24 at 64.
 template <int HD>
 __global__ void __launch_bounds__(128, 2) k_pf_attn(const __grid_constant__ AArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];

@@ -1,10 +1,9 @@
 """The allocation-free product entry point against the ordinary one.
 
 pacer_linear_static serves callers that cannot hand the library any scratch memory (a server whose arena owns
-the whole device, a host without an allocator): its scratch is a fixed array inside the library.  The check:
-through the C ABI, twice in a row on different inputs and shapes (the array keeps the first call's contents),
-its output must equal pacer_linear's, which gets fresh caller scratch.  Both run the same kernels in the same
-order, so the comparison is exact; the tolerance of the other product tests is kept as the stated bound.  The
+the whole device, a host without an allocator): the kernel keeps its partial sums on chip.  The check: through the
+C ABI, twice in a row on different inputs and shapes, its output must equal pacer_linear's.  Both run the same
+kernel, so the outputs are the same; the tolerance of the other product tests is kept as the stated bound.  The
 same output is also compared with the CPU oracle's product on sampled columns."""
 import numpy as np
 import pytest
@@ -38,7 +37,7 @@ def test_static_scratch_product_equals_the_ordinary_one_twice_in_a_row():
 def test_static_scratch_product_refuses_shapes_beyond_its_array():
     from paper_2602_01274_b200 import binding as b
     dev = "cuda:0"
-    rows, N, K = 32, 32000, 4096          # needs about 8 MB of partial sums
+    rows, N, K = 32, 32000, 4096          # the interface's formula: about 8 MB
     assert b._lib.pacer_linear_scratch_bytes(rows, N, K) > b.PACER_LINEAR_STATIC_BYTES
     x = torch.zeros(rows, K, dtype=torch.bfloat16, device=dev)
     w = torch.zeros(N, K, dtype=torch.bfloat16, device=dev)
