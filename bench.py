@@ -146,10 +146,10 @@ def measured_traffic_ratio():
 
 
 def verify_forward_numbers(ctx, cfg, prompt, n_ver, n_warm):
-    """Times the target verify forward with a full draft window (gamma_cap + 1 rows).  The forward is ONE launch
-    of the persistent kernel k_forward, so the dominant kernel's launch duration is the forward's: measured twice,
-    with torch events around n_ver launches on the context's stream, and launch by launch with the library's own
-    event pairs (pacer_profile_*)."""
+    """Times the target verify forward with a full draft window (gamma_cap + 1 rows).  With more than 16 rows the
+    forward is one launch of the persistent kernel k_forward, behind a launch of k_few that returns at once, so the
+    dominant kernel's launch duration is nearly the forward's: measured twice, with torch events around n_ver
+    forwards on the context's stream, and forward by forward with the library's own event pairs (pacer_profile_*)."""
     ctx.pacer_prefill(prompt, cfg.max_new, cfg.gamma_max, -1.0)
     for _ in range(cfg.gamma_cap // cfg.block_b):
         for _ in range(cfg.block_b):
