@@ -17,9 +17,10 @@
 // accumulator over all of K the logits behind a 300-token prompt were 1.7 times as far from an fp64 forward (1.4e-4 against
 // 8e-5 at 14 layers of width 7168).
 //
-// Attention: 64 query rows of a head per block on mma.sync, keys and values (value + remainder) in tiles of 32 through
-// shared memory, FlashAttention style.  Products of two remainders are left out (2^-18).
+// Attention: pf_attention.cuh.
 #include "prefill.h"
+
+#include <cuda.h>
 
 #include <algorithm>
 
@@ -130,6 +131,24 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
                    "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// One lane of the warp (the same one each time).
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p;
+}
+// An MMA and a commit of the lane with `on`, called by the whole warp: only the instruction itself is predicated, so that the
+// descriptors are computed in uniform registers.  In a branch for one lane an MMA took 95 cycles to issue; N = 128 computes for 64.
+__device__ __forceinline__ void umma_if(uint32_t on, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
+                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(on) : "memory");
+}
+__device__ __forceinline__ void umma_commit_if(uint32_t on, uint64_t *bar) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(on) : "memory");
+}
 
 // The row-wise step on 16 accumulator columns (weight rows n0 ..) of token row r.
 template <int EPI>
@@ -352,168 +371,7 @@ __global__ void __launch_bounds__(THREADS_G, 1) k_pf_gemm(const __grid_constant_
 
 // ------------------------------------------------------------------ attention
 
-struct AArgs {
-    const float *q;
-    const bf16 *kc, *vc;
-    size_t kv_lo;
-    bf16 *out;
-    int32_t H, Hkv, max_ctx, nj, c0, rows;
-};
-
-constexpr int AQ = 64, AK = 32;            // query rows of a block (16 per warp), keys of a tile
-template <int HD>
-constexpr int attn_smem() { return 2 * 4 * AK * (HD * 2 + 16); }
-
-__device__ __forceinline__ void cp16(uint32_t dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
-}
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t a) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
-}
-
-// Query rows j0 .. j0+63 of one head over the keys 0 .. c0 + j, from the cache (the chunk's own keys are there already).
-// Bound by the mma.sync rate: 48 MMAs per 16 rows and 8 keys at head dimension 128, 24 at 64.
-template <int HD>
-__global__ void __launch_bounds__(128, 2) k_pf_attn(const __grid_constant__ AArgs a) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    constexpr int PITCH = HD * 2 + 16, PLANE = AK * PITCH, NK16 = HD / 16, NC = HD / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int qt = gridDim.x - 1 - blockIdx.x, h = blockIdx.y, seq = blockIdx.z, kh = h / (a.H / a.Hkv);   // longest rows first
-    const int j0 = qt * AQ, jw = j0 + warp * 16;
-    const int n_keys = a.c0 + min(j0 + AQ, a.nj), n_tiles = (n_keys + AK - 1) / AK;
-    const size_t cb = ((size_t)seq * a.Hkv + kh) * a.max_ctx * HD;
-    const bf16 *src[4] = {a.kc + cb, a.kc + a.kv_lo + cb, a.vc + cb, a.vc + a.kv_lo + cb};
-    auto load = [&](int tile) {
-        const uint32_t base = smem_u32(smem) + (uint32_t)(tile & 1) * 4u * PLANE;
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-            for (int i = threadIdx.x; i < AK * (HD / 8); i += 128) {
-                const int key = i / (HD / 8), c = i - key * (HD / 8);
-                cp16(base + p * PLANE + key * PITCH + c * 16, src[p] + (size_t)min(tile * AK + key, n_keys - 1) * HD + c * 8);
-            }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    load(0);
-    // the warp's 16 query rows as the first operand, values and remainders
-    uint32_t qh[NK16][4], ql[NK16][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int j = jw + g + 8 * i;
-        const float *p = a.q + (size_t)(seq * a.nj + min(j, a.nj - 1)) * (a.H * HD) + h * HD + 2 * t;
-#pragma unroll
-        for (int k = 0; k < NK16; ++k) {
-            const float2 u = *reinterpret_cast<const float2 *>(p + k * 16), w = *reinterpret_cast<const float2 *>(p + k * 16 + 8);
-            split2(u.x, u.y, qh[k][i], ql[k][i]);
-            split2(w.x, w.y, qh[k][2 + i], ql[k][2 + i]);
-        }
-    }
-    float o[HD / 8][4], mx[2] = {-INFINITY, -INFINITY}, ls[2] = {0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < HD / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    const int p_lo = a.c0 + jw + g, p_hi = p_lo + 8;     // positions of this lane's two rows
-    for (int tile = 0; tile < n_tiles; ++tile) {
-        if (tile + 1 < n_tiles) { load(tile + 1); asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        const uint32_t base = smem_u32(smem) + (uint32_t)(tile & 1) * 4u * PLANE;
-        const int k0 = tile * AK;
-        if (k0 <= a.c0 + jw + 15) {                      // (the same in the whole warp)
-            float s[4][4];
-#pragma unroll
-            for (int n = 0; n < 4; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
-            const uint32_t krow = base + (uint32_t)(lane & 7) * PITCH + (uint32_t)(lane >> 3) * 16u;
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    uint32_t b[4];
-                    ldsm4(b, krow + n * 8 * PITCH + c * 64);
-                    mma16816(s[n], qh[2 * c][0], qh[2 * c][1], qh[2 * c][2], qh[2 * c][3], b[0], b[1]);
-                    mma16816(s[n], qh[2 * c + 1][0], qh[2 * c + 1][1], qh[2 * c + 1][2], qh[2 * c + 1][3], b[2], b[3]);
-                    mma16816(s[n], ql[2 * c][0], ql[2 * c][1], ql[2 * c][2], ql[2 * c][3], b[0], b[1]);
-                    mma16816(s[n], ql[2 * c + 1][0], ql[2 * c + 1][1], ql[2 * c + 1][2], ql[2 * c + 1][3], b[2], b[3]);
-                    ldsm4(b, krow + PLANE + n * 8 * PITCH + c * 64);
-                    mma16816(s[n], qh[2 * c][0], qh[2 * c][1], qh[2 * c][2], qh[2 * c][3], b[0], b[1]);
-                    mma16816(s[n], qh[2 * c + 1][0], qh[2 * c + 1][1], qh[2 * c + 1][2], qh[2 * c + 1][3], b[2], b[3]);
-                }
-            if (k0 + AK - 1 > a.c0 + jw) {               // the diagonal: causal mask (it also covers keys past the end)
-#pragma unroll
-                for (int n = 0; n < 4; ++n)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int key = k0 + n * 8 + 2 * t + e;
-                        if (key > p_lo) s[n][e] = -INFINITY;
-                        if (key > p_hi) s[n][2 + e] = -INFINITY;
-                    }
-            }
-            uint32_t ph[2][4], pl[2][4];
-            float cr[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                float m = mx[i];
-#pragma unroll
-                for (int n = 0; n < 4; ++n) m = fmaxf(m, fmaxf(s[n][2 * i], s[n][2 * i + 1]));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-                const float corr = m == -INFINITY ? 1.f : __expf(mx[i] - m), ms = m == -INFINITY ? 0.f : m;
-                mx[i] = m;
-                float sum = 0.f;
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    const float p0 = __expf(s[n][2 * i] - ms), p1 = __expf(s[n][2 * i + 1] - ms);
-                    sum += p0 + p1;
-                    split2(p0, p1, ph[n >> 1][(n & 1) * 2 + i], pl[n >> 1][(n & 1) * 2 + i]);
-                }
-                ls[i] = ls[i] * corr + sum;
-                cr[i] = corr;
-            }
-            const uint32_t vrow = base + 2 * PLANE + (uint32_t)((lane & 7) + ((lane >> 3) & 1) * 8) * PITCH + (uint32_t)(lane >> 4) * 16u;
-            // (the tile's products in sums of their own, added in ordinary fp32: the tensor cores truncate)
-#pragma unroll
-            for (int c = 0; c < HD / 16; ++c) {
-                float x[4] = {0.f, 0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    uint32_t b[4];
-                    ldsm4t(b, vrow + k * 16 * PITCH + c * 32);
-                    mma16816(x, ph[k][0], ph[k][1], ph[k][2], ph[k][3], b[0], b[1]);
-                    mma16816(y, ph[k][0], ph[k][1], ph[k][2], ph[k][3], b[2], b[3]);
-                    mma16816(x, pl[k][0], pl[k][1], pl[k][2], pl[k][3], b[0], b[1]);
-                    mma16816(y, pl[k][0], pl[k][1], pl[k][2], pl[k][3], b[2], b[3]);
-                    ldsm4t(b, vrow + PLANE + k * 16 * PITCH + c * 32);
-                    mma16816(x, ph[k][0], ph[k][1], ph[k][2], ph[k][3], b[0], b[1]);
-                    mma16816(y, ph[k][0], ph[k][1], ph[k][2], ph[k][3], b[2], b[3]);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    o[2 * c][e] = o[2 * c][e] * cr[e >> 1] + x[e];
-                    o[2 * c + 1][e] = o[2 * c + 1][e] * cr[e >> 1] + y[e];
-                }
-            }
-        }
-        __syncthreads();                                 // the tile is read; the copy after next may overwrite it
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        ls[i] += __shfl_xor_sync(0xffffffffu, ls[i], 1);
-        ls[i] += __shfl_xor_sync(0xffffffffu, ls[i], 2);
-        const int j = jw + g + 8 * i;
-        if (j >= a.nj) continue;
-        const float inv = 1.f / ls[i];
-        const int r = seq * a.nj + j, plane = operand_plane(r, a.rows);
-#pragma unroll
-        for (int c = 0; c < HD / 8; ++c) {
-            uint32_t hi, lo;
-            split2(o[c][2 * i] * inv, o[c][2 * i + 1] * inv, hi, lo);
-            bf16 *p = a.out + operand_index(r, h * HD + c * 8 + 2 * t, a.H * HD, a.rows);
-            *reinterpret_cast<uint32_t *>(p) = hi;
-            *reinterpret_cast<uint32_t *>(p + plane) = lo;
-        }
-    }
-}
+#include "pf_attention.cuh"
 
 __global__ void k_pf_lengths(SeqState *st, int batch, int n, int target, int draft, int mb) {
     const int s = threadIdx.x;
@@ -568,21 +426,6 @@ static cudaError_t launch_gemm(GArgs &a, int n_sm, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <int HD>
-static cudaError_t launch_attn(const AArgs &a, int batch, cudaStream_t st) {
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(k_pf_attn<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem<HD>());
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
-    k_pf_attn<HD><<<dim3((a.nj + AQ - 1) / AQ, a.H, batch), 128, attn_smem<HD>(), st>>>(a);
-    return cudaGetLastError();
-}
-
 #define PF(call)                                     \
     do {                                             \
         cudaError_t e_ = (call);                     \
@@ -597,6 +440,10 @@ cudaError_t run(const ModelDev &m, const DevPtrs &d, const Bufs &b, int32_t *abo
     InArgs in{d.x, m.embed, m.norm1, normf, b.x, b.xg, b.ssq, d.max_ctx, dm, nj, c0, rows, (int32_t)input, k.rms_eps};
     k_pf_input<<<rows, 256, 0, st>>>(in);
     PF(cudaGetLastError());
+    CUtensorMap mk, mv;
+    cudaError_t e = attn_map(&mk, m, m.kcache, d.max_batch, d.max_ctx);
+    if (e == cudaSuccess) e = attn_map(&mv, m, m.vcache, d.max_batch, d.max_ctx);
+    if (e != cudaSuccess) return e;
     int nss = 1;
     for (int l = 0; l < L; ++l) {
         const size_t kv = (size_t)l * d.max_batch * k.n_kv_heads * (size_t)d.max_ctx * m.hd;
@@ -612,8 +459,8 @@ cudaError_t run(const ModelDev &m, const DevPtrs &d, const Bufs &b, int32_t *abo
         g.H = k.n_heads; g.Hkv = k.n_kv_heads; g.hd = m.hd; g.max_ctx = d.max_ctx;
         PF(launch_gemm<E_QKV>(g, n_sm, st));
         if (l == L - 1 && !need_x) break;                // nothing reads the rest of the last layer
-        AArgs at{b.q, g.kc, g.vc, m.kv_lo, b.att, k.n_heads, k.n_kv_heads, d.max_ctx, nj, c0, rows};
-        PF(m.hd == 64 ? launch_attn<64>(at, batch, st) : launch_attn<128>(at, batch, st));
+        const AArgs at{b.q, b.att, k.n_heads, k.n_kv_heads, nj, c0, rows, l * d.max_batch * k.n_kv_heads, abort_flag};
+        PF(m.hd == 64 ? launch_attn<64>(mk, mv, at, batch, st) : launch_attn<128>(mk, mv, at, batch, st));
         op(OP_O, b.att, dm, hh, (dm + 15) / 16);
         g.x = b.x; g.ssq_out = b.ssq; g.gain = m.norm2 + (size_t)l * dm; g.out = b.xg; g.out_k = dm;
         PF(launch_gemm<E_RES>(g, n_sm, st));
