@@ -1,6 +1,7 @@
-// Skinny weight-streaming product: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32, bf16 in, fp32 sums, ONE launch.
+// Skinny weight-streaming product: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32, bf16 in, fp32 sums, ONE launch.  Two
+// kernels: k_linear_wide where every SM has its share of whole weight rows, k_linear else (see lin_run).
 //
-// Bound by reading W once from HBM.  Every lane reads its share of W with 128-bit loads straight into registers
+// k_linear.  Bound by reading W once from HBM.  Every lane reads its share of W with 128-bit loads straight into registers
 // (each weight is used exactly once, so staging it in shared memory would only add traffic), 8 to 32 loads in flight
 // per lane.  The activations come out of L2 through shared memory, eight chunks ahead: a lane copies exactly the 16-byte
 // pieces that it reads, so nothing is synchronised.  mma.m16n8k16 with
@@ -189,6 +190,123 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear(const LinArgs a) {
     }
 }
 
+struct LinWideArgs {
+    const bf16 *x, *w;
+    float *y;
+    int32_t rows, N, K;
+    int32_t per;             // weight rows of a pass at most (a multiple of 2, at most LW_ROWS)
+    int32_t xr;              // token rows of a stage (rows, up to a multiple of 8)
+};
+
+constexpr int LW_ROWS = 32;
+
+__device__ __forceinline__ void lin_ldsm4(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+
+// Everything through shared memory.  A block owns a run of weight rows (units of two, as even as they come: 4096 rows on 148 SMs
+// are 28 each, tiles of eight rows would be 32) and takes it in passes of up to 32; warp w owns the 64-column chunks w, w + 8, ...
+// of k, token and weight rows alike, and copies them for itself, D chunks deep: whole 128-byte lines, nothing but the sums at
+// the end of a pass is shared between warps, and the next pass's first chunks travel while a pass is summed up.  Two sets of
+// accumulators: the tensor cores truncate, and K / 16 products a set are what k_linear has with two slices (with one set the
+// error against fp64 was twice as large, 1.3e-6 at K = 11 008).  17 x 4096 x 11008: 23.2 us with k_linear (its loads of 64
+// bytes a row straight into registers), 19.2 here (4.7 TB/s); 17 x 4096 x 4096 13.1, 9.6; 5 x 2304 x 768 3.6, 3.1.
+template <int RM, int NA, int D>
+__global__ void __launch_bounds__(LIN_THREADS, 1) k_linear_wide(const LinWideArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    constexpr int R = RM * 16, P = NA * 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int units = (a.N + 1) >> 1, ub = units / (int)gridDim.x, ur = units - ub * (int)gridDim.x, b = blockIdx.x;
+    const int r0 = 2 * (b * ub + min(b, ur)), r1 = min(a.N, r0 + 2 * (ub + (b < ur ? 1 : 0)));
+    const int np = (r1 - r0 + a.per - 1) / a.per, chunks = (a.K + 63) >> 6, mine = (chunks - warp + 7) >> 3;
+    const int stage_bytes = (a.xr + a.per) * 128;
+    unsigned char *ring = smem + warp * D * stage_bytes;
+    float *red = reinterpret_cast<float *>(smem + (np > 1 ? 8 * D * stage_bytes : 0));      // [8 warps][R][P]; a single pass is done with the ring
+    auto pass_rows = [&](int p, int &lo, int &n) {                              // as even as they come
+        const int u = (r1 - r0 + 1) >> 1, q = u / np, m = u - q * np;
+        lo = r0 + 2 * (p * q + min(p, m)); n = min(r1 - lo, 2 * (q + (p < m ? 1 : 0)));
+    };
+    int lp = 0, lc = 0, lslot = 0, llo = 0, ln = 0;                              // what is copied next: pass, chunk, slot
+    if (np > 0) pass_rows(0, llo, ln);
+    auto load = [&]() {                                                          // a group per chunk, also when there is none left
+        if (lp < np && mine > 0) {
+            const int col = (warp + 8 * lc) * 64 + (lane & 7) * 8, sz = col < a.K ? 16 : 0;
+            unsigned char *st = ring + lslot * stage_bytes;
+            const bf16 *src = a.x + (sz ? col : 0);
+            for (int r = lane >> 3; r < a.rows; r += 4)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(st + r * 128 + (((lane & 7) ^ (r & 7)) << 4))), "l"(src + (size_t)r * a.K), "r"(sz) : "memory");
+            st += a.xr * 128;
+            src = a.w + (size_t)llo * a.K + (sz ? col : 0);
+#pragma unroll 4
+            for (int r = lane >> 3; r < ln; r += 4)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(st + r * 128 + (((lane & 7) ^ (r & 7)) << 4))), "l"(src + (size_t)r * a.K), "r"(sz) : "memory");
+            lslot = lslot + 1 == D ? 0 : lslot + 1;
+            if (++lc == mine) { lc = 0; if (++lp < np) pass_rows(lp, llo, ln); }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int i = 0; i < D - 1; ++i) load();
+    int slot = 0;
+    for (int p = 0; p < np; ++p) {
+        int lo, n;
+        pass_rows(p, lo, n);
+        float acc[2][NA][RM][4];
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int m = 0; m < RM; ++m)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[0][i][m][e] = acc[1][i][m][e] = 0.f;
+        for (int c = 0; c < mine; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(D - 2) : "memory");
+            __syncwarp();                                                        // every lane's copies; and the slot before is read
+            load();
+            const uint32_t xa = (uint32_t)__cvta_generic_to_shared(ring + slot * stage_bytes), wa = xa + (uint32_t)a.xr * 128u;
+            slot = slot + 1 == D ? 0 : slot + 1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {                                        // 16 columns
+                uint32_t x[RM][4], w[NA][2];
+#pragma unroll
+                for (int m = 0; m < RM; ++m)                                     // matrices: rows 0..7, 8..15 of columns 0..7, then of 8..15
+                    lin_ldsm4(x[m], xa + (uint32_t)(m * 16 + (lane & 15)) * 128u + (uint32_t)(((2 * k + (lane >> 4)) ^ (lane & 7)) << 4));
+#pragma unroll
+                for (int i = 0; i < NA; i += 2) {                                // two atoms: columns 0..7, 8..15 of each
+                    uint32_t v[4];
+                    lin_ldsm4(v, wa + (uint32_t)(i * 8 + (lane & 7) + ((lane >> 4) << 3)) * 128u + (uint32_t)(((2 * k + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
+                    w[i][0] = v[0]; w[i][1] = v[1]; w[i + 1][0] = v[2]; w[i + 1][1] = v[3];
+                }
+#pragma unroll
+                for (int i = 0; i < NA; ++i)
+#pragma unroll
+                    for (int m = 0; m < RM; ++m) mma_bf16_16816(acc[k & 1][i][m], x[m][0], x[m][1], x[m][2], x[m][3], w[i][0], w[i][1]);
+            }
+        }
+        if (np == 1) __syncthreads();
+        float *my = red + (size_t)warp * R * P;
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+#pragma unroll
+            for (int m = 0; m < RM; ++m)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    *reinterpret_cast<float2 *>(my + (m * 16 + h * 8 + g) * P + i * 8 + 2 * t) = make_float2(acc[0][i][m][2 * h] + acc[1][i][m][2 * h], acc[0][i][m][2 * h + 1] + acc[1][i][m][2 * h + 1]);
+        __syncthreads();
+        constexpr int RT = LIN_THREADS / P;                                      // rows at a time
+        const int col = threadIdx.x & (P - 1);
+        if (col < n)
+            for (int r = threadIdx.x / P; r < a.rows; r += RT) {
+                const float *q = red + r * P + col;
+                float v = q[0];
+#pragma unroll
+                for (int k = 1; k < 8; ++k) v += q[k * R * P];
+                a.y[(size_t)r * a.N + lo + col] = v;
+            }
+        if (p + 1 < np) __syncthreads();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 struct LinPlan {
     int S, groups, NW, TT;
 };
@@ -258,8 +376,44 @@ static cudaError_t lin_dispatch(int TT, const LinArgs &a, cudaStream_t st) {
     }
 }
 
+template <int RM, int NA, int D>
+static cudaError_t lin_wide_launch(const LinWideArgs &a, int smem, cudaStream_t st) {
+    static bool attr_set[64] = {};           // the opt-in is per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(k_linear_wide<RM, NA, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    const int units = (a.N + 1) / 2;
+    k_linear_wide<RM, NA, D><<<units < LIN_SMS ? units : LIN_SMS, LIN_THREADS, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int RM, int NA>
+static cudaError_t lin_wide_depth(const LinWideArgs &a, int np, cudaStream_t st) {
+    // room behind the ring: the sums of a pass, or (one pass) what the last atoms read past their rows
+    const int stage = 8 * (a.xr + a.per) * 128, sums = 8 * RM * 16 * NA * 8 * 4;
+    auto bytes = [&](int d) { return np > 1 ? d * stage + sums : d * stage + 4096 > sums ? d * stage + 4096 : sums; };
+    return bytes(4) <= 227 * 1024 ? lin_wide_launch<RM, NA, 4>(a, bytes(4), st) : lin_wide_launch<RM, NA, 3>(a, bytes(3), st);
+}
+
+static inline cudaError_t lin_wide_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
+    LinWideArgs a;
+    a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.xr = (rows + 7) & ~7;
+    const int units = (N + 1) / 2, most = 2 * ((units + LIN_SMS - 1) / LIN_SMS), np = (most + LW_ROWS - 1) / LW_ROWS;
+    a.per = 2 * ((most / 2 + np - 1) / np);
+    if (rows <= 16) return a.per <= 16 ? lin_wide_depth<1, 2>(a, np, st) : lin_wide_depth<1, 4>(a, np, st);
+    return a.per <= 16 ? lin_wide_depth<2, 2>(a, np, st) : lin_wide_depth<2, 4>(a, np, st);
+}
+
 static inline cudaError_t lin_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
     const LinPlan p = lin_plan(N, K);
+    // k_linear_wide unless few weight rows make k_linear cut k into four or eight slices (1 x 1185 x 11008: 9.6 us, 11.1 with
+    // whole rows a block, and twice the error) or a block would take more than three passes of 32 (17 x 32000 x 1408: 24.6, 26.5).
+    if (((uintptr_t)x & 15) == 0 && p.S <= 2 && N <= 3 * LW_ROWS * LIN_SMS) return lin_wide_run(x, w, y, rows, N, K, st);
     LinArgs a;
     a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.S = p.S; a.groups = p.groups; a.NW = p.NW;
     a.x_aligned = ((uintptr_t)x & 15) == 0;
