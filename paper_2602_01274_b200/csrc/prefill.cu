@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(THREADS_G, 1) k_pf_gemm(const __grid_constant_
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (smem_u32(smem) & 1023u) {                        // (the same in every block)
         if (threadIdx.x == 0) atomicCAS(a.abort_flag, 0, 13);
         return;
@@ -274,34 +274,32 @@ __global__ void __launch_bounds__(THREADS_G, 1) k_pf_gemm(const __grid_constant_
                 for (unsigned it = 0; it < MBAR_SPIN_LIMIT && !mbar_try_wait(full + j % STAGES, ((uint32_t)(j / STAGES)) & 1u); ++it) {}
         }
     } else if (warp == 9) {
-        if (lane == 0) {
-            int n = 0, i = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
-                const int m = t % a.mt, u0 = (t / a.mt) * a.w, wu = min(a.w, a.MT - u0), na = m == a.mt - 1 ? na_last : 16;
-                const uint32_t idesc = umma_idesc(wu * 16);
-                for (int kb = 0; kb < nkb && ok; ++kb, ++n) {
-                    if (kb % SEG == 0) {
-                        if (kb) { umma_commit(acc_full + (i & 1)); ++i; }
-                        ok = wait_bar(fb, acc_empty + (i & 1), (((uint32_t)(i >> 1)) & 1u) ^ 1u, 21, i);
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
-                    const uint32_t acc = tmem + (uint32_t)(i & 1) * 256u;
-                    const int slot = n % STAGES;
-                    ok = wait_bar(fb, full + slot, ((uint32_t)(n / STAGES)) & 1u, 22, n);
+        const uint32_t on = elect_lane();                // (all lanes wait, one issues)
+        int n = 0, i = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
+            const int m = t % a.mt, u0 = (t / a.mt) * a.w, wu = min(a.w, a.MT - u0), na = m == a.mt - 1 ? na_last : 16;
+            const uint32_t idesc = umma_idesc(wu * 16);
+            for (int kb = 0; kb < nkb && ok; ++kb, ++n) {
+                if (kb % SEG == 0) {
+                    if (kb) { umma_commit_if(on, acc_full + (i & 1)); ++i; }
+                    ok = __all_sync(0xffffffffu, wait_bar(fb, acc_empty + (i & 1), (((uint32_t)(i >> 1)) & 1u) ^ 1u, 21, i));
                     if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t a0 = smem_u32(smem + slot * (A_BYTES + B_BYTES)), b0 = a0 + A_BYTES, a1 = a0 + (uint32_t)na * 1024u;
-#pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
-                        umma(acc, umma_desc(a0 + k16 * 32), umma_desc(b0 + k16 * 32), idesc, (kb % SEG > 0 || k16 > 0) ? 1u : 0u);
-                        umma(acc, umma_desc(a1 + k16 * 32), umma_desc(b0 + k16 * 32), idesc, 1u);
-                    }
-                    umma_commit(empty + slot);
                 }
-                umma_commit(acc_full + (i & 1));
+                const uint32_t acc = tmem + (uint32_t)(i & 1) * 256u;
+                const int slot = n % STAGES;
+                ok = __all_sync(0xffffffffu, wait_bar(fb, full + slot, ((uint32_t)(n / STAGES)) & 1u, 22, n));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t a0 = smem_u32(smem + slot * (A_BYTES + B_BYTES)), b0 = a0 + A_BYTES, a1 = a0 + (uint32_t)na * 1024u;
+#pragma unroll
+                for (int k16 = 0; k16 < 4; ++k16) {
+                    umma_if(on, acc, umma_desc(a0 + k16 * 32), umma_desc(b0 + k16 * 32), idesc, (kb % SEG > 0 || k16 > 0) ? 1u : 0u);
+                    umma_if(on, acc, umma_desc(a1 + k16 * 32), umma_desc(b0 + k16 * 32), idesc, 1u);
+                }
+                umma_commit_if(on, empty + slot);
             }
+            umma_commit_if(on, acc_full + (i & 1));
         }
     } else {
         const int quad = warp & 3, half = warp >> 2;
