@@ -318,13 +318,17 @@ def pacer_linear(x: torch.Tensor, w: torch.Tensor) -> torch.Tensor:
     if nbytes == 0:
         raise PacerError("pacer_linear: unsupported shape")
     dev = x.device
-    scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=dev)
-    sp = (scratch.data_ptr() + 255) // 256 * 256
     y = torch.empty(rows, N, dtype=torch.float32, device=dev)
-    # (switching the current device costs more than the product of a small shape)
+    # (switching the current device costs more than the product of a small shape, and so does an allocation: the product reads no
+    # scratch, and where the entry point without it takes the shape it is the one called)
     with contextlib.nullcontext() if dev.index == torch.cuda.current_device() else torch.cuda.device(dev):
-        rc = _lib.pacer_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, N, K, sp, nbytes,
-                               torch.cuda.current_stream(dev).cuda_stream)
+        stream = torch.cuda.current_stream(dev).cuda_stream
+        if nbytes <= PACER_LINEAR_STATIC_BYTES:
+            rc = _lib.pacer_linear_static(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, N, K, stream)
+        else:
+            scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=dev)
+            rc = _lib.pacer_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), rows, N, K, (scratch.data_ptr() + 255) // 256 * 256,
+                                   nbytes, stream)
     if rc != 0:
         raise PacerError(f"pacer_linear: {_lib.pacer_strerror(rc).decode()}: {_lib.pacer_last_error(None).decode()}")
     return y
