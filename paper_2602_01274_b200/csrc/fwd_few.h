@@ -8,6 +8,7 @@ namespace fwd {
 
 constexpr int FEW_ROWS = 16;                    // live token rows of such a forward at most
 constexpr int FQ = 8;                           // query rows of an attention item
+constexpr int FEW_XBYTES = 5120;                // shared memory for a block's columns of the residual stream
 constexpr int FEW_ITEMS = 1024;                 // attention partials kept: items x FQ rows (or one per unsplit item)
 
 // Whether a forward of these dimensions can take the kernel (when its live rows turn out to be few): the residual columns

@@ -14,6 +14,7 @@ struct Args {
     Plan P;
     FwdBufs fb;
     int32_t kind, aux;
+    int32_t n_fwd;           // k_few, KIND_DRAFT: forwards of this launch, each on the token that the one before chose (else 1)
     int32_t few_max;         // k_forward: a forward of at most this many live rows was k_few's
 };
 

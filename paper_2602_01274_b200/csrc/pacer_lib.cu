@@ -502,7 +502,7 @@ static int prof_stop(pacer_ctx *c, bool on, double weight_bytes) {
 
 // Runs model `which` on the rows `kind` selects: one cooperative launch of k_few or k_forward, or one of each (see below); the
 // kernel that does the work also takes the stage's decisions in its tail.
-static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux, bool head) {
+static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux, bool head, int n_fwd = 1) {
     ModelDev &m = c->model[which];
     if (g.rtot > fwd::MAX_ROWS || g.batch > fwd::MAX_SEQ) return fail(c, PACER_EUNSUPPORTED, "too many rows or sequences in one forward");
     if (head && kind == KIND_VERIFY && g.rtot > c->ncta) return fail(c, PACER_EUNSUPPORTED, "more verify rows than blocks");
@@ -510,7 +510,7 @@ static int run_forward(pacer_ctx *c, int which, const Geom &g, int kind, int aux
     auto it = c->plans.find(key);
     if (it == c->plans.end()) it = c->plans.emplace(key, fwd::make_plan(m, c->d, c->fb, c->ncta, head, g)).first;
     fwd::Args a;
-    a.d = c->d; a.m = m; a.g = g; a.P = it->second; a.fb = c->fb; a.kind = kind; a.aux = aux;
+    a.d = c->d; a.m = m; a.g = g; a.P = it->second; a.fb = c->fb; a.kind = kind; a.aux = aux; a.n_fwd = n_fwd;
     a.fb.prof = (c->prof_on && c->ncta <= fwd::PROF_BLOCKS) ? c->prof_stamps : nullptr;
     bool prof;
     int rc;
@@ -757,8 +757,12 @@ static int enqueue_verify_accept(pacer_ctx *c) {
 static int enqueue_step(pacer_ctx *c, int gamma_max) {
     int rc;
     const int b = c->cfg.block_b;
+    if ((rc = need_ready(c, true))) return rc;
+    // A block's draft forwards as one launch where k_few runs them for certain (not while every launch is stamped for itself).
+    const bool one = !c->prof_on && c->g_draft.rtot <= fwd::FEW_ROWS && fwd::few_rows_ok(c->model[PACER_DRAFT], c->g_draft, KIND_DRAFT, c->ncta);
     for (int blk = 0; blk < gamma_max / b; ++blk) {
-        for (int i = 0; i < b; ++i)
+        if (one && (rc = run_forward(c, PACER_DRAFT, c->g_draft, KIND_DRAFT, 0, true, b))) return rc;
+        for (int i = 0; i < b && !one; ++i)
             if ((rc = pacer_draft_step(c))) return rc;
         if ((rc = pacer_preverify(c))) return rc;
     }
