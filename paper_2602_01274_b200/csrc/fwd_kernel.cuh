@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
         if (c.lane == 0) weight_producer(c, a.fb, a.P, c.warp == W_PRODUCER ? 0 : c.warp - 9);
         return;
     }
-    if (c.warp == MMA_ISSUER) {
-        if (c.lane == 0) mma_issuer<NT, TWO, BIG>(c, a.fb, a.P, g.G);
+    if (__shfl_sync(0xffffffffu, c.warp, 0) == MMA_ISSUER) {
+        mma_issuer<NT, TWO, BIG>(c, a.fb, a.P, g.G);
         __syncwarp();
         asm volatile("bar.sync 2, 288;" ::: "memory");        // the phase warps have read their last accumulator
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(TMEM_COLS) : "memory");

@@ -91,7 +91,7 @@ __device__ __forceinline__ void weight_producer(Ctx &c, const FwdBufs &fb, const
     }
 }
 
-// Lane 0 of warp MMA_ISSUER: the tensor-core instructions of every stage.  Per k block four MMAs of K = 16 per row
+// Warp MMA_ISSUER (all lanes wait, one issues, see umma_if): the tensor-core instructions of every stage.  Per k block four MMAs of K = 16 per row
 // group; the A operand is the group's part of the activation stage (128 rows are read from its base: values,
 // remainders, then whatever follows in shared memory, which only reaches accumulator lanes nobody reads), the B
 // operand the weight stage.  BIG: forwards with more than 32 rows (up to three row groups, each with its own
@@ -102,11 +102,12 @@ __device__ __forceinline__ void mma_issuer(Ctx &c, const FwdBufs &fb, const Plan
     const int XS = BIG ? P.xs : x_stages(NT), XKBN = BIG ? P.xkb : XK / KB;          // stages; k blocks per stage
     const int XKB_BYTES = BIG ? P.xkb_bytes : 2 * NT * 1024, XSTAGE_BYTES = XKBN * XKB_BYTES;
     const int GROUP_BYTES = 2 * NT * 1024;
+    const uint32_t on = elect_lane(), tmem = __shfl_sync(0xffffffffu, c.tmem, 0);
     int n = 0, head = 0, m = 0, np = 0;
     for (int q = 0; q < n_ops(P); ++q) {
         const GemmOp &op = P.op[op_index(P, q)];
         int t0, T, k_lo, k_hi;
-        op_range(op, c.cta, c.ncta, t0, T, k_lo, k_hi);
+        op_range(op, blockIdx.x, gridDim.x, t0, T, k_lo, k_hi);
         for (int p = 0; p < n_passes(T, P.max_tiles); ++p, ++np) {
             int p0, Tp;
             pass_range(T, p, P.max_tiles, p0, Tp);
@@ -114,32 +115,32 @@ __device__ __forceinline__ void mma_issuer(Ctx &c, const FwdBufs &fb, const Plan
             const int T0 = TWO ? min(Tp, MMA_TILES) : Tp, T1 = Tp - T0;      // tiles of the first / second accumulator
             const uint32_t idesc = umma_idesc(T0 * 16), idesc1 = umma_idesc(T1 ? T1 * 16 : 16);
             // the phase warps have copied the previous pass's accumulator out
-            if (!wait_bar(fb, c.acc_empty, (((uint32_t)np) & 1u) ^ 1u, 11, np)) return;
+            if (!__all_sync(0xffffffffu, wait_bar(fb, c.acc_empty, (((uint32_t)np) & 1u) ^ 1u, 11, np))) return;
             for (int k = k_lo; k < k_hi; k += KB, ++n) {
                 const int kx = ((k - k_lo) / KB) % XKBN, xslot = m % XS;
-                if (kx == 0 && !wait_bar(fb, c.xfull + xslot, ((uint32_t)(m / XS)) & 1u, 8, m)) return;
+                if (kx == 0 && !__all_sync(0xffffffffu, wait_bar(fb, c.xfull + xslot, ((uint32_t)(m / XS)) & 1u, 8, m))) return;
                 const int at = ring_place(head, bytes, c.ring_bytes);
-                if (!wait_bar(fb, c.wfull + n % NB, ((uint32_t)(n / NB)) & 1u, 9, n)) return;
+                if (!__all_sync(0xffffffffu, wait_bar(fb, c.wfull + n % NB, ((uint32_t)(n / NB)) & 1u, 9, n))) return;
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(c.scratch + xslot * XSTAGE_BYTES + kx * XKB_BYTES), b0 = smem_u32(c.ring + at);
                 const uint32_t acc = (k > k_lo) ? 1u : 0u;
                 for (int g = 0; g < G; ++g) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        umma(c.tmem + g * P.acc_stride, umma_desc(a0 + g * GROUP_BYTES + k16 * 32), umma_desc(b0 + k16 * 32), idesc,
+                        umma_if(on, tmem + g * P.acc_stride, umma_desc(a0 + g * GROUP_BYTES + k16 * 32), umma_desc(b0 + k16 * 32), idesc,
                              (acc || k16 > 0) ? 1u : 0u);
                 }
                 if (TWO && T1) {                         // (only in the kernel variant with two accumulators: the common
                                                          // variant's loop is the kernel's critical path and stays minimal)
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16)
-                        umma(c.tmem + ACC_COLS, umma_desc(a0 + k16 * 32), umma_desc(b0 + T0 * 2048 + k16 * 32), idesc1,
+                        umma_if(on, tmem + ACC_COLS, umma_desc(a0 + k16 * 32), umma_desc(b0 + T0 * 2048 + k16 * 32), idesc1,
                              (acc || k16 > 0) ? 1u : 0u);
                 }
-                umma_commit(c.wempty + n % NB);
-                if (kx == XKBN - 1 || k + KB >= k_hi) { umma_commit(c.xempty + xslot); ++m; }
+                umma_commit_if(on, c.wempty + n % NB);
+                if (kx == XKBN - 1 || k + KB >= k_hi) { umma_commit_if(on, c.xempty + xslot); ++m; }
             }
-            umma_commit(c.acc_full);
+            umma_commit_if(on, c.acc_full);
         }
     }
 }

@@ -132,24 +132,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// One lane of the warp (the same one each time).
-__device__ __forceinline__ uint32_t elect_lane() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p;
-}
-// An MMA and a commit of the lane with `on`, called by the whole warp: only the instruction itself is predicated, so that the
-// descriptors are computed in uniform registers.  In a branch for one lane an MMA took 95 cycles to issue; N = 128 computes for 64.
-__device__ __forceinline__ void umma_if(uint32_t on, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
-                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
-                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(on) : "memory");
-}
-__device__ __forceinline__ void umma_commit_if(uint32_t on, uint64_t *bar) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(on) : "memory");
-}
-
 // The row-wise step on 16 accumulator columns (weight rows n0 ..) of token row r.
 template <int EPI>
 __device__ __forceinline__ void tile_epilogue(const GArgs &a, int r, int seq, int pos, int n0, float inv, const float (&v)[16], const float4 (&xr)[4], float &ss) {
