@@ -41,12 +41,19 @@ constexpr int FEW_THREADS = FC_THREADS + 64;
 constexpr int FNB = 32;                         // weight stages in flight (barrier pairs; one lane each in the producer)
 constexpr int F_STAGE = 28 * 1024;              // bytes of weights a stage aims at: a stage costs the producer about 0.35 us
 constexpr int F_PASS = 24;                      // 8-row weight atoms of a pass at most (a k block of a pass is a stage at least)
-constexpr int FXS = 3, F_XROWS = 52;            // activation stages, and 256-byte (row, k block) pieces of one
-constexpr int F_SCRATCH = 47 * 1024;            // activation ring; the sums of a pass and attention use the same bytes
+constexpr int F_XROWS = 52;                     // 256-byte (row, k block) pieces of an activation stage
+// Activation stages, and the bytes they share with the sums of a pass and with attention; the weight ring has the rest.  Up to
+// eight rows three stages; the target's forwards of nine to sixteen five: a stage is then four or five k blocks, the k groups
+// work on 40 of them at a time, and with three stages they wait for each other's (13 rows, 8 layers of width 4096, 12 drafts in
+// front: step 1957 us, now 1931; with five rows the smaller weight ring costs more than it brings: 738 us, 750).
+constexpr int FXS = 3, FXS_MANY = 5;
+__host__ __device__ constexpr int few_scratch(bool many) { return (many ? 71 : 47) * 1024; }
 constexpr int F_MISC = 10 * 1024;
 constexpr int F_GUARD = 1024;                   // before the ring: the rows of an atom ahead of the first one are read, not used
-constexpr int F_RING = (227 * 1024 - F_SCRATCH - F_MISC - F_GUARD) / 1024 * 1024;
-static_assert(FNB == 32 && F_SCRATCH % 1024 == 0 && FXS * F_XROWS * 256 <= F_SCRATCH && F_RING >= 5 * F_PASS * 1024, "layout");
+constexpr int F_SHARED = (227 * 1024 - F_MISC - F_GUARD) / 1024 * 1024;      // weight ring and activations
+__host__ __device__ constexpr int few_ring(bool many) { return F_SHARED - few_scratch(many); }
+static_assert(FNB == 32 && FXS * F_XROWS * 256 <= few_scratch(false) && FXS_MANY * F_XROWS * 256 <= few_scratch(true) &&
+              few_ring(true) >= 5 * F_PASS * 1024, "layout");
 constexpr int F_XBYTES = FEW_XBYTES;                  // of F_MISC: this block's columns of the residual stream
 // Weight rows [r0, r1) of a block in a projection: units of two rows (gate/up: 16, a gate atom and its up atom), as even
 // as they come; kept in shared memory for the whole forward.
@@ -66,7 +73,7 @@ struct FewItem {
 struct FewCtx {
     unsigned char *scratch, *ring;
     uint64_t *wfull, *wempty;      // [FNB] a stage's weights are there / have been read
-    uint64_t *xfull, *xempty;      // [FXS] the same for the activations
+    uint64_t *xfull, *xempty;      // [FXS_MANY] the same for the activations
     volatile int32_t *ready;       // passes begun by the consumers: a later pass of a projection may overwrite the scratch
     int32_t *slot_at;              // [FNB] ring offset of a stage, written by the producer before the stage's barrier
     const FewOp *ops;              // [N_OPS] of this forward; the first forward's are followed by those of the later ones
@@ -151,7 +158,7 @@ __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int 
     // few atoms: ten k groups, so that a warp's chain of k blocks is as short as it can be (14 rows x 5504 columns: 18 k
     // blocks a warp with five groups, 9 with ten)
     o.kgs = o.span <= 3 ? FW : FW / 2;
-    const int atoms = min(nlive <= 8 ? (WIDE ? F_PASS : 16) : (WIDE ? 16 : 12), F_SCRATCH / (o.kgs * nlive * 32)) & ~1;
+    const int atoms = min(nlive <= 8 ? (WIDE ? F_PASS : 16) : (WIDE ? 16 : 12), few_scratch(WIDE && nlive > 8) / (o.kgs * nlive * 32)) & ~1;
     o.npass = (o.span + atoms - 1) / atoms;
     // stage: F_STAGE bytes of weights, but work for every k group.  Only the block's own rows count: a block's 10 to 14 rows
     // of a d_model-wide projection touch two or three atoms, and with whole atoms in the ring the ten stages of a 1.3B
@@ -179,8 +186,8 @@ __device__ __forceinline__ void few_drain(uint64_t *full, int n, int slots) {
 // Producer warps.  Weights: every stage of the block for the whole forward, in order, running ahead into the next
 // projections and, where a launch runs several forwards, into the next of these.  A stage is up to 32 k blocks of the pass's rows, one bulk copy per k block by as many lanes; it takes the
 // next free bytes of the ring once the stages whose bytes it needs have been read (lane n % 32 remembers where stage n
-// begins).  Activations: FXS slots, one bulk copy per stage, once the projection's inputs are complete.
-__device__ __forceinline__ void few_weight_producer(FewCtx &c, const FwdBufs &fb, const Plan &P, int n_fwd, uint64_t policy) {
+// begins).  Activations: NX slots, one bulk copy per stage, once the projection's inputs are complete.
+__device__ __forceinline__ void few_weight_producer(FewCtx &c, const FwdBufs &fb, const Plan &P, int n_fwd, int ring_bytes, uint64_t policy) {
     int n = 0, tail = 0, at = 0;                        // next stage; first stage not known to be read; next byte
     long long head = 0, tail_v = 0, mine = 0;           // virtual ring positions: next byte, first byte still in use, this lane's stage
     bool alive = true;
@@ -198,8 +205,8 @@ __device__ __forceinline__ void few_weight_producer(FewCtx &c, const FwdBufs &fb
             unsigned char *dst = c.ring + c.lane * kbytes;
             for (int k = 0; k < o.nkb; k += o.kbs, ++n) {
                 const int nk = min(o.kbs, o.nkb - k), bytes = nk * (int)kbytes;
-                if (at + bytes > F_RING) { head += F_RING - at; at = 0; }
-                while (tail < n && (tail <= n - FNB || head + bytes > tail_v + F_RING)) {
+                if (at + bytes > ring_bytes) { head += ring_bytes - at; at = 0; }
+                while (tail < n && (tail <= n - FNB || head + bytes > tail_v + ring_bytes)) {
                     if (!wait_bar(fb, c.wempty + (tail & (FNB - 1)), ((uint32_t)(tail / FNB)) & 1u, 5, tail)) { alive = false; break; }
                     ++tail;
                     tail_v = __shfl_sync(0xffffffffu, mine, tail & (FNB - 1));
@@ -221,6 +228,7 @@ __device__ __forceinline__ void few_weight_producer(FewCtx &c, const FwdBufs &fb
     few_drain(c.wfull, n, FNB);
 }
 
+template <int NX>
 __device__ __forceinline__ void few_x_producer(FewCtx &c, const Args &a, uint64_t policy) {
     const Plan &P = a.P;
     int n = 0, pass = 0;
@@ -251,8 +259,8 @@ __device__ __forceinline__ void few_x_producer(FewCtx &c, const Args &a, uint64_
             }
             asm volatile("fence.proxy.async;" ::: "memory");
             for (int k = 0; k < o.nkb; k += c.xk, ++n) {
-                const int slot = n % FXS;
-                if (!__all_sync(0xffffffffu, wait_bar(a.fb, c.xempty + slot, (((uint32_t)(n / FXS)) & 1u) ^ 1u, 7, n))) { few_drain(c.xfull, n, FXS); return; }
+                const int slot = n % NX;
+                if (!__all_sync(0xffffffffu, wait_bar(a.fb, c.xempty + slot, (((uint32_t)(n / NX)) & 1u) ^ 1u, 7, n))) { few_drain(c.xfull, n, NX); return; }
                 if (c.lane == 0) {
                     const uint32_t bytes = (uint32_t)(min(c.xk, o.nkb - k) * c.nlive) * 256u;
                     mbar_expect_tx(c.xfull + slot, bytes);
@@ -262,7 +270,7 @@ __device__ __forceinline__ void few_x_producer(FewCtx &c, const Args &a, uint64_
             }
         }
     }
-    few_drain(c.xfull, n, FXS);
+    few_drain(c.xfull, n, NX);
 }
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t saddr) {
@@ -449,7 +457,7 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t *b, int count) {
 // One warp's share of a pass (weight rows ra .. ra + rows): the weight stages kg, kg + kgs, ... and N atoms of them from atom my_a on (my_n of them
 // its own, the rest is computed and not stored), into the sum buffer.  N is a template parameter because a branch per atom
 // costs more than the atom's instructions.  (A lane of an operand row beyond the live ones reads live row 0.)
-template <int RT, int N>
+template <int RT, int N, int NX>
 __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &o, int kg, int pn, int ra, int rows, int my_a,
                                          int my_n) {
     constexpr int KU = RT * N > 10 ? 1 : 2;              // k blocks whose loads overlap, as far as the registers go
@@ -473,9 +481,9 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
     int xs = 0;                                          // this warp is in activation stage xs - 1 of the pass
     const unsigned char *xb = c.scratch;         // ... whose k block 0 would be here
     auto next_x = [&]() {                                // every warp passes through every activation stage
-        const int n = c.xstage + xs, slot = n % FXS;
-        if (xs > 0) { __syncwarp(); if (c.lane == 0) mbar_arrive(c.xempty + (n - 1) % FXS); }
-        if (xs < nxs && c.ok) c.ok = wait_bar(a.fb, c.xfull + slot, ((uint32_t)(n / FXS)) & 1u, 8, n);
+        const int n = c.xstage + xs, slot = n % NX;
+        if (xs > 0) { __syncwarp(); if (c.lane == 0) mbar_arrive(c.xempty + (n - 1) % NX); }
+        if (xs < nxs && c.ok) c.ok = wait_bar(a.fb, c.xfull + slot, ((uint32_t)(n / NX)) & 1u, 8, n);
         xb = c.scratch + slot * (F_XROWS * 256) - xs * xk * nlive * 256;
         ++xs;
     };
@@ -534,6 +542,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
 template <int MAXRT, bool WIDE>
 __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int layer) {
     const FewOp o = c.ops[opi];
+    constexpr int X2 = WIDE ? FXS_MANY : FXS;            // activation stages of nine and more rows
     const int kg = o.kgs == FW ? c.warp : c.warp >> 1, cg = c.warp & 1, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
     float *red = reinterpret_cast<float *>(c.scratch);
     // (its loads travel with the first activations; also in a block without rows: it may end a sequence's draft step)
@@ -545,23 +554,23 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
         const int h0 = (pn + 1) >> 1, my_a = o.kgs < FW && cg ? h0 : 0, my_n = o.kgs == FW ? pn : cg ? pn - h0 : h0;
         if (threadIdx.x == 0) { __threadfence_block(); *c.ready = ++c.pass; }    // (a later pass:) the activations may be copied
         if (MAXRT == 1 || nlive <= 8) {
-            if (my_n <= 1) few_main<1, 1>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 2) few_main<1, 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 3) few_main<1, 3>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 4) few_main<1, 4>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 6) few_main<1, 6>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (!WIDE || my_n <= 8) few_main<1, 8>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            if (my_n <= 1) few_main<1, 1, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 2) few_main<1, 2, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 3) few_main<1, 3, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 4) few_main<1, 4, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 6) few_main<1, 6, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (!WIDE || my_n <= 8) few_main<1, 8, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
             else if constexpr (WIDE) {
-                if (my_n <= 10) few_main<1, 10>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-                else few_main<1, F_PASS / 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+                if (my_n <= 10) few_main<1, 10, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+                else few_main<1, F_PASS / 2, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
             }
         } else if constexpr (MAXRT == 2) {
-            if (my_n <= 1) few_main<2, 1>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 2) few_main<2, 2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 3) few_main<2, 3>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (my_n <= 4) few_main<2, 4>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if (!WIDE || my_n <= 6) few_main<2, 6>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-            else if constexpr (WIDE) few_main<2, 8>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            if (my_n <= 1) few_main<2, 1, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 2) few_main<2, 2, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 3) few_main<2, 3, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (my_n <= 4) few_main<2, 4, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if (!WIDE || my_n <= 6) few_main<2, 6, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+            else if constexpr (WIDE) few_main<2, 8, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
         }
         c.stage += o.nst; c.xstage += nxs;
         fsync();
@@ -665,7 +674,7 @@ __device__ __forceinline__ void few_attention_item(FewCtx &c, const Args &a, con
     const size_t cbase = (((size_t)layer * d.max_batch + w.seq) * m.cfg.n_kv_heads + w.kh) * (size_t)d.max_ctx * HD;
     unsigned char *qs = c.scratch;                                    // [QR] rows: HD values, HD remainders
     float *red = reinterpret_cast<float *>(c.scratch + QR * QS);      // [FW][QR][PW]
-    static_assert(QR * QS + FW * QR * PW * 4 <= F_SCRATCH, "attention scratch");
+    static_assert(QR * QS + FW * QR * PW * 4 <= few_scratch(false), "attention scratch");
     static_assert(QR * (HD / 4) <= FC_THREADS, "four channels of a query row per thread");
     const int qi = threadIdx.x;
     float4 qx;
@@ -885,15 +894,13 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     FewCtx c;
     c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31; c.cta = blockIdx.x; c.ncta = gridDim.x;
     c.ring = smem + F_GUARD;
-    c.scratch = c.ring + F_RING;
-    static_assert(F_RING % 1024 == 0, "ring");
-    unsigned char *misc = c.scratch + F_SCRATCH;
+    unsigned char *misc = c.ring + F_SHARED;
     c.wfull = reinterpret_cast<uint64_t *>(misc);
     c.wempty = c.wfull + FNB;
     c.xfull = c.wempty + FNB;
-    c.xempty = c.xfull + FXS;
-    c.ready = reinterpret_cast<volatile int32_t *>(c.xempty + FXS);          // one word, and a pad
-    c.slot_at = reinterpret_cast<int32_t *>(c.xempty + FXS + 1);
+    c.xempty = c.xfull + FXS_MANY;
+    c.ready = reinterpret_cast<volatile int32_t *>(c.xempty + FXS_MANY);          // one word, and a pad
+    c.slot_at = reinterpret_cast<int32_t *>(c.xempty + FXS_MANY + 1);
     FewOp *ops = reinterpret_cast<FewOp *>(c.slot_at + FNB);                 // [2][N_OPS]
     c.ops = ops;
     c.row_dst = reinterpret_cast<float **>(ops + 2 * N_OPS);
@@ -914,7 +921,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     c.gamma0 = c.pick + FEW_ROWS;                                            // [FEW_ROWS]
     c.att = reinterpret_cast<FewAtt *>(c.gamma0 + FEW_ROWS);
     c.first = reinterpret_cast<FewItem *>(c.att + 1);
-    static_assert(8 * (2 * FNB + 2 * FXS + 1) + 4 * FNB + 2 * sizeof(FewOp) * N_OPS + 8 * FEW_ROWS + 4 * (3 * MAX_ROWS + 2 * MAX_SEQ + 5 * FEW_ROWS) +
+    static_assert(8 * (2 * FNB + 2 * FXS_MANY + 1) + 4 * FNB + 2 * sizeof(FewOp) * N_OPS + 8 * FEW_ROWS + 4 * (3 * MAX_ROWS + 2 * MAX_SEQ + 5 * FEW_ROWS) +
                   (12 + 16 + 8 + 4) * FEW_ROWS + 16 + sizeof(FewAtt) + sizeof(FewItem) <= F_MISC - F_XBYTES, "tables");
     static_assert(sizeof(FewOp) * N_OPS % 8 == 0, "alignment of the pointer table");
     c.xs = reinterpret_cast<float *>(misc + F_MISC - F_XBYTES);
@@ -936,7 +943,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     }
     if (threadIdx.x == FC_THREADS) {
         for (int i = 0; i < FNB; ++i) { mbar_init(c.wfull + i, 1); mbar_init(c.wempty + i, 2); }
-        for (int i = 0; i < FXS; ++i) { mbar_init(c.xfull + i, 1); mbar_init(c.xempty + i, FW); }
+        for (int i = 0; i < FXS_MANY; ++i) { mbar_init(c.xfull + i, 1); mbar_init(c.xempty + i, FW); }
         *c.ready = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -979,6 +986,8 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
         return;
     }
     c.xk = F_XROWS / c.nlive;
+    const bool many = MAXRT == 2 && WIDE && c.nlive > 8;          // (such a launch is one forward)
+    c.scratch = c.ring + few_ring(many);
     if (threadIdx.x < 2 * N_OPS) {
         const int o = threadIdx.x % N_OPS;
         ops[threadIdx.x] = few_op<WIDE>(a.P.op[o], o, c.cta, c.ncta, threadIdx.x < N_OPS ? c.nlive : c.nlater);
@@ -992,13 +1001,14 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     c.bar_target = *reinterpret_cast<unsigned long long *>(c.flag + 2);
 
     if (c.warp == FW) {
-        few_weight_producer(c, a.fb, a.P, a.n_fwd, policy_evict_first());
+        few_weight_producer(c, a.fb, a.P, a.n_fwd, few_ring(many), policy_evict_first());
         return;
     }
     if (c.warp == FW + 1) {
         uint64_t keep;
         asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
-        few_x_producer(c, a, keep);
+        if (many) few_x_producer<FXS_MANY>(c, a, keep);
+        else few_x_producer<FXS>(c, a, keep);
         return;
     }
     if (c.cta == 0 && threadIdx.x < MAX_ROWS) {
@@ -1141,7 +1151,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
 template <int MAXRT, int HD, bool WIDE>
 static cudaError_t launch_few_variant(const Args &a, int ncta, cudaStream_t st) {
     static bool attr_set[64] = {};           // the opt-in is per device
-    constexpr int smem = F_GUARD + F_RING + F_SCRATCH + F_MISC;
+    constexpr int smem = F_GUARD + F_SHARED + F_MISC;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
