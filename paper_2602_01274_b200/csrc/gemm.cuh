@@ -411,9 +411,10 @@ static inline cudaError_t lin_wide_run(const bf16 *x, const bf16 *w, float *y, i
 
 static inline cudaError_t lin_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
     const LinPlan p = lin_plan(N, K);
-    // k_linear_wide unless few weight rows make k_linear cut k into four or eight slices (1 x 1185 x 11008: 9.6 us, 11.1 with
-    // whole rows a block, and twice the error) or a block would take more than three passes of 32 (17 x 32000 x 1408: 24.6, 26.5).
-    if (((uintptr_t)x & 15) == 0 && p.S <= 2 && N <= 3 * LW_ROWS * LIN_SMS) return lin_wide_run(x, w, y, rows, N, K, st);
+    // k_linear_wide unless few weight rows make k_linear cut k (1 x 1185 x 11008, four slices: 9.6 us, 11.1 with whole rows a block,
+    // and twice the error; 16 x 1536 x 8960, two: 10.4, 10.6; but 3 x 2048 x 2048, two: 5.2, 4.8) or a block would take more than
+    // three passes of 32 (17 x 32000 x 1408: 24.6, 26.5).
+    if (((uintptr_t)x & 15) == 0 && (p.S == 1 || (p.S == 2 && N >= 2048)) && N <= 3 * LW_ROWS * LIN_SMS) return lin_wide_run(x, w, y, rows, N, K, st);
     LinArgs a;
     a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.S = p.S; a.groups = p.groups; a.NW = p.NW;
     a.x_aligned = ((uintptr_t)x & 15) == 0;
