@@ -1,5 +1,5 @@
 // Skinny weight-streaming product: Y[r][n] = sum_k X[r][k] * W[n][k], rows <= 32, bf16 in, fp32 sums, ONE launch.  Two
-// kernels: k_linear_wide where every SM has its share of whole weight rows, k_linear else (see lin_run).
+// kernels: k_linear_wide where every SM has its share of whole weight rows, k_linear else (the rule: lin_plan.h).
 //
 // k_linear.  Bound by reading W once from HBM.  Every lane reads its share of W with 128-bit loads straight into registers
 // (each weight is used exactly once, so staging it in shared memory would only add traffic), 8 to 32 loads in flight
@@ -15,6 +15,7 @@
 // global memory.
 #pragma once
 #include "common.cuh"
+#include "lin_plan.h"
 
 __device__ __forceinline__ uint4 ldg_stream(const void *p) {
     uint4 v;
@@ -40,7 +41,7 @@ struct LinArgs {
     int32_t x_aligned;       // x is 16-byte aligned (a view into a larger tensor need not be)
 };
 
-constexpr int LIN_THREADS = 256, LIN_SMS = 148;
+constexpr int LIN_THREADS = 256;
 
 // Weight loads in flight per lane: D chunks of TT tiles (about 100 KB per SM where registers allow); activations: LIN_XD
 // chunks.  (With the activations in registers, two chunks ahead, 17 x 4096 x 11008 took 30 us: every chunk waited for L2.)
@@ -198,8 +199,6 @@ struct LinWideArgs {
     int32_t xr;              // token rows of a stage (rows, up to a multiple of 8)
 };
 
-constexpr int LW_ROWS = 32;
-
 __device__ __forceinline__ void lin_ldsm4(uint32_t (&r)[4], uint32_t a) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
 }
@@ -307,39 +306,6 @@ __global__ void __launch_bounds__(LIN_THREADS, 1) k_linear_wide(const LinWideArg
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-struct LinPlan {
-    int S, groups, NW, TT;
-};
-
-// The split with the least weight bytes per block: S = 1 or 2 slices over all SMs (every pair of SMs can hold a
-// cluster of two); 4 or 8 only while few clusters are needed (an odd number of SMs per GPC strands some otherwise).  A
-// block keeps at least eight chunks of k, and the smaller S wins ties: 17 x 4096 x 11008 runs as 74 clusters of two,
-// 7 tiles each (full 98.9 %), where one slice would leave 4 tiles on some SMs against a mean of 3.46.  More than eight tiles a
-// block without slices: slices could even out 5 % at most, and the sums of twice the tiles through the cluster cost 1 to 7 us
-// (32 x 12210 x 512 16.2 us with two slices, 9.5 without; 32 x 11008 x 4096 33.3, 26.9).
-static inline LinPlan lin_plan(int N, int K) {
-    const int MT = (N + 7) / 8, nch = K / 32;
-    LinPlan best{};
-    double best_cost = 1e30;
-    const int cap[4] = {LIN_SMS, LIN_SMS / 2, 32, 16};
-    for (int i = 0; i < 4; ++i) {
-        const int S = 1 << i;
-        if (S > 1 && (nch / S < 8 || best.NW > 1)) break;           // (NW > 1: more than eight tiles a block without slices)
-        const int waves = (MT + cap[i] * 64 - 1) / (cap[i] * 64);   // at most 64 tiles per block
-        if (S > 1 && waves > 1) break;
-        const int groups = MT < cap[i] * waves ? MT : cap[i] * waves, tiles = (MT + groups - 1) / groups;
-        const double cost = (double)waves * tiles / S;
-        if (cost < best_cost * 0.97) {
-            best_cost = cost;
-            best.S = S; best.groups = groups;
-            best.NW = 1;
-            while ((tiles + best.NW - 1) / best.NW > 8) best.NW *= 2;
-            best.TT = (tiles + best.NW - 1) / best.NW;
-        }
-    }
-    return best;
-}
-
 template <int RM, int TT>
 static cudaError_t lin_launch(const LinArgs &a, cudaStream_t st) {
     constexpr size_t sums = (size_t)8 * RM * 16 * TT * 8 * sizeof(float), ring = (size_t)8 * LIN_XD * RM * 16 * 64;
@@ -403,18 +369,16 @@ static cudaError_t lin_wide_depth(const LinWideArgs &a, int np, cudaStream_t st)
 static inline cudaError_t lin_wide_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
     LinWideArgs a;
     a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.xr = (rows + 7) & ~7;
-    const int units = (N + 1) / 2, most = 2 * ((units + LIN_SMS - 1) / LIN_SMS), np = (most + LW_ROWS - 1) / LW_ROWS;
-    a.per = 2 * ((most / 2 + np - 1) / np);
+    const LinPasses q = lin_wide_passes(N);
+    const int np = q.np;
+    a.per = q.per;
     if (rows <= 16) return a.per <= 16 ? lin_wide_depth<1, 2>(a, np, st) : lin_wide_depth<1, 4>(a, np, st);
     return a.per <= 16 ? lin_wide_depth<2, 2>(a, np, st) : lin_wide_depth<2, 4>(a, np, st);
 }
 
 static inline cudaError_t lin_run(const bf16 *x, const bf16 *w, float *y, int rows, int N, int K, cudaStream_t st) {
     const LinPlan p = lin_plan(N, K);
-    // k_linear_wide unless few weight rows make k_linear cut k (1 x 1185 x 11008, four slices: 9.6 us, 11.1 with whole rows a block,
-    // and twice the error; 16 x 1536 x 8960, two: 10.4, 10.6; but 3 x 2048 x 2048, two: 5.2, 4.8) or a block would take more than
-    // three passes of 32 (17 x 32000 x 1408: 24.6, 26.5).
-    if (((uintptr_t)x & 15) == 0 && (p.S == 1 || (p.S == 2 && N >= 2048)) && N <= 3 * LW_ROWS * LIN_SMS) return lin_wide_run(x, w, y, rows, N, K, st);
+    if (((uintptr_t)x & 15) == 0 && lin_wide_takes(rows, N, K, p.S)) return lin_wide_run(x, w, y, rows, N, K, st);
     LinArgs a;
     a.x = x; a.w = w; a.y = y; a.rows = rows; a.N = N; a.K = K; a.S = p.S; a.groups = p.groups; a.NW = p.NW;
     a.x_aligned = ((uintptr_t)x & 15) == 0;
