@@ -43,11 +43,14 @@ constexpr int F_STAGE = 28 * 1024;              // bytes of weights a stage aims
 constexpr int F_PASS = 24;                      // 8-row weight atoms of a pass at most (a k block of a pass is a stage at least)
 constexpr int F_XROWS = 52;                     // 256-byte (row, k block) pieces of an activation stage
 // Activation stages, and the bytes they share with the sums of a pass and with attention; the weight ring has the rest.  Up to
-// eight rows three stages; the target's forwards of nine to sixteen five: a stage is then four or five k blocks, the k groups
-// work on 40 of them at a time, and with three stages they wait for each other's (13 rows, 8 layers of width 4096, 12 drafts in
-// front: step 1957 us, now 1931; with five rows the smaller weight ring costs more than it brings: 738 us, 750).
+// eight rows three stages; the target's forwards of more rows five (few_many): a stage is then four or five k blocks, the k groups
+// work on 40 of them at a time, and with three stages they wait for each other's (13 rows, 4 layers of width 4096: 490 us with
+// three, 471 with five; head dimension 64: width 2048 262, 251, width 256 129, 130).  The smaller weight ring costs more than that
+// with five rows (step of 8 layers of width 4096, 12 drafts in front: 738 us with three, 750 with five), and with nine and ten rows
+// of wider models (9 rows, 4 layers of width 7168 844 with three, 869 with five; 3 of width 8192 955, 978; 4 of width 4096 450, 449).
 constexpr int FXS = 3, FXS_MANY = 5;
 __host__ __device__ constexpr int few_scratch(bool many) { return (many ? 71 : 47) * 1024; }
+__device__ __forceinline__ bool few_many(int nlive, int d_model) { return nlive > (d_model > 4096 ? 10 : 8); }
 constexpr int F_MISC = 10 * 1024;
 constexpr int F_GUARD = 1024;                   // before the ring: the rows of an atom ahead of the first one are read, not used
 constexpr int F_SHARED = (227 * 1024 - F_MISC - F_GUARD) / 1024 * 1024;      // weight ring and activations
@@ -90,6 +93,7 @@ struct FewCtx {
     int stage, xstage;             // weight and activation stages of the passes done so far
     int pass;                      // passes begun (thread 0)
     int xk;                        // k blocks of an activation stage
+    bool many;                     // five activation stages, the same for the whole launch
     unsigned long long bar_target;
     // epilogues
     float **row_dst;               // [FEW_ROWS] where an LM-head row goes, or NULL
@@ -146,7 +150,7 @@ __device__ __forceinline__ void few_store(bf16 *base, int i, int k, int nlive, f
 }
 
 template <bool WIDE>
-__device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int ncta, int nlive) {
+__device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int ncta, int nlive, bool many) {
     const int unit = opi == OP_GU ? 16 : 2, units = (op.N + unit - 1) / unit, base = units / ncta, rem = units - base * ncta;
     FewOp o;
     o.r0 = (cta * base + min(cta, rem)) * unit;
@@ -158,7 +162,7 @@ __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int 
     // few atoms: ten k groups, so that a warp's chain of k blocks is as short as it can be (14 rows x 5504 columns: 18 k
     // blocks a warp with five groups, 9 with ten)
     o.kgs = o.span <= 3 ? FW : FW / 2;
-    const int atoms = min(nlive <= 8 ? (WIDE ? F_PASS : 16) : (WIDE ? 16 : 12), few_scratch(WIDE && nlive > 8) / (o.kgs * nlive * 32)) & ~1;
+    const int atoms = min(nlive <= 8 ? (WIDE ? F_PASS : 16) : (WIDE ? 16 : 12), few_scratch(many) / (o.kgs * nlive * 32)) & ~1;
     o.npass = (o.span + atoms - 1) / atoms;
     // stage: F_STAGE bytes of weights, but work for every k group.  Only the block's own rows count: a block's 10 to 14 rows
     // of a d_model-wide projection touch two or three atoms, and with whole atoms in the ring the ten stages of a 1.3B
@@ -456,7 +460,8 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t *b, int count) {
 
 // One warp's share of a pass (weight rows ra .. ra + rows): the weight stages kg, kg + kgs, ... and N atoms of them from atom my_a on (my_n of them
 // its own, the rest is computed and not stored), into the sum buffer.  N is a template parameter because a branch per atom
-// costs more than the atom's instructions.  (A lane of an operand row beyond the live ones reads live row 0.)
+// costs more than the atom's instructions.  NX: activation stages, 0 for three or five by c.many.  (A lane of an operand row beyond
+// the live ones reads live row 0.)
 template <int RT, int N, int NX>
 __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &o, int kg, int pn, int ra, int rows, int my_a,
                                          int my_n) {
@@ -480,10 +485,13 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
         for (int m = 0; m < RT; ++m) acc[i][m][0] = acc[i][m][1] = acc[i][m][2] = acc[i][m][3] = 0.f;
     int xs = 0;                                          // this warp is in activation stage xs - 1 of the pass
     const unsigned char *xb = c.scratch;         // ... whose k block 0 would be here
+    int slot_x = 0;                                      // (NX = 0) the stage this warp is in
     auto next_x = [&]() {                                // every warp passes through every activation stage
-        const int n = c.xstage + xs, slot = n % NX;
-        if (xs > 0) { __syncwarp(); if (c.lane == 0) mbar_arrive(c.xempty + (n - 1) % NX); }
-        if (xs < nxs && c.ok) c.ok = wait_bar(a.fb, c.xfull + slot, ((uint32_t)(n / NX)) & 1u, 8, n);
+        const int n = c.xstage + xs, turn = NX > 0 ? n / max(NX, 1) : c.many ? n / FXS_MANY : n / FXS;
+        const int slot = n - turn * (NX > 0 ? NX : c.many ? FXS_MANY : FXS), left = NX > 0 ? (n - 1) % max(NX, 1) : slot_x;
+        if (xs > 0) { __syncwarp(); if (c.lane == 0) mbar_arrive(c.xempty + left); }
+        if (NX == 0) slot_x = slot;
+        if (xs < nxs && c.ok) c.ok = wait_bar(a.fb, c.xfull + slot, (uint32_t)turn & 1u, 8, n);
         xb = c.scratch + slot * (F_XROWS * 256) - xs * xk * nlive * 256;
         ++xs;
     };
@@ -542,7 +550,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
 template <int MAXRT, bool WIDE>
 __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int layer) {
     const FewOp o = c.ops[opi];
-    constexpr int X2 = WIDE ? FXS_MANY : FXS;            // activation stages of nine and more rows
+    constexpr int X2 = WIDE ? 0 : FXS;                   // activation stages of nine and more rows
     const int kg = o.kgs == FW ? c.warp : c.warp >> 1, cg = c.warp & 1, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
     float *red = reinterpret_cast<float *>(c.scratch);
     // (its loads travel with the first activations; also in a block without rows: it may end a sequence's draft step)
@@ -986,11 +994,12 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
         return;
     }
     c.xk = F_XROWS / c.nlive;
-    const bool many = MAXRT == 2 && WIDE && c.nlive > 8;          // (such a launch is one forward)
-    c.scratch = c.ring + few_ring(many);
+    // (in a launch of several forwards the later ones have at most eight rows)
+    c.many = MAXRT == 2 && WIDE && a.n_fwd == 1 && few_many(c.nlive, m.cfg.d_model);
+    c.scratch = c.ring + few_ring(c.many);
     if (threadIdx.x < 2 * N_OPS) {
         const int o = threadIdx.x % N_OPS;
-        ops[threadIdx.x] = few_op<WIDE>(a.P.op[o], o, c.cta, c.ncta, threadIdx.x < N_OPS ? c.nlive : c.nlater);
+        ops[threadIdx.x] = few_op<WIDE>(a.P.op[o], o, c.cta, c.ncta, threadIdx.x < N_OPS ? c.nlive : c.nlater, c.many);
     }
     if (threadIdx.x == 32) {
         const unsigned long long v = ld_acquire_u64(a.fb.bar);
@@ -1001,13 +1010,13 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     c.bar_target = *reinterpret_cast<unsigned long long *>(c.flag + 2);
 
     if (c.warp == FW) {
-        few_weight_producer(c, a.fb, a.P, a.n_fwd, few_ring(many), policy_evict_first());
+        few_weight_producer(c, a.fb, a.P, a.n_fwd, few_ring(c.many), policy_evict_first());
         return;
     }
     if (c.warp == FW + 1) {
         uint64_t keep;
         asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
-        if (many) few_x_producer<FXS_MANY>(c, a, keep);
+        if (c.many) few_x_producer<FXS_MANY>(c, a, keep);
         else few_x_producer<FXS>(c, a, keep);
         return;
     }

@@ -23,12 +23,17 @@ SHAPES = {
     "passes": (synth.ModelShape(1, 768, 6, 2, 20480, 50000), synth.ModelShape(1, 256, 2, 2, 512, 50000)),
 }
 
+# reached by name: a target wider than 4096, whose nine and ten rows take three activation stages and eleven five
+WIDER = {
+    "stages": (synth.ModelShape(1, 4224, 33, 3, 320, 1001), synth.ModelShape(1, 64, 1, 1, 64, 1001)),
+}
+
 
 @pytest.mark.parametrize("shape", sorted(SHAPES))
 @pytest.mark.parametrize("window,n_prompt", [(4, 2), (7, 33), (8, 97), (15, 40), (16, 300)])
 def test_verify_rows(shape, window, n_prompt):
     from paper_2602_01274_b200 import binding as b
-    T, D = SHAPES[shape]
+    T, D = {**SHAPES, **WIDER}[shape]
     cfg = synth.PairConfig("few", T, D, agree=0.8, n_prompt=n_prompt, max_new=24, gamma_max=window, block_b=1 if window % 4 else 4)
     gpu = synth.make_pair(cfg, seed=3, device="cuda:0")
     cpu = {k: ({n: t.cpu() for n, t in v.items()} if isinstance(v, dict) else v.cpu()) for k, v in gpu.items()}
@@ -62,6 +67,11 @@ def test_verify_rows(shape, window, n_prompt):
     al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, window)[:gamma]
     assert np.abs(al - o.alpha()[:gamma]).max() < ALPHA_TOL
     ctx.close()
+
+
+@pytest.mark.parametrize("shape,window", [("stages", 8), ("stages", 9), ("stages", 10)])
+def test_verify_rows_of_wider_models(shape, window):
+    test_verify_rows(shape, window, 9)
 
 
 @pytest.mark.parametrize("batch", [1, 9, 16, 17])
