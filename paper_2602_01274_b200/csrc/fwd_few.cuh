@@ -29,6 +29,7 @@
 // as whole warps, the ring's bookkeeping in registers.
 #pragma once
 #include "fwd_few.h"
+#include "few_plan.h"
 
 #include "fwd_attention.cuh"
 #include "fwd_tails.cuh"
@@ -40,7 +41,6 @@ constexpr int FC_THREADS = 32 * FW;             // three warps per scheduler: 16
 constexpr int FEW_THREADS = FC_THREADS + 64;
 constexpr int FNB = 32;                         // weight stages in flight (barrier pairs; one lane each in the producer)
 constexpr int F_STAGE = 28 * 1024;              // bytes of weights a stage aims at: a stage costs the producer about 0.35 us
-constexpr int F_PASS = 24;                      // 8-row weight atoms of a pass at most (a k block of a pass is a stage at least)
 constexpr int F_XROWS = 52;                     // 256-byte (row, k block) pieces of an activation stage
 // Activation stages, and the bytes they share with the sums of a pass and with attention; the weight ring has the rest.  Up to
 // eight rows three stages; the target's forwards of more rows five (few_many): a stage is then four or five k blocks, the k groups
@@ -56,7 +56,7 @@ constexpr int F_GUARD = 1024;                   // before the ring: the rows of 
 constexpr int F_SHARED = (227 * 1024 - F_MISC - F_GUARD) / 1024 * 1024;      // weight ring and activations
 __host__ __device__ constexpr int few_ring(bool many) { return F_SHARED - few_scratch(many); }
 static_assert(FNB == 32 && FXS * F_XROWS * 256 <= few_scratch(false) && FXS_MANY * F_XROWS * 256 <= few_scratch(true) &&
-              few_ring(true) >= 5 * F_PASS * 1024, "layout");
+              few_ring(true) >= 5 * FEW_LONGER * 1024, "layout");
 constexpr int F_XBYTES = FEW_XBYTES;                  // of F_MISC: this block's columns of the residual stream
 // Weight rows [r0, r1) of a block in a projection: units of two rows (gate/up: 16, a gate atom and its up atom), as even
 // as they come; kept in shared memory for the whole forward.
@@ -149,7 +149,7 @@ __device__ __forceinline__ void few_store(bf16 *base, int i, int k, int nlive, f
     *reinterpret_cast<uint2 *>(base + few_frag(i, k, nlive)) = w;
 }
 
-template <bool WIDE>
+template <int PASS>
 __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int ncta, int nlive, bool many) {
     const int unit = opi == OP_GU ? 16 : 2, units = (op.N + unit - 1) / unit, base = units / ncta, rem = units - base * ncta;
     FewOp o;
@@ -158,11 +158,12 @@ __device__ __forceinline__ FewOp few_op(const GemmOp &op, int opi, int cta, int 
     o.atom0 = o.r0 >> 3;
     o.span = o.r1 > o.r0 ? ((o.r1 + 7) >> 3) - o.atom0 : 0;
     o.nkb = op.K / KB;
-    // a pass: what the accumulators (see launch_few) and the buffer of the sums hold, an even number of atoms
+    // a pass (a k block of it is a stage at least): what the accumulators (see few_plan.h) and the buffer of the sums hold, an
+    // even number of atoms
     // few atoms: ten k groups, so that a warp's chain of k blocks is as short as it can be (14 rows x 5504 columns: 18 k
     // blocks a warp with five groups, 9 with ten)
     o.kgs = o.span <= 3 ? FW : FW / 2;
-    const int atoms = min(nlive <= 8 ? (WIDE ? F_PASS : 16) : (WIDE ? 16 : 12), few_scratch(many) / (o.kgs * nlive * 32)) & ~1;
+    const int atoms = min(nlive <= 8 ? PASS : PASS > FEW_SHORT ? 16 : 12, few_scratch(many) / (o.kgs * nlive * 32)) & ~1;
     o.npass = (o.span + atoms - 1) / atoms;
     // stage: F_STAGE bytes of weights, but work for every k group.  Only the block's own rows count: a block's 10 to 14 rows
     // of a d_model-wide projection touch two or three atoms, and with whole atoms in the ring the ten stages of a 1.3B
@@ -547,9 +548,10 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
 
 // A projection of the forward.  Warp (kg, cg) takes its share of the k range and of the pass's atoms; the k groups' sums
 // go through shared memory; then warp w runs the epilogue for the live rows w, w + 10.
-template <int MAXRT, bool WIDE>
+template <int MAXRT, int PASS>
 __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int layer) {
     const FewOp o = c.ops[opi];
+    constexpr bool WIDE = PASS > FEW_SHORT;
     constexpr int X2 = WIDE ? 0 : FXS;                   // activation stages of nine and more rows
     const int kg = o.kgs == FW ? c.warp : c.warp >> 1, cg = c.warp & 1, nlive = c.nlive, nxs = (o.nkb + c.xk - 1) / c.xk;
     float *red = reinterpret_cast<float *>(c.scratch);
@@ -570,7 +572,7 @@ __device__ __forceinline__ void few_gemm(FewCtx &c, const Args &a, int opi, int 
             else if (!WIDE || my_n <= 8) few_main<1, 8, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
             else if constexpr (WIDE) {
                 if (my_n <= 10) few_main<1, 10, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
-                else few_main<1, F_PASS / 2, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
+                else few_main<1, PASS / 2, FXS>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
             }
         } else if constexpr (MAXRT == 2) {
             if (my_n <= 1) few_main<2, 1, X2>(c, a, o, kg, pn, ra, rb - ra, my_a, my_n);
@@ -892,7 +894,7 @@ __device__ __forceinline__ void few_tail_draft(const FewCtx &c, const Args &a, i
 
 // ------------------------------------------------------------------ the kernel
 
-template <int MAXRT, int HD, bool WIDE>
+template <int MAXRT, int HD, int PASS>
 __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ Args a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     if (smem_u32(smem) & 1023u) {               // the swizzled weight atoms need this alignment (the same in every block)
@@ -995,11 +997,11 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     }
     c.xk = F_XROWS / c.nlive;
     // (in a launch of several forwards the later ones have at most eight rows)
-    c.many = MAXRT == 2 && WIDE && a.n_fwd == 1 && few_many(c.nlive, m.cfg.d_model);
+    c.many = MAXRT == 2 && PASS > FEW_SHORT && a.n_fwd == 1 && few_many(c.nlive, m.cfg.d_model);
     c.scratch = c.ring + few_ring(c.many);
     if (threadIdx.x < 2 * N_OPS) {
         const int o = threadIdx.x % N_OPS;
-        ops[threadIdx.x] = few_op<WIDE>(a.P.op[o], o, c.cta, c.ncta, threadIdx.x < N_OPS ? c.nlive : c.nlater, c.many);
+        ops[threadIdx.x] = few_op<PASS>(a.P.op[o], o, c.cta, c.ncta, threadIdx.x < N_OPS ? c.nlive : c.nlater, c.many);
     }
     if (threadIdx.x == 32) {
         const unsigned long long v = ld_acquire_u64(a.fb.bar);
@@ -1083,7 +1085,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
             // that the projections need (68M draft step 90.7 -> 86.5 us, 7B forward of 5 rows 742 -> 727)
             asm volatile("" : "+r"(c.lane), "+r"(c.warp), "+r"(c.nlive), "+r"(c.cta), "+r"(c.ncta), "+r"(c.xk));
             if (opi == OP_QKV && c.warp == FW - 1 && c.cta < c.att->items) few_kv_prefetch(c, a, *c.first, l);
-            few_gemm<MAXRT, WIDE>(c, a, opi, l);
+            few_gemm<MAXRT, PASS>(c, a, opi, l);
             stamp();
             few_grid_barrier(c, a.fb);
             stamp();
@@ -1157,7 +1159,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     stamp();
 }
 
-template <int MAXRT, int HD, bool WIDE>
+template <int MAXRT, int HD, int PASS>
 static cudaError_t launch_few_variant(const Args &a, int ncta, cudaStream_t st) {
     static bool attr_set[64] = {};           // the opt-in is per device
     constexpr int smem = F_GUARD + F_SHARED + F_MISC;
@@ -1165,12 +1167,12 @@ static cudaError_t launch_few_variant(const Args &a, int ncta, cudaStream_t st) 
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(k_few<MAXRT, HD, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(k_few<MAXRT, HD, PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     void *params[] = {(void *)&a};
-    return cudaLaunchCooperativeKernel((const void *)k_few<MAXRT, HD, WIDE>, dim3(ncta), dim3(FEW_THREADS), params, smem, st);
+    return cudaLaunchCooperativeKernel((const void *)k_few<MAXRT, HD, PASS>, dim3(ncta), dim3(FEW_THREADS), params, smem, st);
 }
 
 }  // namespace fwd

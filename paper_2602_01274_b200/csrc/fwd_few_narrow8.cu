@@ -1,8 +1,8 @@
-// k_few for at most 8 live rows, short passes (see fwd_few.cuh), a translation unit of its own like every variant.
+// k_few for at most 8 live rows, short passes (see few_plan.h), a translation unit of its own like every variant.
 #include "fwd_few.cuh"
 
 namespace fwd {
 cudaError_t launch_few_narrow8(const Args &a, int ncta, cudaStream_t st) {
-    return a.m.hd == 64 ? launch_few_variant<1, 64, false>(a, ncta, st) : launch_few_variant<1, 128, false>(a, ncta, st);
+    return a.m.hd == 64 ? launch_few_variant<1, 64, FEW_SHORT>(a, ncta, st) : launch_few_variant<1, 128, FEW_SHORT>(a, ncta, st);
 }
 }  // namespace fwd

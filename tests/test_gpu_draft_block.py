@@ -13,12 +13,16 @@ SHAPES = {
     "tiny": synth.CONFIGS["tiny"],
     "gqa": synth.PairConfig("gqa", synth.ModelShape(2, 512, 4, 2, 1088, 2048), synth.ModelShape(2, 768, 6, 2, 1536, 2048), agree=0.8, n_prompt=40,
                             max_new=24, gamma_max=8),
+    # a draft whose gate/up projection takes the variant with long passes
+    "long": synth.PairConfig("long", synth.ModelShape(2, 128, 2, 1, 192, 2048), synth.ModelShape(1, 256, 4, 4, 10240, 2048), agree=0.8, n_prompt=40,
+                             max_new=24, gamma_max=8),
 }
 
 
 @pytest.mark.parametrize("shape,batch,window,block,sample", [
     ("tiny", 1, 8, 4, False), ("tiny", 3, 8, 4, False), ("tiny", 8, 8, 4, True), ("tiny", 2, 8, 2, False),
     ("gqa", 1, 8, 4, True), ("gqa", 4, 4, 4, False), ("gqa", 8, 8, 8, False),
+    ("long", 1, 8, 4, True), ("long", 6, 8, 4, False), ("long", 8, 8, 4, False),
 ])
 def test_one_launch_per_block(shape, batch, window, block, sample):
     from paper_2602_01274_b200 import binding as b

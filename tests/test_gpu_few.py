@@ -23,9 +23,13 @@ SHAPES = {
     "passes": (synth.ModelShape(1, 768, 6, 2, 20480, 50000), synth.ModelShape(1, 256, 2, 2, 512, 50000)),
 }
 
-# reached by name: a target wider than 4096, whose nine and ten rows take three activation stages and eleven five
+# reached by name: a target wider than 4096, whose nine and ten rows take three activation stages and eleven five; drafts whose
+# gate/up projection takes one pass of 18 or 26 atoms in the variant with long passes (28: two, also there)
 WIDER = {
     "stages": (synth.ModelShape(1, 4224, 33, 3, 320, 1001), synth.ModelShape(1, 64, 1, 1, 64, 1001)),
+    "long18": (SHAPES["narrow"][0], synth.ModelShape(1, 256, 4, 4, 10240, 1001)),
+    "long26": (SHAPES["narrow"][0], synth.ModelShape(1, 128, 2, 2, 15360, 1001)),
+    "long28": (SHAPES["narrow"][0], synth.ModelShape(1, 128, 1, 1, 16576, 1001)),
 }
 
 
@@ -69,7 +73,7 @@ def test_verify_rows(shape, window, n_prompt):
     ctx.close()
 
 
-@pytest.mark.parametrize("shape,window", [("stages", 8), ("stages", 9), ("stages", 10)])
+@pytest.mark.parametrize("shape,window", [("stages", 8), ("stages", 9), ("stages", 10), ("long18", 4), ("long26", 8), ("long28", 4)])
 def test_verify_rows_of_wider_models(shape, window):
     test_verify_rows(shape, window, 9)
 
