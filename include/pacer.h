@@ -195,8 +195,8 @@ int pacer_accept_rollback(pacer_ctx *ctx);
 /* Test hook for the error path: writes the device status word exactly as a kernel's
  * bounded wait that ran out would (code != 0, and the block, warp and detail it
  * records).  Until the next pacer_prefill / pacer_generate* resets the word, every
- * [sync] entry point returns PACER_EDEVICE with the decoded text, and forwards
- * launched meanwhile fall through their waits.  No kernel is launched.  [sync] */
+ * [sync] entry point returns PACER_EDEVICE with the decoded text, and decoding forwards
+ * launched meanwhile return at once.  No kernel is launched.  [sync] */
 int pacer_debug_set_device_status(pacer_ctx *ctx, int code, int block, int warp, int detail);
 
 /* [sync] Copies the per-sequence scalars of sequences 0..batch-1 to host memory.

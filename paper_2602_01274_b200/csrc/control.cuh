@@ -13,6 +13,10 @@ struct Top2 {
 // or block without columns, and the next forward would look that column up as a token.
 __device__ __forceinline__ Top2 top2_one(float v, int i) { return Top2{fmaxf(v, -INFINITY), i, -INFINITY}; }
 
+// A token from candidates that other blocks left in memory.  After a wait that gave up they can be anything, and the token is looked
+// up by the next forward, which may be in the same launch: an index outside the vocabulary (also that of no candidate) becomes 0.
+__device__ __forceinline__ int in_vocab(int i, int V) { return (unsigned)i < (unsigned)V ? i : 0; }
+
 __device__ __forceinline__ Top2 top2_merge(Top2 a, Top2 b) {
     // larger value wins; equal values keep the lower index
     Top2 r;

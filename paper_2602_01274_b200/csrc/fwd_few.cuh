@@ -502,7 +502,7 @@ __device__ __forceinline__ void few_main(FewCtx &c, const Args &a, const FewOp &
         // back from a warp whose weights must be read before its own can arrive
         while (st * o.kbs >= xs * xk) next_x();
         if (c.ok) c.ok = wait_bar(a.fb, c.wfull + slot, ((uint32_t)(n / FNB)) & 1u, 9, n);
-        uint32_t base = ring + (uint32_t)c.slot_at[slot];
+        uint32_t base = ring + (c.ok ? (uint32_t)c.slot_at[slot] : 0u);        // (a stage that never came has no place)
         for (int kb = st * o.kbs; kb < k_end;) {
             while (kb >= xs * xk) next_x();
             const int run = min(k_end, xs * xk);
@@ -951,6 +951,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
         }
         c.row_pos[r] = pos; c.row_tok[r] = tok;
     }
+    if (threadIdx.x == MAX_ROWS) c.flag[2] = *(volatile int32_t *)a.fb.abort_flag;
     if (threadIdx.x == FC_THREADS) {
         for (int i = 0; i < FNB; ++i) { mbar_init(c.wfull + i, 1); mbar_init(c.wempty + i, 2); }
         for (int i = 0; i < FXS_MANY; ++i) { mbar_init(c.xfull + i, 1); mbar_init(c.xempty + i, FW); }
@@ -970,7 +971,8 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
             if (r < g.rtot) c.idx_of[r] = i;
             n += __popc(mask);
         }
-        if (c.lane == 0) c.flag[1] = n;
+        // (after a wait that gave up nothing is computed: what the forward would read is not complete)
+        if (c.lane == 0) c.flag[1] = c.flag[2] != 0 ? -1 : n;
     } else if (c.warp == 1) {
         const int s = c.lane;
         int n = 0, ks = 0;
@@ -991,7 +993,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
     }
     __syncthreads();
     c.nlive = c.flag[1]; c.nlater = c.flag[0];
-    if (c.nlive == 0 || c.nlive > FEW_ROWS) {   // nothing to do, or k_forward's work: the same decision in every block
+    if (c.nlive <= 0 || c.nlive > FEW_ROWS) {   // nothing to do, or k_forward's work: the same decision in every block
         if (c.nlive == 0 && c.cta == 0 && threadIdx.x < g.batch) d.n_rows[threadIdx.x] = 0;
         return;
     }
@@ -1111,8 +1113,9 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
                 }
                 tp = few_warp_top2(tp);
                 if (c.lane == 0) {
-                    if (own) { d.row_arg[r] = tp.i1; d.row_margin[r] = tp.v1 - tp.v2; }
-                    if (kind != KIND_VERIFY && c.draw_pos[i] < 0) c.pick[s] = tp.i1;
+                    const int best = in_vocab(tp.i1, m.cfg.vocab);
+                    if (own) { d.row_arg[r] = best; d.row_margin[r] = tp.v1 - tp.v2; }
+                    if (kind != KIND_VERIFY && c.draw_pos[i] < 0) c.pick[s] = best;
                 }
                 if (c.draw_pos[i] >= 0) {           // (one row of the sequence at most)
                     BestD bd{-INFINITY, 0x7fffffff};
@@ -1121,7 +1124,7 @@ __global__ void __launch_bounds__(FEW_THREADS, 1) k_few(const __grid_constant__ 
                         bd = best_merge(bd, BestD{__ldcg(&p->v), __ldcg(&p->i)});
                     }
                     bd = few_warp_best(bd);
-                    if (c.lane == 0) c.pick[s] = drawn_token(bd);
+                    if (c.lane == 0) c.pick[s] = drawn_token(bd, m.cfg.vocab);
                 }
             }
             if (kind == KIND_DRAFT && c.cta < g.batch) few_tail_draft_rows(c, a, c.cta);

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
         }
         c.row_pos[r] = pos; c.row_tok[r] = tok;
     }
+    if (threadIdx.x == MAX_ROWS) c.flag[1] = *(volatile int32_t *)a.fb.abort_flag;
     __syncthreads();
     if (threadIdx.x < MAX_SEQ) {
         const int s = threadIdx.x;
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward(const __grid_constant__ 
         c.key_start[s] = ks;
     }
     __syncthreads();
+    if (c.flag[1]) return;                  // after a wait that gave up nothing is computed (see k_few)
     int live = 0;
     for (int s = 0; s < g.batch; ++s) live += c.n_rows[s];
     if (live <= a.few_max && a.few_max > 0) return;     // done by k_few already (the same decision in every block)

@@ -350,7 +350,7 @@ __device__ __forceinline__ void head_row_argmax(const Args &a, int r, Top2 *sm) 
         t = top2_merge(t, Top2{v.x, __float_as_int(v.y), v.z});
     }
     t = mma_block_top2(t, sm);
-    if (threadIdx.x == 0) { a.d.row_arg[r] = t.i1; a.d.row_margin[r] = t.v1 - t.v2; }
+    if (threadIdx.x == 0) { a.d.row_arg[r] = in_vocab(t.i1, a.m.cfg.vocab); a.d.row_margin[r] = t.v1 - t.v2; }
     bsync();
 }
 

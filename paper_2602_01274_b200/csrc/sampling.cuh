@@ -44,9 +44,8 @@ __device__ __forceinline__ BestD best_merge(BestD a, BestD b) {       // larger 
     return (a.v > b.v || (a.v == b.v && a.i <= b.i)) ? a : b;
 }
 
-// The token of a finished draw.  No column wins where every score is NaN or -inf: token 0 then, inside the vocabulary as every
-// later lookup needs it.
-__device__ __forceinline__ int drawn_token(BestD t) { return t.i == 0x7fffffff ? 0 : t.i; }
+// The token of a finished draw.  No column wins where every score is NaN or -inf: token 0 then.
+__device__ __forceinline__ int drawn_token(BestD t, int V) { return in_vocab(t.i, V); }
 
 // Block-wide arg-max of a per-thread candidate; every thread gets the result.
 // sm: at least blockDim.x / 32 entries.  All threads of the block must call it.
@@ -78,7 +77,7 @@ __device__ __forceinline__ int gumbel_argmax(const float *logits, int V, uint64_
         const double s = (double)__ldcg(logits + v) + gumbel_noise(seed, (uint32_t)v, (uint32_t)pos, (uint32_t)seq, (uint32_t)tag);
         if (s > t.v) { t.v = s; t.i = v; }
     }
-    return drawn_token(block_best(t, sm, named_barrier));
+    return drawn_token(block_best(t, sm, named_barrier), V);
 }
 
 // Block-wide sum of doubles (plain __syncthreads version, for the acceptance kernels).
@@ -205,7 +204,7 @@ static __global__ void __launch_bounds__(PICK_THREADS) k_accept_sample(DevPtrs d
             const double pv = (double)__ldcg(p + v);
             if (pv > a.v) { a.v = pv; a.i = v; }
         }
-        next = drawn_token(block_best(a, smb, false));
+        next = drawn_token(block_best(a, smb, false), V);
     }
     if (threadIdx.x == 0) {
         ab.arrived[s] = 0;

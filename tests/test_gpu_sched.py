@@ -121,3 +121,28 @@ def test_device_status_word_reaches_the_host_as_an_error(tiny2):
     assert ctx.pacer_read_state()[0]["finished"] == 1
     ref, _ = ctx.pacer_generate_ar(prompt, 8)
     np.testing.assert_array_equal(tok[0], ref[0])
+
+
+def test_forwards_after_a_wait_that_gave_up_return_at_once(tiny2):
+    """What such a forward would read is not complete, its tokens need not lie in the vocabulary: nothing is drafted, scored or
+    accepted until a new run, with few rows (one sequence) and with many (two windows of eight)."""
+    import ctypes
+    b, cfg, ctx = tiny2["b"], tiny2["cfg"], tiny2["ctx"]
+    for batch in (1, 2):
+        prompts = tiny2["prompts"][:batch]
+        ctx.pacer_prefill(prompts, 8, cfg.gamma_max, -1.0)
+        for _ in range(cfg.block_b):
+            ctx.pacer_draft_step()
+        ctx.pacer_preverify()
+        before = ctx.pacer_read_state(batch)
+        ctx.pacer_debug_set_device_status(9, 17, 9, 1234)
+        for _ in range(cfg.block_b):
+            ctx.pacer_draft_step()
+        ctx.pacer_preverify()
+        ctx.pacer_verify()
+        after = (b.SeqState * batch)()
+        assert b._lib.pacer_read_state(ctx._h, after, batch) != 0           # (the state is filled in all the same)
+        assert [a.as_dict() for a in after] == before
+        tok, *_ = ctx.pacer_generate(prompts, 8, cfg.gamma_max, -1.0)
+        ref, _ = ctx.pacer_generate_ar(prompts, 8)
+        np.testing.assert_array_equal(tok, ref)
