@@ -27,7 +27,7 @@ SHAPES = {
     ("hd64", 1, 2050), ("hd64", 5, 500), ("hd128_gqa", 1, 65), ("hd128_gqa", 1, 300), ("hd128_gqa", 4, 97),
     ("hd128_gqa", 1, 2305), ("long_k", 1, 140), ("long_k", 2, 50),
 ])
-def test_prefill_edges(shape, batch, n_prompt):
+def test_prefill_edges(shape, batch, n_prompt, sequences=None):
     from paper_2602_01274_b200 import binding as b
     T, D = SHAPES[shape]
     cfg = synth.PairConfig("pf", T, D, agree=0.8, n_prompt=n_prompt, max_new=8, gamma_max=4, batch=batch)
@@ -50,7 +50,7 @@ def test_prefill_edges(shape, batch, n_prompt):
     al = ctx.pacer_read_buffer(b.BUF_ALPHA, np.float32, batch * 4).reshape(batch, 4)
     pl = ctx.pacer_read_buffer(b.BUF_VERIFY_LOGITS, np.float32, batch * 5 * V).reshape(batch, 5, V)
     checked = 0
-    for s in range(batch if n_prompt < 400 else 1):
+    for s in sequences or range(batch if n_prompt < 400 else 1):
         o = orc.Pacer(To, Do, Bo, max_ctx, b=4, gamma_cap=4, t0=-1.0, rho=cfg.rho)
         o.prefill(prompts[s])
         o.draft_block(); o.preverify(); o.verify()

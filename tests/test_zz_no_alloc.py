@@ -11,6 +11,7 @@ import torch
 
 from oracle import pacer_oracle as orc
 from paper_2602_01274_b200 import synth
+from tests.test_gpu_linear import c_linear
 
 pytestmark = pytest.mark.gpu
 
@@ -21,7 +22,8 @@ def test_static_scratch_product_equals_the_ordinary_one_twice_in_a_row():
     for i, (rows, N, K) in enumerate([(17, 4096, 4096), (5, 2304, 768)]):
         w = synth.normal_bf16(7 + i, 21, (N, K), std=0.02, device=dev)
         x = synth.normal_bf16(8 + i, 22, (rows, K), std=1.0, device=dev)
-        ref = b.pacer_linear(x, w)
+        rc, ref = c_linear(b, x, w)                  # the C entry point with scratch of the caller
+        assert rc == 0
         out = torch.full((rows, N), float("nan"), dtype=torch.float32, device=dev)   # allocated by the caller
         b.pacer_linear_static(x, w, out)
         torch.cuda.synchronize()
