@@ -256,7 +256,9 @@ int pacer_generate_ar(pacer_ctx *ctx, const int32_t *prompt, int batch, int n_pr
  * and every block of every decoding forward (any model) stamps the device clock at its phase
  * boundaries (PACER_BUF_PHASE_NS keeps the last forward's).  pacer_profile_end [sync] returns the summed device time
  * of those forwards (ms), the bf16 weight bytes they streamed and their count.
- * Whole-loop timings are taken without it. */
+ * Meanwhile every forward is a launch of its own: the draft forwards of a block,
+ * which pacer_generate otherwise runs in one launch, are stamped one by one, and no
+ * step is replayed as a graph.  Whole-loop timings are taken without it. */
 int pacer_profile_begin(pacer_ctx *ctx);
 int pacer_profile_end(pacer_ctx *ctx, double *fwd_ms, double *fwd_weight_bytes, int64_t *fwd_launches);
 

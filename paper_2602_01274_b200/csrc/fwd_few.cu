@@ -14,8 +14,11 @@ cudaError_t launch_few_wider16(const Args &a, int ncta, cudaStream_t st);
 
 bool few_rows_ok(const ModelDev &m, const Geom &g, int kind, int ncta) {
     if (g.batch > FEW_ROWS || (kind != KIND_DRAFT && kind != KIND_VERIFY && kind != KIND_AR && kind != KIND_MB)) return false;
+    // this block's columns of the residual stream: in shared memory, and (the two residual projections) in one pass, the shortest
+    // being twelve atoms
+    static_assert(FEW_XBYTES / (FEW_ROWS * 4) + 16 <= 8 * 12, "a residual projection in one pass");
     const int xc = 2 * ((m.cfg.d_model / 2 + ncta - 1) / ncta);
-    return FEW_ROWS * xc * 4 <= FEW_XBYTES && xc + 16 <= 8 * 12;       // (a pass of twelve atoms: nine and more rows)
+    return FEW_ROWS * xc * 4 <= FEW_XBYTES;
 }
 
 // How long a pass: few_plan.h.  The target's forwards of windows that may have nine and more live rows take long passes whatever

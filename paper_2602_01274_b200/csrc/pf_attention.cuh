@@ -14,10 +14,15 @@
 //   warp 13            issues the MMAs: scores of tile i + 1 before the values of tile i, so the tensor cores run while
 //                      the softmax of tile i does.
 // One tile's planes of K, then of V, pass through a ring of NSLOT slots; scores and tile sums have two buffers each.
-// 56 heads (8 of keys), 2047 rows: 653 us on mma.sync with 64-row blocks, 310 with the MMAs issued from a one-lane branch and
-// the scores read twice, 253 with uniform descriptors, 196 as it is (0.9 PFLOP/s, the three passes counted): bound by the chain
-// softmax - values - next scores of a warpgroup, 4000 cycles a tile against the MMAs' 3072.  Error against fp64 5.8e-6
-// (mma.sync, 32 keys a tile: 6.0e-6).
+// 56 heads (8 of keys), 2047 rows, launches in a row: 653 us on mma.sync with 64-row blocks, 264 here (0.67 PFLOP/s, the three passes
+// counted); between the projections of a layer of width 7168, under the power cap, 780 and 330.  A block takes 10 us and 3.7 us a
+// tile (148 heads of 256 to 2048 rows, the same work on every SM, within 10 %).  The tile: the chain softmax - values - next scores of
+// a warpgroup; its MMAs are 1.6 us at 1965 MHz.  The 10 us overlap nothing, one block being all that an SM holds: barriers and tensor
+// memory, the conversion of the queries, the first keys, the last sums and the stores.  Up to some 200 rows they outweigh the rest
+// (128 rows, 56 heads: 12.8 us on mma.sync, 14.4 here; head dimension 64 8.5, 12.0).  The softmax warps hold 128 scores in 152
+// registers (104 bytes spilled at head dimension 128, 28 at 64).
+// Error against fp64: 0.96 to 1.006 of what mma.sync with 32 keys a tile had, 33 to 2047 rows, flat, ordinary and peaked softmax,
+// values with and without a mean (ordinary: 4.9e-6).
 constexpr int AQ = 128, AK = 128;          // query rows of a block, keys of a tile
 constexpr int A_SM_WARPS = 8, A_TMA = 12, A_MMA = 13, A_THREADS = 512;
 // Registers a thread of a softmax, the output and the last warpgroup: 128 at launch, 2 * 152 + 168 + 40 = 4 * 128.

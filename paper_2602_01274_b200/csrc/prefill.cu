@@ -10,8 +10,8 @@
 // rotary embedding + cache append, residual add + next operand, SwiGLU; 1/rms is applied to the output of the projection
 // that follows a norm, from shares of sum(x^2) left by the epilogue before.  A stage is 64 KB for 0.52 us of tensor time at 1965
 // MHz.  The widest projections are bound by the tensor cores at the clock that the power cap leaves them (2047 rows x 38400 x
-// 7168, two planes: 1.48 ms = 1.52 PFLOP/s, tensor pipe 90 % active at 1.45 GHz, L2 50 % busy); narrower ones keep the pipe 67
-// to 80 % active, with L2 no busier.
+// 7168, two planes: 1.47 ms = 1.54 PFLOP/s, tensor pipe 95 % active at 1.43 GHz, L2 50 % busy); narrower ones keep the pipe 70
+// to 84 % active, with L2 no busier.
 // The tensor cores truncate when they add to an accumulator, so a tile's products over 512 columns are taken out and added
 // in ordinary fp32 (registers of the epilogue warps) while the next 512 run into the other accumulator: with one
 // accumulator over all of K the logits behind a 300-token prompt were 1.7 times as far from an fp64 forward (1.4e-4 against
